@@ -4,14 +4,12 @@
 // free run of the augmented model and its closed loop with the PD law of
 // Eq. 28.
 //
-// One thread carries one trajectory.  The state (nx <= 8), the scheduling
-// network (two layers of four tanh neurons) and the 7 x 7 matrices of the
-// paper's model are far below a tensor-core tile, and every step depends on
-// the previous one, so the work is FP32 FMA chains with the parameters
-// broadcast from shared memory.  The gradient kernel accumulates each
-// thread's gradient in its own shared-memory column ([parameter][thread],
-// conflict-free) and sums the columns in a fixed order in FP64, so results
-// are deterministic.
+// The state (nx <= 8), the scheduling network (two layers of four tanh
+// neurons) and the 7 x 7 matrices of the paper's model are far below a
+// tensor-core tile, and every step depends on the previous one, so the work
+// is FP32 FMA chains.  The fit splits each trajectory's recurrences over a
+// few lanes and does everything that is not serial in k over all samples at
+// once; sums are taken in a fixed order, so results are deterministic.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -30,7 +28,6 @@ int set_last_error(int code, const char* msg);
 namespace slpvk {
 
 constexpr int NU = 3, NY = 3, NH = 4;
-constexpr int kThreads = 64;  // trajectories per block of the gradient kernel
 
 // Offsets of the blocks of theta (see include/slpv.h).
 template <int NX>
@@ -103,176 +100,493 @@ __device__ __forceinline__ void mz(const float* th, float p, const float* z, flo
 }
 
 // ---------------------------------------------------------------------------
-// Loss and gradient: per block, partial sums part[block][0..N) (gradient of
-// the data term, already divided by the sample count) and part[block][N]
-// (sum of squared normalised errors).
+// Loss and gradient in four passes.
+//
+// Only two recurrences are serial in k: the state x_{k+1} and the adjoint
+// lambda_k.  The adjoint's step is linear, lambda_k = J_k^T lambda_{k+1} +
+// c_k, with J_k and c_k functions of x_k alone, and so are every sample's
+// residual and its contribution to the gradient once lambda is known:
+//   state_kernel    x_k for all k (serial; NX lanes or more per trajectory)
+//   sample_kernel   squared errors, J_k and c_k (one thread per sample)
+//   adjoint_kernel  lambda_k (serial; one lane per state)
+//   outer_kernel    the gradient's outer products over all samples
+//   final_kernel    sums of the block partials, the l2 term, the mask
+// One thread per trajectory running both recurrences with everything on the
+// chain took 2,600 cycles per sample: 2.73 ms for 24 trajectories of 2,200
+// samples (n_x = 4), now 0.46 ms (state 339 us, adjoint 87, outer 12, sample
+// 10, final 7).  The state chain's latencies add up to 293 cycles of its 318
+// a sample: 7 FMAs, tanhf (62), a shuffle (26), 4 FMAs, tanhf, a shuffle, 4
+// FMAs, 8 FMAs and a shuffle.
 // ---------------------------------------------------------------------------
+
+// Lanes that share a trajectory in the serial passes: one per state and at
+// least one per neuron.
 template <int NX>
-__global__ void __launch_bounds__(kThreads) grad_kernel(const float* __restrict__ theta, const float* __restrict__ u,
-                                                        const float* __restrict__ y, const float* __restrict__ scales,
-                                                        int n_traj, int T, float inv_n, int want_grad,
-                                                        float* __restrict__ xh, double* __restrict__ part)
+constexpr int kLanes = NX <= 4 ? 4 : 8;
+
+template <int N>
+__device__ __forceinline__ void load_vec(const float* __restrict__ p, float* v)  // N even, p 8-byte aligned (16 for N % 4 == 0)
+{
+    if constexpr (N % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(p + i);
+            v[i] = q.x, v[i + 1] = q.y, v[i + 2] = q.z, v[i + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 2) {
+            const float2 q = *reinterpret_cast<const float2*>(p + i);
+            v[i] = q.x, v[i + 1] = q.y;
+        }
+    }
+}
+
+// Asynchronous copies into shared memory, a queue of whole chunks: the serial
+// passes read their inputs there, so that no step waits on a global load (a
+// register ring of loads was measured first: a wait on one load also waited
+// for later ones, 200 of 527 cycles a step).
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait()  // until at most the N youngest chunks are in flight
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+    __syncwarp();
+}
+constexpr int kStages = 4;   // chunks in shared memory: one in use, three in flight
+constexpr int kChunk = 32;   // steps per chunk of the state pass
+
+template <int N>
+__device__ __forceinline__ void store_vec(float* p, const float* v)
+{
+    if constexpr (N % 4 == 0) {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) *reinterpret_cast<float4*>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 2) *reinterpret_cast<float2*>(p + i) = make_float2(v[i], v[i + 1]);
+    }
+}
+
+// States x_k, k in [k0, k0 + len), of every trajectory into xh[traj][ld][NX]
+// (row k - k0), from carry[traj][NX] (k0 = 0: from rest); the state after the
+// window goes to carry.  Lane l of a trajectory's group computes neuron l % 4
+// of each layer and row l % NX of M(p) z, each by the same chain of FMAs as
+// the sample pass, so both see the same bits; shuffles hand the neurons and
+// the new state around.  Bound by that chain: two layers (an FMA chain, a
+// tanhf and a shuffle each), eta's output, the row's FMAs and a shuffle.
+// One warp per block: the few trajectories of a fit spread over the SMs.
+template <int NX>
+__global__ void __launch_bounds__(32) state_kernel(const float* __restrict__ theta, const float* __restrict__ u,
+                                                   const float* __restrict__ scales, int n_traj, int T, int k0, int len,
+                                                   int ld, float* __restrict__ carry, float* __restrict__ xh)
 {
     using Q = Lay<NX>;
-    extern __shared__ float4 shm4[];
-    float* th = reinterpret_cast<float*>(shm4);
-    float* acc = th + ((Q::N + 3) & ~3);                            // [N][kThreads]
-    double* lbuf = reinterpret_cast<double*>(acc + Q::N * kThreads);  // [kThreads]
-    const int tid = threadIdx.x;
-    for (int i = tid; i < Q::N; i += kThreads) th[i] = theta[i];
-    if (want_grad)
-        for (int i = tid; i < Q::N * kThreads; i += kThreads) acc[i] = 0.f;
+    constexpr int L = kLanes<NX>, PER = 32 / L;
+    const int l = (int)threadIdx.x % L, nr = l % NH, row = l % NX;
+    const int tr = blockIdx.x * PER + (int)threadIdx.x / L;
+    const bool own = tr < n_traj && l < NX;
+    const size_t t = tr < n_traj ? tr : n_traj - 1;
+    float w1[Q::NZ], w2[NH], w3[NH], m0[Q::NZ], m1[Q::NZ], x[NX];
+#pragma unroll
+    for (int j = 0; j < Q::NZ; ++j) {
+        w1[j] = theta[Q::W1 + nr * Q::NZ + j];
+        m0[j] = theta[Q::M0 + row * Q::NZ + j];
+        m1[j] = theta[Q::M1 + row * Q::NZ + j];
+    }
+#pragma unroll
+    for (int j = 0; j < NH; ++j) {
+        w2[j] = theta[Q::W2 + nr * NH + j];
+        w3[j] = theta[Q::W3 + j];
+    }
+    const float b1 = theta[Q::B1 + nr], b2 = theta[Q::B2 + nr], b3 = theta[Q::B3];
+    float isu[NU];
+#pragma unroll
+    for (int c = 0; c < NU; ++c) isu[c] = 1.0f / scales[c];
+#pragma unroll
+    for (int i = 0; i < NX; ++i) x[i] = k0 ? carry[t * NX + i] : 0.f;
+    float* xo = xh + t * ld * NX + row;
+    __shared__ float su[kStages][PER][kChunk * NU + 1];
+    const int n_chunk = (len + kChunk - 1) / kChunk, grp = (int)threadIdx.x / L;
+    const float* ul = u + (t * T + k0) * NU + l;
+    auto fetch = [&](int c) {  // the lanes of a group copy their trajectory's inputs
+        float* dst = &su[c % kStages][grp][l];
+        const float* src = ul + (size_t)c * (kChunk * NU);
+        const int n = (len - c * kChunk) * NU - l;
+        if (n > kChunk * NU - L) {
+#pragma unroll
+            for (int i = 0; i < kChunk * NU; i += L) copy_async<4>(dst + i, src + i);
+        } else {
+            for (int i = 0; i < n; i += L) copy_async<4>(dst + i, src + i);
+        }
+        copy_commit();
+    };
+#pragma unroll
+    for (int c = 0; c < kStages - 1; ++c) fetch(c);
+    float mine = x[0];
+#pragma unroll
+    for (int i = 1; i < NX; ++i) mine = row == i ? x[i] : mine;
+    auto step = [&](int k, const float* us) {
+        if (own) xo[(size_t)k * NX] = mine;
+        float z[Q::NZ], h1[NH], h2[NH];
+#pragma unroll
+        for (int i = 0; i < NX; ++i) z[i] = x[i];
+#pragma unroll
+        for (int c = 0; c < NU; ++c) z[NX + c] = us[c] * isu[c];
+        float a = b1;
+#pragma unroll
+        for (int j = 0; j < Q::NZ; ++j) a = fmaf(w1[j], z[j], a);
+        float h = tanhf(a);
+#pragma unroll
+        for (int j = 0; j < NH; ++j) h1[j] = __shfl_sync(0xffffffffu, h, j, L);
+        a = b2;
+#pragma unroll
+        for (int j = 0; j < NH; ++j) a = fmaf(w2[j], h1[j], a);
+        h = tanhf(a);
+#pragma unroll
+        for (int j = 0; j < NH; ++j) h2[j] = __shfl_sync(0xffffffffu, h, j, L);
+        float p = b3;
+#pragma unroll
+        for (int j = 0; j < NH; ++j) p = fmaf(w3[j], h2[j], p);
+        a = 0.f;
+#pragma unroll
+        for (int j = 0; j < Q::NZ; ++j) a = fmaf(fmaf(p, m1[j], m0[j]), z[j], a);
+        mine = a;
+#pragma unroll
+        for (int i = 0; i < NX; ++i) x[i] = __shfl_sync(0xffffffffu, a, i, L);
+    };
+    for (int c = 0; c < n_chunk; ++c) {
+        copy_wait<kStages - 2>();
+        fetch(c + kStages - 1);  // its buffer was read in the chunk before: that reading is behind the wait's barrier
+        const float* us = su[c % kStages][grp];
+        const int n = min(kChunk, len - c * kChunk);
+        if (n == kChunk) {
+#pragma unroll 4
+            for (int s = 0; s < kChunk; ++s) step(c * kChunk + s, us + s * NU);
+        } else {
+            for (int s = 0; s < n; ++s) step(c * kChunk + s, us + s * NU);
+        }
+    }
+    if (own) carry[t * NX + row] = mine;
+}
+
+// z_k = [x_k; u_k / s_u], the scheduling and the outputs of one sample.
+template <int NX>
+struct Sample {
+    float z[Lay<NX>::NZ], h1[NH], h2[NH], p, res[NY];  // res: y_hat - y / s_y
+};
+
+template <int NX>
+__device__ __forceinline__ void eval_sample(const float* th, const float* __restrict__ scales, const float* x,
+                                            const float* __restrict__ u, const float* __restrict__ y, Sample<NX>& S)
+{
+    using Q = Lay<NX>;
+    load_vec<NX>(x, S.z);
+#pragma unroll
+    for (int c = 0; c < NU; ++c) S.z[NX + c] = u[c] * (1.0f / scales[c]);
+    S.p = eta<NX>(th, S.z, S.h1, S.h2);
+#pragma unroll
+    for (int c = 0; c < NY; ++c) {
+        float a = 0.f;
+#pragma unroll
+        for (int j = 0; j < Q::NZ; ++j)
+            a = fmaf(fmaf(S.p, th[Q::M1 + (NX + c) * Q::NZ + j], th[Q::M0 + (NX + c) * Q::NZ + j]), S.z[j], a);
+        S.res[c] = a - y[c] * (1.0f / scales[3 + c]);
+    }
+}
+
+// e[i] = d eta / d (pre-activation of neuron i of the first layer).
+template <int NX>
+__device__ __forceinline__ void eta_back(const float* th, const float* h1, const float* h2, float* d2, float* e)
+{
+    using Q = Lay<NX>;
+#pragma unroll
+    for (int i = 0; i < NH; ++i) d2[i] = th[Q::W3 + i] * (1.0f - h2[i] * h2[i]);
+#pragma unroll
+    for (int i = 0; i < NH; ++i) {
+        float b = 0.f;
+#pragma unroll
+        for (int j = 0; j < NH; ++j) b = fmaf(th[Q::W2 + j * NH + i], d2[j], b);
+        e[i] = b * (1.0f - h1[i] * h1[i]);
+    }
+}
+
+// One thread per sample of the window (k fastest): the squared error, summed
+// per block in FP64 into loss_part[block], and, when the gradient is wanted,
+// the adjoint's step as a record adj[traj][k] of kRec floats: dx_{k+1,r} /
+// dx_{k,j} at j NX + r, then the output residuals' part of each lambda_{k,j}.
+// With M(p) and p = eta(z), do_r / dz_j = M(p)_rj + (M_1 z)_r E_j, E = W1^T e.
+constexpr int kSampleThreads = 64;
+template <int NX>
+constexpr int kRec = (NX * NX + NX + 3) / 4 * 4;  // whole 16-byte vectors
+
+template <int NX>
+__global__ void __launch_bounds__(kSampleThreads)
+    sample_kernel(const float* __restrict__ theta, const float* __restrict__ u, const float* __restrict__ y,
+                  const float* __restrict__ scales, int n_traj, int T, int k0, int len, int ld, int xld, int xk0,
+                  float inv_n, int want_grad, const float* __restrict__ xh, float* __restrict__ adj,
+                  double* __restrict__ loss_part)
+{
+    using Q = Lay<NX>;
+    __shared__ float th[Q::N];
+    __shared__ double red[kSampleThreads / 32];
+    for (int i = threadIdx.x; i < Q::N; i += kSampleThreads) th[i] = theta[i];
     __syncthreads();
-    const int tr = blockIdx.x * kThreads + tid;
+    const long long n = (long long)n_traj * len;
     double lsum = 0.0;
-    if (tr < n_traj) {
-        float isu[NU], isy[NY];
+    for (long long s = blockIdx.x * (long long)kSampleThreads + threadIdx.x; s < n;
+         s += (long long)gridDim.x * kSampleThreads) {
+        const size_t t = (size_t)(s / len);
+        const int k = (int)(s % len);
+        Sample<NX> S;
+        const size_t row = (t * T + k0 + k) * 3;
+        eval_sample<NX>(th, scales, xh + (t * xld + (k0 - xk0) + k) * NX, u + row, y + row, S);
+        float e2 = 0.f;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            isu[c] = 1.0f / scales[c];
-            isy[c] = 1.0f / scales[3 + c];
+        for (int c = 0; c < NY; ++c) e2 = fmaf(S.res[c], S.res[c], e2);
+        lsum += (double)e2;
+        if (!want_grad) continue;
+        float d2[NH], e[NH], m1z[Q::NO], ar[NY];
+        eta_back<NX>(th, S.h1, S.h2, d2, e);
+#pragma unroll
+        for (int r = 0; r < Q::NO; ++r) {
+            m1z[r] = 0.f;
+#pragma unroll
+            for (int j = 0; j < Q::NZ; ++j) m1z[r] = fmaf(th[Q::M1 + r * Q::NZ + j], S.z[j], m1z[r]);
         }
-        const float* ut = u + (size_t)tr * T * NU;
-        const float* yt = y + (size_t)tr * T * NY;
-        float x[NX];
+        float sr = 0.f;  // the residuals' part of dJ/dp
 #pragma unroll
-        for (int i = 0; i < NX; ++i) x[i] = 0.f;
-        for (int k = 0; k < T; ++k) {
-            if (want_grad) {
-#pragma unroll
-                for (int i = 0; i < NX; ++i) xh[((size_t)k * n_traj + tr) * NX + i] = x[i];
-            }
-            float z[Q::NZ], h1[NH], h2[NH], o[Q::NO];
-#pragma unroll
-            for (int i = 0; i < NX; ++i) z[i] = x[i];
-#pragma unroll
-            for (int c = 0; c < NU; ++c) z[NX + c] = ut[NU * k + c] * isu[c];
-            const float p = eta<NX>(th, z, h1, h2);
-            mz<NX>(th, p, z, o);
-            float e2 = 0.f;
-#pragma unroll
-            for (int c = 0; c < NY; ++c) {
-                const float r = o[NX + c] - yt[NY * k + c] * isy[c];
-                e2 = fmaf(r, r, e2);
-            }
-            lsum += (double)e2;
-#pragma unroll
-            for (int i = 0; i < NX; ++i) x[i] = o[i];
+        for (int c = 0; c < NY; ++c) {
+            ar[c] = 2.0f * S.res[c] * inv_n;
+            sr = fmaf(ar[c], m1z[NX + c], sr);
         }
-        if (want_grad) {
-            float lam[NX];  // dJ / dx_{k+1}
+        float* o = adj + (t * ld + k) * kRec<NX>;
+        float cv[NX];
 #pragma unroll
-            for (int i = 0; i < NX; ++i) lam[i] = 0.f;
-            float* my = acc + tid;
-            for (int k = T - 1; k >= 0; --k) {
-                float z[Q::NZ], h1[NH], h2[NH], o[Q::NO], a[Q::NO];
+        for (int j = 0; j < NX; ++j) {
+            float E = 0.f, J[NX];
 #pragma unroll
-                for (int i = 0; i < NX; ++i) z[i] = xh[((size_t)k * n_traj + tr) * NX + i];
+            for (int i = 0; i < NH; ++i) E = fmaf(th[Q::W1 + i * Q::NZ + j], e[i], E);
+            auto M = [&](int r) { return fmaf(S.p, th[Q::M1 + r * Q::NZ + j], th[Q::M0 + r * Q::NZ + j]); };
 #pragma unroll
-                for (int c = 0; c < NU; ++c) z[NX + c] = ut[NU * k + c] * isu[c];
-                const float p = eta<NX>(th, z, h1, h2);
-                mz<NX>(th, p, z, o);
+            for (int r = 0; r < NX; ++r) J[r] = fmaf(m1z[r], E, M(r));
+            store_vec<NX>(o + j * NX, J);
+            float v = sr * E;
 #pragma unroll
-                for (int i = 0; i < NX; ++i) a[i] = lam[i];
+            for (int c = 0; c < NY; ++c) v = fmaf(M(NX + c), ar[c], v);
+            cv[j] = v;
+        }
+        store_vec<NX>(o + NX * NX, cv);
+    }
 #pragma unroll
-                for (int c = 0; c < NY; ++c) a[NX + c] = 2.0f * (o[NX + c] - yt[NY * k + c] * isy[c]) * inv_n;
-                // M_0 and M_1 (outer product a z^T, scaled by p for M_1); s = dJ/dp
-                float s = 0.f;
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lsum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double v = red[0];
+        for (int w = 1; w < kSampleThreads / 32; ++w) v += red[w];
+        loss_part[blockIdx.x] = v;
+    }
+}
+
+// lambda_k = J_k^T lambda_{k+1} + c_k over the window, backwards from
+// carry[traj][NX] (last window: zero); lam[traj][ld][NX] receives lambda_{k+1}
+// at row k.  Lane j owns lambda_j: a step is NX shuffles and a chain of NX / 2
+// FMAs and an add.  The records pass through shared memory in chunks, copied
+// by the lanes of their own trajectory.
+template <int NX>
+constexpr int kAdjChunk = NX <= 4 ? 16 : 8;
+
+template <int NX>
+__global__ void __launch_bounds__(32) adjoint_kernel(const float* __restrict__ adj, int n_traj, int len, int ld,
+                                                     int first, float* __restrict__ carry, float* __restrict__ lam)
+{
+    constexpr int L = kLanes<NX>, PER = 32 / L, C = kAdjChunk<NX>, R = kRec<NX>;
+    // a trajectory's chunk padded by 4 floats: the groups of a warp read distinct banks
+    __shared__ __align__(16) float sj[kStages][PER][C * R + 4];
+    const int l = (int)threadIdx.x % L, j = l % NX, grp = (int)threadIdx.x / L;
+    const int tr = blockIdx.x * PER + grp;
+    const bool own = tr < n_traj && l < NX;
+    const size_t t = tr < n_traj ? tr : n_traj - 1;
+    float v = first ? 0.f : carry[t * NX + j];
+    float* lt = lam + t * ld * NX + j;
+    const float* at = adj + t * ld * R;
+    const int n_chunk = (len + C - 1) / C;
+    // chunk c holds steps [max(len - (c + 1) C, 0), len - c C), in order
+    auto fetch = [&](int c) {
+        const int lo = len - (c + 1) * C;
+        float* dst = &sj[c % kStages][grp][4 * l];
+        if (lo >= 0) {
+            const float* src = at + (size_t)lo * R + 4 * l;
+#pragma unroll
+            for (int i = 0; i < C * R; i += 4 * L)
+                if (C * R % (4 * L) == 0 || i + 4 * l < C * R) copy_async<16>(dst + i, src + i);
+        } else {
+            for (int i = 4 * l; i < (lo + C) * R; i += 4 * L) copy_async<16>(dst + (i - 4 * l), at + i);
+        }
+        copy_commit();
+    };
+    auto step = [&](int k, const float* rec) {
+        if (own) lt[(size_t)k * NX] = v;
+        float J[NX], n = rec[NX * NX + j], m = 0.f;
+        load_vec<NX>(rec + j * NX, J);
+#pragma unroll
+        for (int r = 0; r < NX; r += 2) {
+            n = fmaf(J[r], __shfl_sync(0xffffffffu, v, r, L), n);
+            m = fmaf(J[r + 1], __shfl_sync(0xffffffffu, v, r + 1, L), m);
+        }
+        v = n + m;
+    };
+#pragma unroll
+    for (int c = 0; c < kStages - 1; ++c) fetch(c);
+    for (int c = 0; c < n_chunk; ++c) {
+        copy_wait<kStages - 2>();
+        fetch(c + kStages - 1);
+        const int lo = len - (c + 1) * C;
+        const float* rec = sj[c % kStages][grp];
+        if (lo >= 0) {
+#pragma unroll
+            for (int q = C - 1; q >= 0; --q) step(lo + q, rec + q * R);
+        } else {
+            for (int q = lo + C - 1; q >= 0; --q) step(q, rec + q * R);
+        }
+    }
+    if (own) carry[t * NX + j] = v;
+}
+
+// The gradient's data term: every entry of theta is a sum over the samples of
+// a product of two of the sample's quantities (a z^T for M_0, p a z^T for M_1,
+// d1 z^T for W1, d2 h1^T for W2, ...).  A block takes tiles of kTile samples:
+// each thread puts one sample's quantities into shared memory, then each
+// entry's threads sum the tile (FP32 in parts of kPart samples, added up in
+// FP64).  part[block][q].
+template <int NX>
+struct Outer {
+    using Q = Lay<NX>;
+    // rows of the tile: a, p a, d1, d2, s, z, h1, h2, 1
+    static constexpr int A = 0, PA = Q::NO, D1 = 2 * Q::NO, D2 = D1 + NH, S = D2 + NH, Z = S + 1, H1 = Z + Q::NZ,
+                         H2 = H1 + NH, ONE = H2 + NH, ROWS = ONE + 1;
+    static constexpr int kTile = 128, kLd = kTile + 1;   // odd row stride: rows of one column lie in distinct banks
+    static constexpr int kThreads = ((Q::N + 31) / 32) * 32 < kTile ? kTile : ((Q::N + 31) / 32) * 32;
+    static constexpr int kPart = 32;
+};
+
+template <int NX>
+__global__ void __launch_bounds__(Outer<NX>::kThreads)
+    outer_kernel(const float* __restrict__ theta, const float* __restrict__ u, const float* __restrict__ y,
+                 const float* __restrict__ scales, int n_traj, int T, int k0, int len, int ld, float inv_n, int first,
+                 const float* __restrict__ xh, const float* __restrict__ lam, double* __restrict__ part)
+{
+    using Q = Lay<NX>;
+    using O = Outer<NX>;
+    __shared__ float th[Q::N];
+    __shared__ float tile[O::ROWS][O::kLd];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < Q::N; i += O::kThreads) th[i] = theta[i];
+    // the two rows whose product this thread's entry sums
+    int ra = O::ONE, rb = O::ONE;
+    {
+        const int q = tid;
+        auto outer = [&](int base, int cols, int r0, int c0) { ra = r0 + (q - base) / cols, rb = c0 + (q - base) % cols; };
+        if (q < Q::M1) outer(Q::M0, Q::NZ, O::A, O::Z);
+        else if (q < Q::W1) outer(Q::M1, Q::NZ, O::PA, O::Z);
+        else if (q < Q::B1) outer(Q::W1, Q::NZ, O::D1, O::Z);
+        else if (q < Q::W2) ra = O::D1 + q - Q::B1;
+        else if (q < Q::B2) outer(Q::W2, NH, O::D2, O::H1);
+        else if (q < Q::W3) ra = O::D2 + q - Q::B2;
+        else if (q < Q::B3) ra = O::S, rb = O::H2 + q - Q::W3;
+        else if (q == Q::B3) ra = O::S;
+    }
+    const long long n = (long long)n_traj * len;
+    double acc = 0.0;
+    for (long long s0 = blockIdx.x * (long long)O::kTile; s0 < n; s0 += (long long)gridDim.x * O::kTile) {
+        __syncthreads();
+        if (tid < O::kTile) {
+            const long long s = s0 + tid;
+            float q[O::ROWS];
+#pragma unroll
+            for (int i = 0; i < O::ROWS; ++i) q[i] = 0.f;
+            if (s < n) {
+                const size_t t = (size_t)(s / len);
+                const int k = (int)(s % len);
+                Sample<NX> S;
+                const size_t row = (t * T + k0 + k) * 3;
+                eval_sample<NX>(th, scales, xh + (t * T + k0 + k) * NX, u + row, y + row, S);
+                float a[Q::NO], d2[NH], e[NH];
+                load_vec<NX>(lam + (t * ld + k) * NX, a);
+#pragma unroll
+                for (int c = 0; c < NY; ++c) a[NX + c] = 2.0f * S.res[c] * inv_n;
+                float sp = 0.f;  // dJ/dp
 #pragma unroll
                 for (int r = 0; r < Q::NO; ++r) {
                     float m1z = 0.f;
 #pragma unroll
-                    for (int j = 0; j < Q::NZ; ++j) {
-                        const int q = r * Q::NZ + j;
-                        const float az = a[r] * z[j];
-                        my[(Q::M0 + q) * kThreads] += az;
-                        my[(Q::M1 + q) * kThreads] += p * az;
-                        m1z = fmaf(th[Q::M1 + q], z[j], m1z);
-                    }
-                    s = fmaf(a[r], m1z, s);
+                    for (int j = 0; j < Q::NZ; ++j) m1z = fmaf(th[Q::M1 + r * Q::NZ + j], S.z[j], m1z);
+                    sp = fmaf(a[r], m1z, sp);
+                    q[O::A + r] = a[r];
+                    q[O::PA + r] = S.p * a[r];
                 }
-                // back through the scheduling network
-                float d2[NH], d1[NH];
+                eta_back<NX>(th, S.h1, S.h2, d2, e);
 #pragma unroll
                 for (int i = 0; i < NH; ++i) {
-                    my[(Q::W3 + i) * kThreads] += s * h2[i];
-                    d2[i] = s * th[Q::W3 + i] * (1.0f - h2[i] * h2[i]);
-                    my[(Q::B2 + i) * kThreads] += d2[i];
+                    q[O::D1 + i] = sp * e[i];
+                    q[O::D2 + i] = sp * d2[i];
+                    q[O::H1 + i] = S.h1[i];
+                    q[O::H2 + i] = S.h2[i];
                 }
-                my[Q::B3 * kThreads] += s;
+                q[O::S] = sp;
+                q[O::ONE] = 1.0f;
 #pragma unroll
-                for (int i = 0; i < NH; ++i) {
-                    float b = 0.f;
-#pragma unroll
-                    for (int j = 0; j < NH; ++j) {
-                        my[(Q::W2 + i * NH + j) * kThreads] += d2[i] * h1[j];
-                        b = fmaf(th[Q::W2 + j * NH + i], d2[j], b);
-                    }
-                    d1[i] = b * (1.0f - h1[i] * h1[i]);
-                    my[(Q::B1 + i) * kThreads] += d1[i];
-                }
-#pragma unroll
-                for (int i = 0; i < NH; ++i)
-#pragma unroll
-                    for (int j = 0; j < Q::NZ; ++j) my[(Q::W1 + i * Q::NZ + j) * kThreads] += d1[i] * z[j];
-                // dJ/dx_k = (M^T a + W1^T d1)[0..nx)
-#pragma unroll
-                for (int j = 0; j < NX; ++j) {
-                    float v = 0.f;
-#pragma unroll
-                    for (int r = 0; r < Q::NO; ++r)
-                        v = fmaf(fmaf(p, th[Q::M1 + r * Q::NZ + j], th[Q::M0 + r * Q::NZ + j]), a[r], v);
-#pragma unroll
-                    for (int i = 0; i < NH; ++i) v = fmaf(th[Q::W1 + i * Q::NZ + j], d1[i], v);
-                    lam[j] = v;
-                }
+                for (int j = 0; j < Q::NZ; ++j) q[O::Z + j] = S.z[j];
             }
+#pragma unroll
+            for (int i = 0; i < O::ROWS; ++i) tile[i][tid] = q[i];
+        }
+        __syncthreads();
+        for (int b = 0; b < O::kTile; b += O::kPart) {
+            float f = 0.f;
+#pragma unroll 8
+            for (int i = b; i < b + O::kPart; ++i) f = fmaf(tile[ra][i], tile[rb][i], f);
+            acc += (double)f;
         }
     }
-    lbuf[tid] = lsum;
-    __syncthreads();
-    double* pb = part + (size_t)blockIdx.x * (Q::N + 1);
-    if (want_grad) {
-        for (int q = tid; q < Q::N; q += kThreads) {
-            double s = 0.0;
-            for (int t = 0; t < kThreads; ++t) s += (double)acc[q * kThreads + t];
-            pb[q] = s;
-        }
-    }
-    if (tid == 0) {
-        double s = 0.0;
-        for (int t = 0; t < kThreads; ++t) s += lbuf[t];
-        pb[Q::N] = s;
+    if (tid < Q::N) {
+        double* o = part + (size_t)blockIdx.x * Q::N + tid;
+        *o = first ? acc : *o + acc;  // windows add up in order
     }
 }
 
-// Sums the block partials in block order, adds the l2 term, masks the fixed
-// entries: loss = sum_sq * inv_n + sigma2/2 |theta|^2, grad = sum + sigma2 theta.
-__global__ void final_kernel(const double* __restrict__ part, int nblk, int N, int nx, const float* __restrict__ theta,
-                             float sigma2, double inv_n, int want_grad, int stage, double* __restrict__ loss,
-                             float* __restrict__ grad)
+// Block q < N: grad[q] = sum of the partials (fixed order) + sigma2 theta[q],
+// zero where the stage holds it; block N: loss = sum_sq inv_n + sigma2/2 |theta|^2.
+// One warp per block: lane-strided sums, then a shuffle tree.
+__global__ void __launch_bounds__(32)
+    final_kernel(const double* __restrict__ part, int nblk, const double* __restrict__ loss_part, int nloss, int N,
+                 int nx, const float* __restrict__ theta, float sigma2, double inv_n, int stage,
+                 double* __restrict__ loss, float* __restrict__ grad)
 {
-    __shared__ double sq[512];
-    const int q = threadIdx.x;
-    double t2 = 0.0;
+    const int q = (int)blockIdx.x + (grad ? 0 : N), lane = threadIdx.x;  // without a gradient only the loss
+    double v = 0.0, t2 = 0.0;
     if (q < N) {
-        const double th = (double)theta[q];
-        t2 = th * th;
-        if (want_grad) {
-            double g = 0.0;
-            for (int b = 0; b < nblk; ++b) g += part[(size_t)b * (N + 1) + q];
-            g += (double)sigma2 * th;
-            grad[q] = trainable(q, nx, stage) ? (float)g : 0.f;
-        }
+        for (int b = lane; b < nblk; b += 32) v += part[(size_t)b * N + q];
+    } else {
+        for (int b = lane; b < nloss; b += 32) v += loss_part[b];
+        for (int i = lane; i < N; i += 32) t2 += (double)theta[i] * (double)theta[i];
     }
-    sq[q] = t2;
-    __syncthreads();
-    if (q == 0) {
-        double s = 0.0, r = 0.0;
-        for (int i = 0; i < N; ++i) r += sq[i];
-        for (int b = 0; b < nblk; ++b) s += part[(size_t)b * (N + 1) + N];
-        *loss = s * inv_n + 0.5 * (double)sigma2 * r;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        v += __shfl_down_sync(0xffffffffu, v, o);
+        t2 += __shfl_down_sync(0xffffffffu, t2, o);
     }
+    if (lane) return;
+    if (q < N) grad[q] = trainable(q, nx, stage) ? (float)(v + (double)sigma2 * (double)theta[q]) : 0.f;
+    else *loss = v * inv_n + 0.5 * (double)sigma2 * t2;
 }
 
 // ---------------------------------------------------------------------------
@@ -687,10 +1001,10 @@ struct slpv_model {
     float* scales = nullptr;
     double *acc_loss = nullptr, *loss = nullptr;
     int* t = nullptr;
-    double* part = nullptr;
-    size_t part_cap = 0;
-    float* xh = nullptr;
-    size_t xh_cap = 0;
+    double *part = nullptr, *loss_part = nullptr;  // block partials of the gradient and the loss
+    float *xh = nullptr, *win = nullptr, *carry = nullptr;  // state history; adjoint window; state and adjoint between windows
+    size_t xh_cap = 0, win_cap = 0, carry_cap = 0;
+    int loss_cap = 0;
     double* spart = nullptr;
     double* lb = nullptr;  // L-BFGS state, allocated on first use
     int* lb_count = nullptr;
@@ -721,53 +1035,85 @@ cudaError_t by_nx(int nx, F&& f)
     }
 }
 
-size_t grad_smem(int N) { return (size_t)((N + 3) & ~3) * 4 + (size_t)N * kThreads * 4 + kThreads * 8; }
+// Bytes of a window of the time axis: the per-sample buffers of the adjoint
+// (NX^2 + 2 NX floats a sample) and, for the loss alone, the states, are
+// bounded by this and stay in L2; a fit of a few dozen trajectories is one window.
+constexpr size_t kWindowBytes = 64ull << 20;
+constexpr int kSampleBlocks = 152 * 8, kOuterBlocks = 152 * 2;
 
-// Ensures the per-call buffers (block partials, state history) are large enough.
-int reserve(slpv_model* m, int n_traj, int T, bool grad)
+int grow(float** p, size_t* cap, size_t n)
 {
-    const size_t nblk = (size_t)(n_traj + kThreads - 1) / kThreads;
-    const size_t pneed = nblk * (m->N + 1);
-    if (pneed > m->part_cap) {
-        cudaFree(m->part);
-        m->part = nullptr;
-        m->part_cap = 0;
-        SCK(cudaMalloc(&m->part, pneed * sizeof(double)));
-        m->part_cap = pneed;
-    }
-    const size_t xneed = grad ? (size_t)n_traj * T * m->cfg.nx : 0;
-    if (xneed > m->xh_cap) {
-        cudaFree(m->xh);
-        m->xh = nullptr;
-        m->xh_cap = 0;
-        cudaError_t e = cudaMalloc(&m->xh, xneed * sizeof(float));
-        if (e != cudaSuccess) return sph::set_last_error(SPH_E_NOMEM, "slpv: state history allocation failed");
-        m->xh_cap = xneed;
-    }
+    if (n <= *cap) return SPH_OK;
+    cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
+    if (cudaMalloc(p, n * sizeof(float)) != cudaSuccess)
+        return sph::set_last_error(SPH_E_NOMEM, "slpv: workspace allocation failed");
+    *cap = n;
     return SPH_OK;
 }
+
+int blocks_for(long long n, int per, int most) { return (int)std::min<long long>((n + per - 1) / per, most); }
 
 // Launches the loss (and gradient) into m->loss / grad_out.
 int loss_grad_launch(slpv_model* m, const float* u, const float* y, int n_traj, int T, int stage, float* grad_out,
                      cudaStream_t st)
 {
     const bool want = grad_out != nullptr;
-    int rc = reserve(m, n_traj, T, want);
+    const int nx = m->cfg.nx;
+    const size_t per = want ? (size_t)(nx * nx + nx + 3) / 4 * 4 + nx : (size_t)nx;  // floats of a sample in the window
+    const int W = (int)std::min<size_t>((size_t)T, std::max<size_t>(kWindowBytes / 4 / per / (size_t)n_traj, 16));
+    int rc = grow(&m->win, &m->win_cap, (size_t)n_traj * W * per);
+    if (!rc) rc = grow(&m->carry, &m->carry_cap, 2 * (size_t)n_traj * nx);
+    if (!rc && want) rc = grow(&m->xh, &m->xh_cap, (size_t)n_traj * T * nx);
     if (rc) return rc;
-    const int nblk = (n_traj + kThreads - 1) / kThreads;
-    const float inv_n = (float)(1.0 / ((double)n_traj * T));
-    const size_t smem = grad_smem(m->N);
-    cudaError_t e = by_nx(m->cfg.nx, [&](auto c) {
+    const double inv_nd = 1.0 / ((double)n_traj * T);
+    const float inv_n = (float)inv_nd;
+    const int n_win = (T + W - 1) / W;
+    const int sblk = blocks_for((long long)n_traj * W, kSampleThreads, kSampleBlocks);
+    if (n_win * (long long)sblk > (long long)m->loss_cap) {
+        cudaFree(m->loss_part);
+        m->loss_part = nullptr;
+        m->loss_cap = 0;
+        SCK(cudaMalloc(&m->loss_part, (size_t)n_win * sblk * sizeof(double)));
+        m->loss_cap = n_win * sblk;
+    }
+    int oblk = 0, n_loss = 0;
+    cudaError_t e = by_nx(nx, [&](auto c) {
         constexpr int NX = decltype(c)::value;
-        cudaError_t a = cudaFuncSetAttribute(grad_kernel<NX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (a != cudaSuccess) return a;
-        grad_kernel<NX><<<nblk, kThreads, smem, st>>>(m->th, u, y, m->scales, n_traj, T, inv_n, want ? 1 : 0, m->xh,
-                                                      m->part);
+        const int sgrid = (n_traj * kLanes<NX> + 31) / 32;
+        float* lam = m->win + (size_t)n_traj * W * kRec<NX>;
+        auto sample = [&](int w, const float* xh, int xld, int xk0) {
+            const int k0 = w * W, len = std::min(W, T - k0);
+            const int nb = blocks_for((long long)n_traj * len, kSampleThreads, kSampleBlocks);
+            sample_kernel<NX><<<nb, kSampleThreads, 0, st>>>(m->th, u, y, m->scales, n_traj, T, k0, len, W, xld, xk0,
+                                                             inv_n, want ? 1 : 0, xh, m->win, m->loss_part + n_loss);
+            n_loss += nb;
+        };
+        if (!want) {  // the states of a window at a time
+            for (int w = 0; w < n_win; ++w) {
+                const int k0 = w * W;
+                state_kernel<NX><<<sgrid, 32, 0, st>>>(m->th, u, m->scales, n_traj, T, k0, std::min(W, T - k0), W,
+                                                       m->carry, m->win);
+                sample(w, m->win, W, k0);
+            }
+            return cudaGetLastError();
+        }
+        state_kernel<NX><<<sgrid, 32, 0, st>>>(m->th, u, m->scales, n_traj, T, 0, T, T, m->carry, m->xh);
+        oblk = blocks_for((long long)n_traj * W, Outer<NX>::kTile, kOuterBlocks);
+        for (int w = n_win - 1; w >= 0; --w) {
+            const int k0 = w * W, len = std::min(W, T - k0), first = w == n_win - 1 ? 1 : 0;
+            sample(w, m->xh, T, 0);
+            adjoint_kernel<NX><<<sgrid, 32, 0, st>>>(m->win, n_traj, len, W, first, m->carry + (size_t)n_traj * NX,
+                                                     lam);
+            outer_kernel<NX><<<oblk, Outer<NX>::kThreads, 0, st>>>(m->th, u, y, m->scales, n_traj, T, k0, len, W, inv_n,
+                                                                   first, m->xh, lam, m->part);
+        }
         return cudaGetLastError();
     });
     SCK(e);
-    final_kernel<<<1, 512, 0, st>>>(m->part, nblk, m->N, m->cfg.nx, m->th, m->cfg.sigma2, 1.0 / ((double)n_traj * T),
-                                    want ? 1 : 0, stage, m->loss, grad_out);
+    final_kernel<<<want ? m->N + 1 : 1, 32, 0, st>>>(m->part, oblk, m->loss_part, n_loss, m->N, nx, m->th,
+                                                     m->cfg.sigma2, inv_nd, stage, m->loss, grad_out);
     SCK(cudaGetLastError());
     return SPH_OK;
 }
@@ -803,7 +1149,10 @@ int slpv_destroy(slpv_model* m)
     cudaFree(m->loss);
     cudaFree(m->t);
     cudaFree(m->part);
+    cudaFree(m->loss_part);
     cudaFree(m->xh);
+    cudaFree(m->win);
+    cudaFree(m->carry);
     cudaFree(m->spart);
     cudaFree(m->lb);
     cudaFree(m->lb_count);
@@ -826,7 +1175,8 @@ int slpv_create(const slpv_config* cfg, slpv_model** out)
               cudaMalloc(&m->scales, 6 * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&m->acc_loss, sizeof(double)) == cudaSuccess &&
               cudaMalloc(&m->loss, sizeof(double)) == cudaSuccess && cudaMalloc(&m->t, sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&m->spart, kStatBlocks * 6 * sizeof(double)) == cudaSuccess;
+              cudaMalloc(&m->spart, kStatBlocks * 6 * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&m->part, (size_t)kOuterBlocks * m->N * sizeof(double)) == cudaSuccess;
     if (!ok) {
         slpv_destroy(m);
         return sph::set_last_error(SPH_E_NOMEM, "slpv_create: cudaMalloc failed");
