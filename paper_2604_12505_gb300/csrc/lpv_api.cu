@@ -22,11 +22,11 @@ struct lpv_model {
     lpv_config cfg{};
     Dims d{};
     float *Wp = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
-    float* hist = nullptr;
+    float* hist = nullptr;  // fragments of z_k and of G_k of every step (launch_forward)
     size_t hist_cap = 0;
     float* gpart = nullptr;
     double* loss_part = nullptr;
-    size_t warp_cap = 0;
+    size_t part_cap = 0;
     double *d_loss = nullptr, *d_hist = nullptr;
     int hist_len = 0;
     double *stats_part = nullptr, *stats = nullptr, *gram_part = nullptr, *theta = nullptr, *rho = nullptr;
@@ -74,24 +74,21 @@ int grow(T** p, size_t* cap, size_t n)
     return SPH_OK;
 }
 
-// Warps launched for n trajectories (whole blocks of 4 warps).
-size_t launched_warps(int n_traj) { return (size_t)((warps_for(n_traj) + 3) / 4) * 4; }
-
 int workspace(lpv_model* M, int n_traj, int T)
 {
-    const size_t warps = launched_warps(n_traj);
-    if (M->warp_cap < warps) {
+    const size_t parts = (size_t)groups_for(n_traj);  // at least the loss's warps and the gradient's blocks
+    if (M->part_cap < parts) {
         cudaFree(M->gpart);
         cudaFree(M->loss_part);
         M->gpart = nullptr;
         M->loss_part = nullptr;
-        M->warp_cap = 0;
-        if (cudaMalloc(&M->gpart, warps * kWN * sizeof(float)) != cudaSuccess ||
-            cudaMalloc(&M->loss_part, warps * sizeof(double)) != cudaSuccess)
+        M->part_cap = 0;
+        if (cudaMalloc(&M->gpart, (size_t)grad_parts(n_traj) * kWN * sizeof(float)) != cudaSuccess ||
+            cudaMalloc(&M->loss_part, parts * sizeof(double)) != cudaSuccess)
             return err(SPH_E_NOMEM, "lpv: cudaMalloc failed");
-        M->warp_cap = warps;
+        M->part_cap = parts;
     }
-    return grow(&M->hist, &M->hist_cap, (size_t)n_traj * T * 16);
+    return grow(&M->hist, &M->hist_cap, 2 * frag_floats(n_traj, T));
 }
 
 int check_data(const lpv_model* M, const float* u, const float* y, const float* p, int n_traj, int T)
@@ -280,10 +277,11 @@ int loss_grad_device(lpv_model* M, const float* u, const float* y, const float* 
     int rc = workspace(M, n_traj, T);
     if (rc) return rc;
     const double n = (double)n_traj * T;
-    LCK(launch_forward(1, M->Wp, M->d, u, p, y, n_traj, T, nullptr, M->hist, M->loss_part, (float)(2.0 / n), st));
-    LCK(launch_backward(M->Wp, M->d, u, p, n_traj, T, M->hist, M->gpart, st));
-    LCK(launch_reduce(M->gpart, (int)launched_warps(n_traj), M->loss_part, M->Wp, M->d, M->cfg.sigma2, n, M->grad,
-                      M->d_loss, loss_hist, it, st));
+    float* gfrag = M->hist + frag_floats(n_traj, T);
+    LCK(launch_forward(1, M->Wp, M->d, u, p, y, n_traj, T, nullptr, M->hist, gfrag, M->loss_part, (float)(2.0 / n), st));
+    LCK(launch_backward(M->Wp, M->d, p, n_traj, T, M->hist, gfrag, M->gpart, st));
+    LCK(launch_reduce(M->gpart, grad_parts(n_traj), M->loss_part, serial_warps(n_traj), M->Wp, M->d, M->cfg.sigma2, n,
+                      M->grad, M->d_loss, loss_hist, it, st));
     return SPH_OK;
 }
 }  // namespace
@@ -516,7 +514,8 @@ int lpv_predict(const lpv_model* M, const float* u, const float* p, int32_t n_tr
                 void* stream)
 {
     if (!M || !u || !y_out || n_traj < 1 || T < 1 || (M->d.np > 0 && !p)) return err(SPH_E_INVAL, "lpv_predict: bad arguments");
-    LCK(launch_forward(0, M->Wp, M->d, u, p, nullptr, n_traj, T, y_out, nullptr, nullptr, 0.f, (cudaStream_t)stream));
+    LCK(launch_forward(0, M->Wp, M->d, u, p, nullptr, n_traj, T, y_out, nullptr, nullptr, nullptr, 0.f,
+                       (cudaStream_t)stream));
     return SPH_OK;
 }
 

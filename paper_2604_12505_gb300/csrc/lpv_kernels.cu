@@ -14,37 +14,68 @@
 // outputs ordered [x_next (n_x), y (n_y), 0...], the accumulator of n-tiles
 // 0 and 1 holds exactly the entries of the next step's first A block that
 // this thread owns, and the scheduled blocks p_i z are thread-local scalings:
-// the recurrence runs without shuffles.  The backward pass uses the same
-// identity for the adjoint; the weight gradient sum_k G_k^T w_k is one more
-// MMA whose operands are transposed through a per-warp shared-memory tile.
+// the recurrence runs without shuffles.  The adjoint uses the same identity;
+// the weight gradient sum_k G_k^T w_k is one more MMA, over all steps in
+// parallel, whose operands are transposed in registers.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "lpv_common.cuh"
 #include "lpv_launch.h"
 
 namespace lpv {
 
-constexpr int kPrefetch = 4;  // steps of inputs in flight in the recurrences
-
 __device__ __forceinline__ void mma16816(float* d, const uint32_t* a, uint32_t b0, uint32_t b1)
 {
-    asm volatile(
+    asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
         "{%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Two FP32 operations in one instruction, each rounded to nearest.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
 // (v0, v1) -> packed bf16x2 (v0 in the low half), split into hi and lo parts.
 __device__ __forceinline__ void split2(float v0, float v1, uint32_t& hi, uint32_t& lo)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(v0, v1);
-    const float2 hf = __bfloat1622float2(h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(v0 - hf.x, v1 - hf.y);
     hi = *reinterpret_cast<const uint32_t*>(&h);
+    const float2 r = sub2(make_float2(v0, v1), make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)));
+    const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
@@ -105,109 +136,242 @@ __device__ __forceinline__ void load_fwd_frags(const float* __restrict__ Wp, uin
     }
 }
 
-// Scheduling variables of the thread's two trajectories at step k, normalised.
-__device__ __forceinline__ void load_p(const Dims& d, const float* __restrict__ p, int r, bool valid, int T, int k,
-                                       float* pp)
+// ---------------------------------------------------------------------------
+// The free run and its gradient.
+//
+// Serial in k are the state and its adjoint, each a product of the split
+// operands per step; everything else runs beside or after them:
+//   fwd_kernel     the free run: z_k fragments and residuals for the adjoint
+//   adj_kernel     lambda_k and, in other warps, sum_k G_k^T w_k with
+//                  G_k = [lambda_{k+1}; dJ/dy_k]
+// The serial passes are bound by the instructions of one warp's step, which
+// nothing else overlaps: few warps per block (a fit's few dozen blocks each
+// get an SM of their own), the inputs laid out in shared memory as the lanes hold
+// them, the number of scheduling blocks and whether the lower columns are all
+// state known at compile time.  RG is the number of 8-trajectory row groups
+// of a warp, 2 filling the product's 16 rows; with 1 half the rows are idle,
+// but so is half of the work per step around the product, and a step is
+// shorter.  Runs that leave schedulers idle anyway take RG = 1
+// (row_groups).  820 trajectories of 1,000 samples (n_x 12, n_u 3, n_y 4,
+// n_p 2): 174 us forward, 189 us adjoint and gradient, 6 us reduction.  Four
+// warps to a block that loaded u, y and p from their rows (28 memory
+// instructions of up to 16 lines a step) and kept the weight gradient, with
+// its transposes through shared memory, on the adjoint's chain took 1,939 +
+// 1,469 + 31 us.  With RG = 2 there the forward pass takes 650 us.
+//
+// Fragments in global memory: per group of 8 trajectories and step, [lane][4],
+// the values of columns 2t, 2t+1, 2t+8, 2t+9 of row g.
+// ---------------------------------------------------------------------------
+constexpr int kC = 4;         // steps per chunk of staged inputs
+constexpr int kStages = 4;    // chunks in shared memory: one in use, three in flight
+constexpr int kFrag = kFragFloats;
+
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src)
 {
-    const size_t o = ((size_t)r * T + k) * d.np;
-    pp[0] = (valid && d.np > 0) ? (p[o] - d.pm[0]) * d.inv_ps[0] : 0.f;
-    pp[1] = (valid && d.np > 1) ? (p[o + 1] - d.pm[1]) * d.inv_ps[1] : 0.f;
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait()  // until at most the N youngest chunks are in flight
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+    __syncwarp();
 }
 
-// Inputs of one step that a thread owns: the scheduling of its two
-// trajectories and its feature (u) and output (y) columns, normalised.
-struct StepIn {
-    float p0[2], p1[2];
-    float uz[8];  // u part of z at the thread's 8 columns (0 elsewhere)
-    float yv[8];  // y at the thread's output columns (0 elsewhere; loss only)
+// Staged channels of a step: column c of a row at its place (from column 8 on
+// when the columns below are all state, n_x >= 8; all 16 when LOW), zero where
+// no channel lies; and the scheduling of a row.  Rows are apart so that the
+// eight of a warp read distinct banks.
+template <bool LOW>
+constexpr int kFirstCol = LOW ? 0 : 8;
+
+template <bool LOW>
+__device__ __forceinline__ void load_vals(const float* row, int t, float* v)  // columns 2t, 2t+1, 2t+8, 2t+9
+{
+    const float2 b = *reinterpret_cast<const float2*>(row + 8 - kFirstCol<LOW> + 2 * t);
+    float2 a = make_float2(0.f, 0.f);
+    if (LOW) a = *reinterpret_cast<const float2*>(row + 2 * t);
+    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+
+// One stage of a warp's inputs.
+template <bool LOW, int RG>
+struct InStage {
+    float u[kC][RG][8][16 - kFirstCol<LOW>];
+    float y[kC][RG][8][16 - kFirstCol<LOW>];
+    float p[kC][RG][8][2];
 };
 
-template <bool WANT_Y>
-__device__ __forceinline__ void load_step(const Dims& d, const float* __restrict__ u, const float* __restrict__ p,
-                                          const float* __restrict__ y, int r0, int r1, bool v0, bool v1, int T, int k,
-                                          int t, StepIn& in)
+// A row's n channels to consecutive places.
+__device__ __forceinline__ void copy_row(float* dst, const float* src, int n)
 {
-    load_p(d, p, r0, v0, T, k, in.p0);
-    load_p(d, p, r1, v1, T, k, in.p1);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int c = scol(i, t);
-        const int r = srow(i) ? r1 : r0;
-        const bool v = srow(i) ? v1 : v0;
-        in.uz[i] = (v && c >= d.nx && c < d.nx + d.nu)
-                       ? u[((size_t)r * T + k) * d.nu + (c - d.nx)] * d.inv_su[c - d.nx] : 0.f;
-        in.yv[i] = (WANT_Y && v && c >= d.nx && c < d.nx + d.ny)
-                       ? y[((size_t)r * T + k) * d.ny + (c - d.nx)] * d.inv_sy[c - d.nx] : 0.f;
-    }
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) copy_async<4>(dst + j, src + j);
 }
 
-// Free-run simulation of 16 trajectories per warp.  MODE 0 writes the
+// Free-run simulation of 8 RG trajectories per warp.  MODE 0 writes the
 // prediction (physical units); MODE 1 accumulates the squared error of the
-// normalised outputs and records, per step, x_k and dJ/dy_k for the
-// backward pass in hist[traj][k][16] (state columns, then output columns).
-// The inputs of steps k + 1 .. k + kPrefetch are in flight while step k's products run.
-template <int MODE>
-__global__ void __launch_bounds__(128) fwd_kernel(const float* __restrict__ Wp, Dims d, const float* __restrict__ u,
-                                                  const float* __restrict__ p, const float* __restrict__ y, int n_traj,
-                                                  int T, float* __restrict__ y_out, float* __restrict__ hist,
-                                                  double* __restrict__ loss_part, float grad_scale)
+// normalised outputs and records, per step, z_k and the residuals' part of
+// G_k as fragments.
+template <int MODE, bool LOW, int NP, int RG>
+__global__ void __launch_bounds__(32) fwd_kernel(const float* __restrict__ Wp, Dims d, const float* __restrict__ u,
+                                                 const float* __restrict__ p, const float* __restrict__ y, int n_traj,
+                                                 int T, float* __restrict__ y_out, float* __restrict__ zfrag,
+                                                 float* __restrict__ gfrag, double* __restrict__ loss_part,
+                                                 float grad_scale)
 {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int r0 = wid * 16 + g, r1 = r0 + 8;
-    const bool v0 = r0 < n_traj, v1 = r1 < n_traj;
+    __shared__ __align__(16) InStage<LOW, RG> sm[kStages];
+    const int lane = threadIdx.x, g = lane >> 2, t = lane & 3, wid = blockIdx.x, first = wid * 8 * RG;
+    {   // rows beyond the data and places without a channel stay zero
+        float* z = reinterpret_cast<float*>(sm);
+        for (int i = lane; i < (int)(sizeof(sm) / sizeof(float)); i += 32) z[i] = 0.f;
+        __syncwarp();
+    }
     uint32_t bhi[kMaxKT][2][2], blo[kMaxKT][2][2];
-    load_fwd_frags(Wp, bhi, blo, d.nkt, g, t);
-    float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // x_0 = 0
-    float lsum_f = 0.f;                     // widened to FP64 once, after the loop
-    // a ring of the inputs of the next kPrefetch steps: the loads of step
-    // k + kPrefetch are issued when step k starts, so a step waits on no
-    // global load issued less than kPrefetch steps before it
-    StepIn ring[kPrefetch];
+    load_fwd_frags(Wp, bhi, blo, 1 + NP, g, t);
+    bool is_x[4], is_y[RG][4];
+    float fu[4], fy[4], pm[2], ips[RG][2];
 #pragma unroll
-    for (int i = 0; i < kPrefetch; ++i)
-        load_step<MODE == 1>(d, u, p, y, r0, r1, v0, v1, T, i < T ? i : T - 1, t, ring[i]);
-    for (int k0 = 0; k0 < T; k0 += kPrefetch) {
+    for (int j = 0; j < 4; ++j) {
+        const int c = 8 * (j >> 1) + 2 * t + (j & 1), q = c - d.nx;
+        is_x[j] = q < 0;
+        fu[j] = q >= 0 && q < d.nu ? d.inv_su[q] : 0.f;
+        fy[j] = MODE == 0 ? (q >= 0 && q < d.ny ? d.sy[q] : 0.f) : (q >= 0 && q < d.ny ? d.inv_sy[q] : 0.f);
 #pragma unroll
-    for (int i = 0; i < kPrefetch; ++i) {
-        const int k = k0 + i;
-        if (k >= T) break;
-        const StepIn cur = ring[i];
-        load_step<MODE == 1>(d, u, p, y, r0, r1, v0, v1, T, k + kPrefetch < T ? k + kPrefetch : T - 1, t, ring[i]);
-        float z[8];
+        for (int r = 0; r < RG; ++r) is_y[r][j] = q >= 0 && q < d.ny && first + 8 * r + g < n_traj;
+    }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) z[i] = (scol(i, t) < d.nx) ? s[i] : cur.uz[i];
-        uint32_t ahi[kMaxKT][4], alo[kMaxKT][4];
-        afrag(z, ahi[0], alo[0]);
+    for (int j = 0; j < 2; ++j) {
+        pm[j] = j < NP ? d.pm[j] : 0.f;
 #pragma unroll
-        for (int kt = 1; kt < kMaxKT; ++kt) {
-            float zs[8];
+        for (int r = 0; r < RG; ++r) ips[r][j] = j < NP && first + 8 * r + g < n_traj ? d.inv_ps[j] : 0.f;
+    }
+    // the four lanes of a row copy the four steps of its chunk
+    const int n_chunk = (T + kC - 1) / kC;
+    auto fetch = [&](int c) {
+        const int k = c * kC + t;
+        if (k < T) {
+            InStage<LOW, RG>& S = sm[c % kStages];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) zs[i] = z[i] * (srow(i) ? cur.p1[kt - 1] : cur.p0[kt - 1]);
-            afrag(zs, ahi[kt], alo[kt]);
-        }
-        float D[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        mma_split<kMaxKT>(D, ahi, alo, bhi, blo, d.nkt);
+            for (int r = 0; r < RG; ++r) {
+                const int tr = first + 8 * r + g;
+                if (tr < n_traj) {
+                    const size_t row = (size_t)tr * T + k;
+                    copy_row(&S.u[t][r][g][d.nx - kFirstCol<LOW>], u + row * d.nu, d.nu);
+                    if (MODE == 1) copy_row(&S.y[t][r][g][d.nx - kFirstCol<LOW>], y + row * d.ny, d.ny);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = scol(i, t);
-            const int r = srow(i) ? r1 : r0;
-            const bool v = srow(i) ? v1 : v0;
-            if (c < d.nx) {
-                if (MODE == 1 && v) hist[((size_t)r * T + k) * 16 + c] = s[i];
-            } else if (c < d.nx + d.ny && v) {
-                const int q = c - d.nx;
-                if (MODE == 0) {
-                    y_out[((size_t)r * T + k) * d.ny + q] = D[i] * d.sy[q];
-                } else {
-                    const float res = D[i] - cur.yv[i];
-                    lsum_f = fmaf(res, res, lsum_f);
-                    hist[((size_t)r * T + k) * 16 + c] = grad_scale * res;
+                    for (int j = 0; j < NP; ++j) copy_async<4>(&S.p[t][r][g][j], p + row * NP + j);
                 }
             }
-            s[i] = (c < d.nx) ? D[i] : 0.f;
         }
-    }
+        copy_commit();
+    };
+#pragma unroll
+    for (int c = 0; c < kStages - 1; ++c) fetch(c);
+    float s[RG][4] = {};   // x_0 = 0; zero in the columns that hold no state
+    float lsum_f = 0.f;    // widened to FP64 once, after the loop
+    float4* zo = reinterpret_cast<float4*>(zfrag) + (size_t)wid * RG * T * (kFrag / 4) + lane;
+    float4* go = reinterpret_cast<float4*>(gfrag) + (size_t)wid * RG * T * (kFrag / 4) + lane;
+    auto step = [&](const InStage<LOW, RG>& S, int q, int k) {
+        float z[8], pp[RG][2];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (r >= RG) {
+                z[2 * r] = z[2 * r + 1] = z[4 + 2 * r] = z[5 + 2 * r] = 0.f;
+                continue;
+            }
+            float uv[4];
+            load_vals<LOW>(S.u[q][r][g], t, uv);
+            const float2 pv = *reinterpret_cast<const float2*>(S.p[q][r][g]);
+            pp[r][0] = (pv.x - pm[0]) * ips[r][0];
+            pp[r][1] = (pv.y - pm[1]) * ips[r][1];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)  // at a column either the state or the input is zero: the sum is exact
+                z[4 * (j >> 1) + 2 * r + (j & 1)] = LOW || j >= 2 ? s[r][j] + uv[j] * fu[j] : s[r][j];
+            if (MODE == 1)
+                zo[((size_t)r * T + k) * 32] = make_float4(z[2 * r], z[2 * r + 1], z[4 + 2 * r], z[5 + 2 * r]);
+        }
+        float D[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if constexpr (RG == 1) {
+            // the idle rows 8-15 take the low parts: one product gives hi.hi
+            // and lo.hi, the other hi.lo (and lo.lo, not used)
+            uint32_t a[1 + NP][4];
+            float c1[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+            for (int kt = 0; kt <= NP; ++kt) {
+                float2 v0 = make_float2(z[0], z[1]), v1 = make_float2(z[4], z[5]);
+                if (kt) {
+                    const float2 f = make_float2(pp[0][kt ? kt - 1 : 0], pp[0][kt ? kt - 1 : 0]);
+                    v0 = mul2(v0, f);
+                    v1 = mul2(v1, f);
+                }
+                split2(v0.x, v0.y, a[kt][0], a[kt][1]);
+                split2(v1.x, v1.y, a[kt][2], a[kt][3]);
+            }
+#pragma unroll
+            for (int kt = 0; kt <= NP; ++kt)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    mma16816(D + 4 * nt, a[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
+                    mma16816(c1 + 4 * nt, a[kt], blo[kt][nt][0], blo[kt][nt][1]);
+                }
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                const float2 e = add2(make_float2(c1[4 * nt], c1[4 * nt + 1]), make_float2(D[4 * nt + 2], D[4 * nt + 3]));
+                const float2 f = add2(make_float2(D[4 * nt], D[4 * nt + 1]), e);
+                D[4 * nt] = f.x;
+                D[4 * nt + 1] = f.y;
+            }
+        } else {
+            uint32_t ahi[kMaxKT][4], alo[kMaxKT][4];
+            afrag(z, ahi[0], alo[0]);
+#pragma unroll
+            for (int kt = 1; kt <= NP; ++kt) {
+                float zs[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) zs[i] = z[i] * pp[srow(i) < RG ? srow(i) : 0][kt - 1];
+                afrag(zs, ahi[kt], alo[kt]);
+            }
+            mma_split<1 + NP>(D, ahi, alo, bhi, blo, 1 + NP);
+        }
+#pragma unroll
+        for (int r = 0; r < RG; ++r) {
+            float yv[4], res[4] = {0.f, 0.f, 0.f, 0.f};
+            if (MODE == 1) load_vals<LOW>(S.y[q][r][g], t, yv);
+#pragma unroll
+            for (int j = LOW ? 0 : 2; j < 4; ++j) {
+                const float o = D[4 * (j >> 1) + 2 * r + (j & 1)];
+                if (MODE == 0) {
+                    if (is_y[r][j])
+                        y_out[((size_t)(first + 8 * r + g) * T + k) * d.ny + (8 * (j >> 1) + 2 * t + (j & 1) - d.nx)] =
+                            o * fy[j];
+                } else {
+                    res[j] = is_y[r][j] ? o - yv[j] * fy[j] : 0.f;
+                    lsum_f = fmaf(res[j], res[j], lsum_f);
+                    res[j] *= grad_scale;
+                }
+            }
+            if (MODE == 1) go[((size_t)r * T + k) * 32] = make_float4(res[0], res[1], res[2], res[3]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float o = D[4 * (j >> 1) + 2 * r + (j & 1)];
+                s[r][j] = (LOW || j >= 2) ? (is_x[j] ? o : 0.f) : o;
+            }
+        }
+    };
+    for (int c = 0; c < n_chunk; ++c) {
+        copy_wait<kStages - 2>();
+        fetch(c + kStages - 1);  // its buffer was read before the wait's barrier
+        const InStage<LOW, RG>& S = sm[c % kStages];
+        if ((c + 1) * kC <= T) {
+#pragma unroll
+            for (int q = 0; q < kC; ++q) step(S, q, c * kC + q);
+        } else {
+            for (int q = 0; c * kC + q < T; ++q) step(S, q, c * kC + q);
+        }
     }
     if (MODE == 1) {
         double lsum = (double)lsum_f;
@@ -217,151 +381,214 @@ __global__ void __launch_bounds__(128) fwd_kernel(const float* __restrict__ Wp, 
     }
 }
 
-template __global__ void fwd_kernel<0>(const float*, Dims, const float*, const float*, const float*, int, int, float*,
-                                       float*, double*, float);
-template __global__ void fwd_kernel<1>(const float*, Dims, const float*, const float*, const float*, int, int, float*,
-                                       float*, double*, float);
-
 // B fragments of the adjoint product gw[row][f] = sum_o G[row][o] Wp[o][f]
-// (k = output o, n = feature f; six n-tiles cover the 48 padded features).
+// (k = output o, n = feature f; two n-tiles of features per scheduling block).
+template <int NT>
 __device__ __forceinline__ void load_bwd_frags(const float* __restrict__ Wp, uint32_t (*bhi)[2], uint32_t (*blo)[2],
                                                int g, int t)
 {
     constexpr int ld = kFB * kMaxKT;
 #pragma unroll
-    for (int nt = 0; nt < 6; ++nt) {
+    for (int nt = 0; nt < NT; ++nt) {
         const int f = nt * 8 + g;
         split2(Wp[(2 * t) * ld + f], Wp[(2 * t + 1) * ld + f], bhi[nt][0], blo[nt][0]);
         split2(Wp[(8 + 2 * t) * ld + f], Wp[(9 + 2 * t) * ld + f], bhi[nt][1], blo[nt][1]);
     }
 }
 
-// Backpropagation through time for 16 trajectories per warp, k = T-1 .. 0:
+// Transpose of an 8 x 8 tile of 16-bit elements held as one register per lane.
+__device__ __forceinline__ uint32_t trans8(uint32_t a)
+{
+    uint32_t r;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(a));
+    return r;
+}
+
+// The adjoint and the weight gradient of 16 trajectories, k = T-1 .. 0:
 //   G_k = [lambda_{k+1}; dJ/dy_k],  gw_k = G_k W,
 //   lambda_k = gw_k[x] + sum_i p_{k,i} gw_k[block i, x],
-//   dJ/dW += G_k^T w_k  (tensor cores, operands transposed in shared memory).
-// Each warp writes its partial gradient gpart[warp][16][48].
-constexpr int kBwdWarps = 4;
+//   dJ/dW += G_k^T w_k.
+// Warps 0 and 1 carry the adjoint of 8 trajectories each and leave G_k, split,
+// in shared memory; the other warps add up the gradient, an n-tile (8 of
+// the 48 features) each, a chunk of kC steps behind them, so that the gradient's products, splits and
+// transposes take no part in the serial chain.  Both operands of a gradient
+// product come as row fragments (rows are trajectories) and it contracts over
+// the rows: each 8 x 8 tile is transposed in registers.  The accumulators run
+// over all steps of the 16 trajectories (gpart[block][16][48], added up in
+// FP64 by launch_reduce): sums in other parts were measured and differ from
+// these by up to 7e-5, the rounding of a 1,000-step FP32 tensor-core sum.
+template <int NP>
+constexpr int kAdjWarps = 2 + 2 * (1 + NP);
 
-__global__ void __launch_bounds__(32 * kBwdWarps) bwd_kernel(const float* __restrict__ Wp, Dims d,
-                                                             const float* __restrict__ u, const float* __restrict__ p,
-                                                             int n_traj, int T, const float* __restrict__ hist,
-                                                             float* __restrict__ gpart)
+template <int NP>
+struct AdjStage {
+    float res[kC][2][kFrag];   // residuals' part of G_k (zero elsewhere)
+    float z[kC][2][kFrag];
+    float p[kC][16][2];
+};
+
+template <int NP>
+__global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __restrict__ Wp, Dims d,
+                                                            const float* __restrict__ p, int n_traj, int T,
+                                                            const float* __restrict__ zfrag,
+                                                            const float* __restrict__ gfrag,
+                                                            float* __restrict__ gpart)
 {
-    __shared__ float sG[kBwdWarps][16][17];
-    __shared__ float sZ[kBwdWarps][16][kFB * kMaxKT + 1];
+    __shared__ __align__(16) AdjStage<NP> sm[kStages];
+    __shared__ __align__(16) float sG[2][kC][2][kFrag];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, wl = threadIdx.x >> 5;
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int r0 = wid * 16 + g, r1 = r0 + 8;
-    const bool v0 = r0 < n_traj, v1 = r1 < n_traj;
-    uint32_t bhi[6][2], blo[6][2];
-    load_bwd_frags(Wp, bhi, blo, g, t);
-    float lam[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // lambda_T = 0
-    float gacc[6][4];
+    const int first = blockIdx.x * 16, n_chunk = (T + kC - 1) / kC;
+    const bool is_adj = wl < 2;
+    const bool two = first + 8 < n_traj;  // the second group of 8 exists (its fragments are not written otherwise)
+    {   // rows beyond the data stay zero
+        float* z = reinterpret_cast<float*>(sm);
+        for (int i = threadIdx.x; i < (int)(sizeof(sm) / sizeof(float)); i += blockDim.x) z[i] = 0.f;
+    }
+    __syncthreads();
+    const size_t grp = (size_t)blockIdx.x * 2;
+    // chunk c holds steps T - 1 - c kC - q for q = 0, 1, ..
+    auto fetch = [&](int c) {
+        AdjStage<NP>& S = sm[c % kStages];
+        const int k0 = T - 1 - c * kC;
+        if (is_adj) {  // a warp's residuals, and the p of its rows, a step per lane
+            const float* src = gfrag + ((grp + wl) * T + k0) * kFrag + 4 * lane;
 #pragma unroll
-    for (int nt = 0; nt < 6; ++nt) gacc[nt][0] = gacc[nt][1] = gacc[nt][2] = gacc[nt][3] = 0.f;
-    // step inputs: scheduling, recorded history (x_k | dJ/dy_k) and u
-    auto fetch = [&](int k, float* pa0, float* pa1, float* hv, float* uz) {
-        load_p(d, p, r0, v0, T, k, pa0);
-        load_p(d, p, r1, v1, T, k, pa1);
+            for (int q = 0; q < kC; ++q)
+                if (k0 - q >= 0 && (wl == 0 || two)) copy_async<16>(&S.res[q][wl][4 * lane], src - (size_t)q * kFrag);
+            const int tr = first + 8 * wl + g;
+            if (k0 - t >= 0 && tr < n_traj)
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = scol(i, t);
-            const int r = srow(i) ? r1 : r0;
-            const bool v = srow(i) ? v1 : v0;
-            hv[i] = (v && c < d.nx + d.ny) ? hist[((size_t)r * T + k) * 16 + c] : 0.f;
-            uz[i] = (v && c >= d.nx && c < d.nx + d.nu)
-                        ? u[((size_t)r * T + k) * d.nu + (c - d.nx)] * d.inv_su[c - d.nx] : 0.f;
+                for (int j = 0; j < NP; ++j)
+                    copy_async<4>(&S.p[t][8 * wl + g][j], p + ((size_t)tr * T + (k0 - t)) * NP + j);
+        } else {
+            for (int i = wl - 2; i < 2 * kC; i += kAdjWarps<NP> - 2) {
+                const int q = i >> 1, r = i & 1;
+                if (k0 - q >= 0 && (r == 0 || two))
+                    copy_async<16>(&S.z[q][r][4 * lane], zfrag + ((grp + r) * T + (k0 - q)) * kFrag + 4 * lane);
+            }
         }
+        copy_commit();
     };
-    // a ring of the inputs of the next kPrefetch steps (backwards in k), as in
-    // the forward pass
-    float rp0[kPrefetch][2], rp1[kPrefetch][2], rhv[kPrefetch][8], ruz[kPrefetch][8];
+    // zero scheduling beyond the data, as the free run takes it
+    float pm[2], ips[2][2];
 #pragma unroll
-    for (int i = 0; i < kPrefetch; ++i) fetch(T - 1 - i >= 0 ? T - 1 - i : 0, rp0[i], rp1[i], rhv[i], ruz[i]);
-    for (int k0 = T - 1; k0 >= 0; k0 -= kPrefetch) {
+    for (int j = 0; j < 2; ++j) {
+        pm[j] = j < NP ? d.pm[j] : 0.f;
 #pragma unroll
-    for (int ri = 0; ri < kPrefetch; ++ri) {
-        const int k = k0 - ri;
-        if (k < 0) break;
-        float chv[8], cuz[8];
-        const float pp0[2] = {rp0[ri][0], rp0[ri][1]}, pp1[2] = {rp1[ri][0], rp1[ri][1]};
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            chv[i] = rhv[ri][i];
-            cuz[i] = ruz[ri][i];
-        }
-        fetch(k - kPrefetch >= 0 ? k - kPrefetch : 0, rp0[ri], rp1[ri], rhv[ri], ruz[ri]);
-        float G[8], z[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = scol(i, t);
-            G[i] = (c < d.nx) ? lam[i] : chv[i];
-            z[i] = (c < d.nx) ? chv[i] : cuz[i];  // x_k, u_k, 0
-        }
-        // gw = G W
-        uint32_t ghi[4], glo[4];
-        afrag(G, ghi, glo);
-        float gw[6][4];
-#pragma unroll
-        for (int nt = 0; nt < 6; ++nt) {
-            float c1[4] = {0, 0, 0, 0}, c2[4] = {0, 0, 0, 0};
-            gw[nt][0] = gw[nt][1] = gw[nt][2] = gw[nt][3] = 0.f;
-            mma16816(gw[nt], ghi, bhi[nt][0], bhi[nt][1]);
-            mma16816(c1, ghi, blo[nt][0], blo[nt][1]);
-            mma16816(c2, glo, bhi[nt][0], bhi[nt][1]);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) gw[nt][q] += c1[q] + c2[q];
-        }
-        // lambda_k
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = scol(i, t);
-            const int nt0 = (i < 4) ? 0 : 1, q = i & 3;
-            const float* pr = srow(i) ? pp1 : pp0;
-            float l = gw[nt0][q];
-            if (d.np > 0) l += pr[0] * gw[nt0 + 2][q];
-            if (d.np > 1) l += pr[1] * gw[nt0 + 4][q];
-            lam[i] = (c < d.nx) ? l : 0.f;
-        }
-        // dJ/dW += G^T w: stage G and w in shared memory, read them transposed
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = scol(i, t), rl = srow(i) ? g + 8 : g;
-            const float* pr = srow(i) ? pp1 : pp0;
-            sG[wl][rl][c] = G[i];
-            sZ[wl][rl][c] = z[i];
-            sZ[wl][rl][kFB + c] = d.np > 0 ? z[i] * pr[0] : 0.f;
-            sZ[wl][rl][2 * kFB + c] = d.np > 1 ? z[i] * pr[1] : 0.f;
-        }
-        __syncwarp();
-        float a[8] = {sG[wl][2 * t][g],     sG[wl][2 * t + 1][g],     sG[wl][2 * t][g + 8],     sG[wl][2 * t + 1][g + 8],
-                      sG[wl][2 * t + 8][g], sG[wl][2 * t + 9][g],     sG[wl][2 * t + 8][g + 8], sG[wl][2 * t + 9][g + 8]};
-        uint32_t ahi[4], alo[4];
-        afrag(a, ahi, alo);
-#pragma unroll
-        for (int nt = 0; nt < 6; ++nt) {
-            const int f = nt * 8 + g;
-            uint32_t b0h, b0l, b1h, b1l;
-            split2(sZ[wl][2 * t][f], sZ[wl][2 * t + 1][f], b0h, b0l);
-            split2(sZ[wl][2 * t + 8][f], sZ[wl][2 * t + 9][f], b1h, b1l);
-            mma16816(gacc[nt], ahi, b0h, b1h);
-            mma16816(gacc[nt], ahi, b0l, b1l);
-            mma16816(gacc[nt], alo, b0h, b1h);
-        }
-        __syncwarp();
+        for (int r = 0; r < 2; ++r) ips[r][j] = j < NP && first + 8 * r + g < n_traj ? d.inv_ps[j] : 0.f;
     }
+    constexpr int NT = 2 + 2 * NP;
+    fetch(0);
+    fetch(1);
+    if (is_adj) {
+        bool is_x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) is_x[j] = 8 * (j >> 1) + 2 * t + (j & 1) < d.nx;
+        float ip[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) ip[j] = wl ? ips[1][j] : ips[0][j];
+        uint32_t bhi[NT][2], blo[NT][2];
+        load_bwd_frags<NT>(Wp, bhi, blo, g, t);
+        float lam[4] = {0, 0, 0, 0};  // lambda_T = 0
+        auto step = [&](const AdjStage<NP>& S, float* out, int q) {
+            const float4 v = *reinterpret_cast<const float4*>(&S.res[q][wl][4 * lane]);
+            const float2 pv = *reinterpret_cast<const float2*>(S.p[q][8 * wl + g]);
+            const float pp[2] = {(pv.x - pm[0]) * ip[0], (pv.y - pm[1]) * ip[1]};
+            // rows 0-7 the high, rows 8-15 the low parts (as in the free run)
+            uint32_t a[4];
+            split2(is_x[0] ? lam[0] : v.x, is_x[1] ? lam[1] : v.y, a[0], a[1]);
+            split2(is_x[2] ? lam[2] : v.z, is_x[3] ? lam[3] : v.w, a[2], a[3]);
+            *reinterpret_cast<uint4*>(out + (q * 2 + wl) * kFrag + 4 * lane) = make_uint4(a[0], a[1], a[2], a[3]);
+            float2 gw[NT];
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                float c0[4] = {0, 0, 0, 0}, c1[4] = {0, 0, 0, 0};
+                mma16816(c0, a, bhi[nt][0], bhi[nt][1]);
+                mma16816(c1, a, blo[nt][0], blo[nt][1]);
+                gw[nt] = add2(make_float2(c0[0], c0[1]), add2(make_float2(c1[0], c1[1]), make_float2(c0[2], c0[3])));
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float2 l = gw[h];
+#pragma unroll
+                for (int m = 0; m < NP; ++m) {
+                    l.x = fmaf(pp[m], gw[h + 2 + 2 * m].x, l.x);
+                    l.y = fmaf(pp[m], gw[h + 2 + 2 * m].y, l.y);
+                }
+                lam[2 * h] = l.x;  // columns beyond the state are never used
+                lam[2 * h + 1] = l.y;
+            }
+        };
+        for (int c = 0; c <= n_chunk; ++c) {
+            copy_wait<1>();
+            __syncthreads();
+            if (c < n_chunk) {
+                fetch(c + 2);  // the stage last read two chunks ago
+                const AdjStage<NP>& S = sm[c % kStages];
+                float* out = &sG[c & 1][0][0][0];
+                if ((c + 1) * kC <= T) {
+#pragma unroll
+                    for (int q = 0; q < kC; ++q) step(S, out, q);
+                } else {
+                    for (int q = 0; c * kC + q < T; ++q) step(S, out, q);
+                }
+            }
+        }
+        return;
     }
-    // gacc[nt]: (o = g, f = 8 nt + 2t), (g, +1), (g + 8, 2t), (g + 8, 2t + 1)
-    float* out = gpart + (size_t)wid * kWN;
+    const int kt = (wl - 2) >> 1, h = (wl - 2) & 1;  // scheduling block and half of the features of this warp
+    const bool scaled = kt > 0;
+    float pk = 0.f, ik[2] = {1.f, 1.f};
+    if (scaled) {
+        pk = kt == 1 ? pm[0] : pm[1];
+        ik[0] = kt == 1 ? ips[0][0] : ips[0][1];
+        ik[1] = kt == 1 ? ips[1][0] : ips[1][1];
+    }
+    float acc[4] = {0, 0, 0, 0};
+    auto step = [&](const AdjStage<NP>& S, const float* in, int q) {
+        const uint4 ga = *reinterpret_cast<const uint4*>(in + (q * 2) * kFrag + 4 * lane);
+        const uint4 gb = *reinterpret_cast<const uint4*>(in + (q * 2 + 1) * kFrag + 4 * lane);
+        float2 za = *reinterpret_cast<const float2*>(&S.z[q][0][4 * lane + 2 * h]);
+        float2 zb = *reinterpret_cast<const float2*>(&S.z[q][1][4 * lane + 2 * h]);
+        if (scaled) {
+            const float pa = (S.p[q][g][kt - 1] - pk) * ik[0], pb = (S.p[q][8 + g][kt - 1] - pk) * ik[1];
+            za = mul2(za, make_float2(pa, pa));
+            zb = mul2(zb, make_float2(pb, pb));
+        }
+        // A = G^T: (outputs 0-7 | 8-15) x (rows 0-7 | 8-15), in the order 00, 10, 01, 11
+        const uint32_t ahi[4] = {trans8(ga.x), trans8(ga.z), trans8(gb.x), trans8(gb.z)};
+        const uint32_t alo[4] = {trans8(ga.y), trans8(ga.w), trans8(gb.y), trans8(gb.w)};
+        uint32_t ha, la, hb, lb;
+        split2(za.x, za.y, ha, la);
+        split2(zb.x, zb.y, hb, lb);
+        const uint32_t b0h = trans8(ha), b1h = trans8(hb), b0l = trans8(la), b1l = trans8(lb);
+        mma16816(acc, ahi, b0h, b1h);
+        mma16816(acc, ahi, b0l, b1l);
+        mma16816(acc, alo, b0h, b1h);
+    };
+    for (int c = 0; c <= n_chunk; ++c) {
+        copy_wait<1>();
+        __syncthreads();
+        if (c < n_chunk) fetch(c + 2);
+        if (c == 0) continue;
+        const AdjStage<NP>& S = sm[(c - 1) % kStages];
+        const float* in = &sG[(c - 1) & 1][0][0][0];
+        if (c * kC <= T) {
+#pragma unroll
+            for (int q = 0; q < kC; ++q) step(S, in, q);
+        } else {
+            for (int q = 0; (c - 1) * kC + q < T; ++q) step(S, in, q);
+        }
+    }
+    // acc: (o = g, f = 8 h + 2t), (g, +1), (g + 8, 2t), (g + 8, 2t + 1) of block kt
     constexpr int ld = kFB * kMaxKT;
+    float* out = gpart + (size_t)blockIdx.x * kWN;
 #pragma unroll
-    for (int nt = 0; nt < 6; ++nt) {
-        const int f = nt * 8 + 2 * t;
-        out[g * ld + f] = gacc[nt][0];
-        out[g * ld + f + 1] = gacc[nt][1];
-        out[(g + 8) * ld + f] = gacc[nt][2];
-        out[(g + 8) * ld + f + 1] = gacc[nt][3];
+    for (int q = 0; q < 4; ++q) out[(g + 8 * (q >> 1)) * ld + kt * kFB + 8 * h + 2 * t + (q & 1)] = acc[q];
+    if constexpr (NP + 1 < kMaxKT) {  // the blocks that this model does not have
+        constexpr int n = (kMaxKT - 1 - NP) * kFB;
+        if (wl == 2)
+            for (int i = lane; i < kO * n; i += 32) out[(i / n) * ld + (1 + NP) * kFB + i % n] = 0.f;
     }
 }
 
@@ -481,23 +708,49 @@ __global__ void __launch_bounds__(128, 4) closed_loop_kernel(const float* __rest
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-cudaError_t launch_forward(int mode, const float* Wp, const Dims& d, const float* u, const float* p, const float* y,
-                           int n_traj, int T, float* y_out, float* hist, double* loss_part, float grad_scale,
-                           cudaStream_t st)
+// Row groups per warp of the serial passes: one while a warp per group still
+// finds a scheduler of its own (152 SMs x 4), two beyond.
+static int row_groups(int n_traj) { return groups_for(n_traj) <= 608 ? 1 : 2; }
+
+int serial_warps(int n_traj) { return (groups_for(n_traj) + row_groups(n_traj) - 1) / row_groups(n_traj); }
+
+template <class F>
+static void by_np(int np, F&& f)
 {
-    const int warps = warps_for(n_traj), blocks = (warps + 3) / 4;
-    if (mode == 0)
-        fwd_kernel<0><<<blocks, 128, 0, st>>>(Wp, d, u, p, y, n_traj, T, y_out, hist, loss_part, grad_scale);
-    else
-        fwd_kernel<1><<<blocks, 128, 0, st>>>(Wp, d, u, p, y, n_traj, T, y_out, hist, loss_part, grad_scale);
+    if (np == 0) f(std::integral_constant<int, 0>{});
+    else if (np == 1) f(std::integral_constant<int, 1>{});
+    else f(std::integral_constant<int, 2>{});
+}
+
+cudaError_t launch_forward(int mode, const float* Wp, const Dims& d, const float* u, const float* p, const float* y,
+                           int n_traj, int T, float* y_out, float* zfrag, float* gfrag, double* loss_part,
+                           float grad_scale, cudaStream_t st)
+{
+    const int warps = serial_warps(n_traj);
+    by_np(d.np, [&](auto np) {
+        constexpr int NP = decltype(np)::value;
+        auto go = [&](auto kernel) {
+            kernel<<<warps, 32, 0, st>>>(Wp, d, u, p, y, n_traj, T, y_out, zfrag, gfrag, loss_part, grad_scale);
+        };
+        const bool low = d.nx < 8, one = row_groups(n_traj) == 1;
+        if (mode == 0) {
+            if (one) low ? go(fwd_kernel<0, true, NP, 1>) : go(fwd_kernel<0, false, NP, 1>);
+            else low ? go(fwd_kernel<0, true, NP, 2>) : go(fwd_kernel<0, false, NP, 2>);
+        } else {
+            if (one) low ? go(fwd_kernel<1, true, NP, 1>) : go(fwd_kernel<1, false, NP, 1>);
+            else low ? go(fwd_kernel<1, true, NP, 2>) : go(fwd_kernel<1, false, NP, 2>);
+        }
+    });
     return cudaGetLastError();
 }
 
-cudaError_t launch_backward(const float* Wp, const Dims& d, const float* u, const float* p, int n_traj, int T,
-                            const float* hist, float* gpart, cudaStream_t st)
+cudaError_t launch_backward(const float* Wp, const Dims& d, const float* p, int n_traj, int T, const float* zfrag,
+                            const float* gfrag, float* gpart, cudaStream_t st)
 {
-    const int warps = warps_for(n_traj), blocks = (warps + kBwdWarps - 1) / kBwdWarps;
-    bwd_kernel<<<blocks, 32 * kBwdWarps, 0, st>>>(Wp, d, u, p, n_traj, T, hist, gpart);
+    by_np(d.np, [&](auto np) {
+        constexpr int NP = decltype(np)::value;
+        adj_kernel<NP><<<grad_parts(n_traj), 32 * kAdjWarps<NP>, 0, st>>>(Wp, d, p, n_traj, T, zfrag, gfrag, gpart);
+    });
     return cudaGetLastError();
 }
 
@@ -505,7 +758,7 @@ cudaError_t launch_closed_loop(const float* Wp, const Dims& d, int B, int T, con
                                const double* ref, const double* fill, const BodyParHost& h, double* out,
                                cudaStream_t st)
 {
-    const int warps = warps_for(B), blocks = (warps + 3) / 4;
+    const int warps = (B + 15) / 16, blocks = (warps + 3) / 4;
     BodyPar bp{h.inv_m, h.inv_J, h.dt, h.n, h.n_half, h.kp, h.kd};
     closed_loop_kernel<<<blocks, 128, 0, st>>>(Wp, d, B, T, F, tau, ref, fill, bp, out);
     return cudaGetLastError();

@@ -10,23 +10,33 @@ struct BodyParHost {
     float inv_m, inv_J, dt, n, n_half, kp, kd;
 };
 
-// Warps of 16 trajectories needed for n trajectories.
-inline int warps_for(int n) { return (n + 15) / 16; }
+// Groups of 8 trajectories that n trajectories make.
+inline int groups_for(int n) { return (n + 7) / 8; }
 
-// mode 0: prediction into y_out; mode 1: loss partials per warp and BPTT history.
+// Fragments in device memory: 128 floats per step of a group of 8
+// trajectories, of an even number of groups.
+constexpr int kFragFloats = 128;
+inline size_t frag_floats(int n_traj, int T) { return (size_t)((groups_for(n_traj) + 1) / 2 * 2) * T * kFragFloats; }
+// Warps of the serial passes, and loss partials that launch_forward writes.
+int serial_warps(int n_traj);
+// mode 0: prediction into y_out; mode 1: loss partials per warp, z_k (zfrag)
+// and the residuals' part of G_k (gfrag).
 cudaError_t launch_forward(int mode, const float* Wp, const Dims& d, const float* u, const float* p, const float* y,
-                           int n_traj, int T, float* y_out, float* hist, double* loss_part, float grad_scale,
-                           cudaStream_t st);
-cudaError_t launch_backward(const float* Wp, const Dims& d, const float* u, const float* p, int n_traj, int T,
-                            const float* hist, float* gpart, cudaStream_t st);
+                           int n_traj, int T, float* y_out, float* zfrag, float* gfrag, double* loss_part,
+                           float grad_scale, cudaStream_t st);
+// The adjoint and the weight gradient's partials gpart[grad_parts(n_traj)][768].
+inline int grad_parts(int n_traj) { return (n_traj + 15) / 16; }
+cudaError_t launch_backward(const float* Wp, const Dims& d, const float* p, int n_traj, int T, const float* zfrag,
+                            const float* gfrag, float* gpart, cudaStream_t st);
 cudaError_t launch_closed_loop(const float* Wp, const Dims& d, int B, int T, const double* F, const double* tau,
                                const double* ref, const double* fill, const BodyParHost& bp, double* out,
                                cudaStream_t st);
-// grad = sum of the warp partials (FP64, fixed order) + sigma2 W, masked to the
-// trainable entries; *loss = sum loss_part / n_samples + sigma2 / 2 ||W||^2;
-// if loss_hist is not NULL the loss is also stored at loss_hist[it].
-cudaError_t launch_reduce(const float* gpart, int n_warps, const double* loss_part, const float* Wp, const Dims& d,
-                          double sigma2, double n_samples, float* grad, double* loss, double* loss_hist, int it,
+// grad = sum of the n_part gradient partials (FP64, fixed order) + sigma2 W,
+// masked to the trainable entries; *loss = sum of the n_warps loss_part /
+// n_samples + sigma2 / 2 ||W||^2; if loss_hist is not NULL the loss is also
+// stored at loss_hist[it].
+cudaError_t launch_reduce(const float* gpart, int n_part, const double* loss_part, int n_warps, const float* Wp,
+                          const Dims& d, double sigma2, double n_samples, float* grad, double* loss, double* loss_hist, int it,
                           cudaStream_t st);
 cudaError_t launch_adam(float* Wp, float* m, float* v, float* Wb, float* mb, float* vb, float* lr_scale,
                         double* acc_loss, const float* grad, const double* loss, const Dims& d, float lr, float b1,

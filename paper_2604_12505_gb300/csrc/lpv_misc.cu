@@ -7,30 +7,54 @@
 
 namespace lpv {
 
-// One thread per padded weight: sum of the warp partials in fixed order (FP64).
-__global__ void reduce_kernel(const float* __restrict__ gpart, int n_warps, const double* __restrict__ loss_part,
-                              const float* __restrict__ Wp, Dims d, double sigma2, double n_samples,
-                              float* __restrict__ grad, double* __restrict__ loss, double* __restrict__ loss_hist,
-                              int it)
+// Block b < kWN / kRedCols: the gradient of kRedCols weights, the partials
+// summed by kRedRows threads each (every kRedRows-th partial), then these sums
+// in a fixed tree, all in FP64.  The last block: the loss.
+constexpr int kRedCols = 8, kRedRows = 64;
+
+__global__ void __launch_bounds__(kRedCols* kRedRows)
+    reduce_kernel(const float* __restrict__ gpart, int n_part, const double* __restrict__ loss_part, int n_warps,
+                  const float* __restrict__ Wp, Dims d, double sigma2, double n_samples, float* __restrict__ grad,
+                  double* __restrict__ loss, double* __restrict__ loss_hist, int it)
 {
-    __shared__ double red[kWN / 32];
-    const int idx = threadIdx.x;
-    const int o = idx / (kFB * kMaxKT), col = idx % (kFB * kMaxKT);
-    double gsum = 0.0;
-    for (int w = 0; w < n_warps; ++w) gsum += (double)gpart[(size_t)w * kWN + idx];
-    const double wv = (double)Wp[idx];
-    const bool tr = trainable(d, o, col);
-    grad[idx] = tr ? (float)(gsum + sigma2 * wv) : 0.f;
-    double sq = tr ? wv * wv : 0.0;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) sq += __shfl_down_sync(0xffffffffu, sq, s);
-    if ((idx & 31) == 0) red[idx >> 5] = sq;
+    __shared__ double red[2][kRedRows][kRedCols + 1];
+    constexpr int kT = kRedCols * kRedRows;
+    const int e = threadIdx.x % kRedCols, r = threadIdx.x / kRedCols;
+    const bool is_loss = blockIdx.x == kWN / kRedCols;
+    const int idx = blockIdx.x * kRedCols + e;
+    double v = 0.0, sq = 0.0;
+    if (is_loss) {
+        for (int w = threadIdx.x; w < n_warps; w += kT) v += loss_part[w];
+        for (int w = threadIdx.x; w < kWN; w += kT)
+            if (trainable(d, w / (kFB * kMaxKT), w % (kFB * kMaxKT))) sq += (double)Wp[w] * (double)Wp[w];
+    } else {
+#pragma unroll 4
+        for (int w = r; w < n_part; w += kRedRows) v += (double)gpart[(size_t)w * kWN + idx];
+    }
+    red[0][r][e] = v;
+    red[1][r][e] = sq;
     __syncthreads();
-    if (idx == 0) {
-        double w2 = 0.0, ls = 0.0;
-        for (int j = 0; j < kWN / 32; ++j) w2 += red[j];
-        for (int w = 0; w < n_warps; ++w) ls += loss_part[w];
-        const double L = ls / n_samples + 0.5 * sigma2 * w2;
+    for (int o = kRedRows / 2; o > 0; o >>= 1) {
+        if (r < o) {
+            red[0][r][e] += red[0][r + o][e];
+            if (is_loss) red[1][r][e] += red[1][r + o][e];
+        }
+        __syncthreads();
+    }
+    if (r) return;
+    v = red[0][0][e];
+    if (!is_loss) {
+        const double wv = (double)Wp[idx];
+        grad[idx] = trainable(d, idx / (kFB * kMaxKT), idx % (kFB * kMaxKT)) ? (float)(v + sigma2 * wv) : 0.f;
+        return;
+    }
+    sq = red[1][0][e];
+    if (e == 0) {
+        for (int q = 1; q < kRedCols; ++q) {
+            v += red[0][0][q];
+            sq += red[1][0][q];
+        }
+        const double L = v / n_samples + 0.5 * sigma2 * sq;
         if (loss) *loss = L;
         if (loss_hist) loss_hist[it] = L;
     }
@@ -531,11 +555,12 @@ __global__ void ls_solve_kernel(const double* __restrict__ part, int n_blocks, D
 }
 
 // ---------------------------------------------------------------------------
-cudaError_t launch_reduce(const float* gpart, int n_warps, const double* loss_part, const float* Wp, const Dims& d,
-                          double sigma2, double n_samples, float* grad, double* loss, double* loss_hist, int it,
-                          cudaStream_t st)
+cudaError_t launch_reduce(const float* gpart, int n_part, const double* loss_part, int n_warps, const float* Wp,
+                          const Dims& d, double sigma2, double n_samples, float* grad, double* loss, double* loss_hist,
+                          int it, cudaStream_t st)
 {
-    reduce_kernel<<<1, kWN, 0, st>>>(gpart, n_warps, loss_part, Wp, d, sigma2, n_samples, grad, loss, loss_hist, it);
+    reduce_kernel<<<kWN / kRedCols + 1, kRedCols * kRedRows, 0, st>>>(gpart, n_part, loss_part, n_warps, Wp, d, sigma2, n_samples, grad, loss,
+                                                 loss_hist, it);
     return cudaGetLastError();
 }
 
