@@ -1,6 +1,6 @@
 // lpv_kernels.cu -- tensor-core kernels of the LPV surrogate (Section 4).
 //
-// One warp carries 16 trajectories through the recurrence
+// One warp carries 16 (or 8) trajectories through the recurrence
 //     [x_{k+1}; y_k] = W w_k,   w_k = [z_k; p_1 z_k; p_2 z_k],  z_k = [x_k; u_k; 0]
 // as one mma.sync.m16n8k16 (BF16 in, FP32 accumulate) product per 16x16x8
 // tile.  Each operand is split into two BF16 halves (v = hi + lo) and the
@@ -15,8 +15,8 @@
 // 0 and 1 holds exactly the entries of the next step's first A block that
 // this thread owns, and the scheduled blocks p_i z are thread-local scalings:
 // the recurrence runs without shuffles.  The adjoint uses the same identity;
-// the weight gradient sum_k G_k^T w_k is one more MMA, over all steps in
-// parallel, whose operands are transposed in registers.
+// the weight gradient sum_k G_k^T w_k is one more MMA, in
+// warps of its own, whose operands are transposed in registers.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -36,6 +36,15 @@ __device__ __forceinline__ void mma16816(float* d, const uint32_t* a, uint32_t b
         "{%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// The same with a zero accumulator.
+__device__ __forceinline__ void mma16816_0(float* d, const uint32_t* a, uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 
 // Two FP32 operations in one instruction, each rounded to nearest.
@@ -79,44 +88,6 @@ __device__ __forceinline__ void split2(float v0, float v1, uint32_t& hi, uint32_
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// A fragment from the 8 values s[] a thread owns (see layout above).
-__device__ __forceinline__ void afrag(const float* s, uint32_t* hi, uint32_t* lo)
-{
-    split2(s[0], s[1], hi[0], lo[0]);
-    split2(s[2], s[3], hi[1], lo[1]);
-    split2(s[4], s[5], hi[2], lo[2]);
-    split2(s[6], s[7], hi[3], lo[3]);
-}
-
-// Column and row (0: g, 1: g + 8) of the thread's value s[i].
-__device__ __forceinline__ int scol(int i, int t) { return ((i < 4) ? 2 * t : 8 + 2 * t) + (i & 1); }
-__device__ __forceinline__ int srow(int i) { return (i >> 1) & 1; }
-
-// d[8] += A[kt] B for the split operands: three independent accumulation
-// chains (hi.hi, hi.lo, lo.hi) over the k-tiles, summed at the end.
-template <int NKT>
-__device__ __forceinline__ void mma_split(float* d, const uint32_t (*ahi)[4], const uint32_t (*alo)[4],
-                                          const uint32_t (*bhi)[2][2], const uint32_t (*blo)[2][2], int nkt)
-{
-    float c1[8] = {0, 0, 0, 0, 0, 0, 0, 0}, c2[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int kt = 0; kt < NKT; ++kt) {
-        if (kt >= nkt) break;
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-            mma16816(d + 4 * nt, ahi[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
-            mma16816(c1 + 4 * nt, ahi[kt], blo[kt][nt][0], blo[kt][nt][1]);
-            mma16816(c2 + 4 * nt, alo[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) d[i] += c1[i] + c2[i];
-}
-
-}  // namespace lpv
-
-namespace lpv {
-
 // B fragments of the forward product D[row][o] = sum_f w[row][f] Wp[o][f].
 __device__ __forceinline__ void load_fwd_frags(const float* __restrict__ Wp, uint32_t (*bhi)[2][2],
                                                uint32_t (*blo)[2][2], int nkt, int g, int t)
@@ -157,7 +128,7 @@ __device__ __forceinline__ void load_fwd_frags(const float* __restrict__ Wp, uin
 // warps to a block that loaded u, y and p from their rows (28 memory
 // instructions of up to 16 lines a step) and kept the weight gradient, with
 // its transposes through shared memory, on the adjoint's chain took 1,939 +
-// 1,469 + 31 us.  With RG = 2 there the forward pass takes 650 us.
+// 1,469 + 31 us.
 //
 // Fragments in global memory: per group of 8 trajectories and step, [lane][4],
 // the values of columns 2t, 2t+1, 2t+8, 2t+9 of row g.
@@ -210,6 +181,82 @@ __device__ __forceinline__ void copy_row(float* dst, const float* src, int n)
 {
 #pragma unroll 4
     for (int j = 0; j < n; ++j) copy_async<4>(dst + j, src + j);
+}
+
+// D = [z; p_1 z; ...] W^T for RG row groups: z[i] of column i, row group
+// (i >> 1) & 1, and the normalised scheduling pp of each row.
+template <int NP, int RG>
+__device__ __forceinline__ void product(float* D, const float* z, const float (*pp)[2], const uint32_t (*bhi)[2][2],
+                                        const uint32_t (*blo)[2][2])
+{
+    if constexpr (RG == 1) {
+        // the idle rows 8-15 take the low parts: one product gives hi.hi and
+        // lo.hi, the other hi.lo (and lo.lo, not used)
+        uint32_t a[1 + NP][4];
+        float c1[8];
+#pragma unroll
+        for (int kt = 0; kt <= NP; ++kt) {
+            float2 v0 = make_float2(z[0], z[1]), v1 = make_float2(z[4], z[5]);
+            if (kt) {
+                const float2 f = make_float2(pp[0][kt ? kt - 1 : 0], pp[0][kt ? kt - 1 : 0]);
+                v0 = mul2(v0, f);
+                v1 = mul2(v1, f);
+            }
+            split2(v0.x, v0.y, a[kt][0], a[kt][1]);
+            split2(v1.x, v1.y, a[kt][2], a[kt][3]);
+        }
+#pragma unroll
+        for (int kt = 0; kt <= NP; ++kt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                auto mma = [kt](float* c, const uint32_t* x, uint32_t b0, uint32_t b1) {
+                    if (kt) mma16816(c, x, b0, b1);
+                    else mma16816_0(c, x, b0, b1);
+                };
+                mma(D + 4 * nt, a[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
+                mma(c1 + 4 * nt, a[kt], blo[kt][nt][0], blo[kt][nt][1]);
+            }
+#pragma unroll
+        for (int nt = 0; nt < 2; ++nt) {
+            const float2 e = add2(make_float2(c1[4 * nt], c1[4 * nt + 1]), make_float2(D[4 * nt + 2], D[4 * nt + 3]));
+            const float2 f = add2(make_float2(D[4 * nt], D[4 * nt + 1]), e);
+            D[4 * nt] = f.x;
+            D[4 * nt + 1] = f.y;
+        }
+    } else {
+        // three independent accumulation chains (hi.hi, hi.lo, lo.hi) over the k-tiles
+        uint32_t ahi[1 + NP][4], alo[1 + NP][4];
+#pragma unroll
+        for (int kt = 0; kt <= NP; ++kt)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float2 v = make_float2(z[2 * i], z[2 * i + 1]);
+                if (kt) {
+                    const float f = pp[i & 1][kt ? kt - 1 : 0];
+                    v = mul2(v, make_float2(f, f));
+                }
+                split2(v.x, v.y, ahi[kt][i], alo[kt][i]);
+            }
+        float c1[8], c2[8];
+#pragma unroll
+        for (int kt = 0; kt <= NP; ++kt)
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                auto mma = [kt](float* c, const uint32_t* x, uint32_t b0, uint32_t b1) {
+                    if (kt) mma16816(c, x, b0, b1);
+                    else mma16816_0(c, x, b0, b1);
+                };
+                mma(D + 4 * nt, ahi[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
+                mma(c1 + 4 * nt, ahi[kt], blo[kt][nt][0], blo[kt][nt][1]);
+                mma(c2 + 4 * nt, alo[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
+            }
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            const float2 f = add2(make_float2(D[i], D[i + 1]), add2(make_float2(c1[i], c1[i + 1]), make_float2(c2[i], c2[i + 1])));
+            D[i] = f.x;
+            D[i + 1] = f.y;
+        }
+    }
 }
 
 // Free-run simulation of 8 RG trajectories per warp.  MODE 0 writes the
@@ -294,49 +341,8 @@ __global__ void __launch_bounds__(32) fwd_kernel(const float* __restrict__ Wp, D
             if (MODE == 1)
                 zo[((size_t)r * T + k) * 32] = make_float4(z[2 * r], z[2 * r + 1], z[4 + 2 * r], z[5 + 2 * r]);
         }
-        float D[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if constexpr (RG == 1) {
-            // the idle rows 8-15 take the low parts: one product gives hi.hi
-            // and lo.hi, the other hi.lo (and lo.lo, not used)
-            uint32_t a[1 + NP][4];
-            float c1[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int kt = 0; kt <= NP; ++kt) {
-                float2 v0 = make_float2(z[0], z[1]), v1 = make_float2(z[4], z[5]);
-                if (kt) {
-                    const float2 f = make_float2(pp[0][kt ? kt - 1 : 0], pp[0][kt ? kt - 1 : 0]);
-                    v0 = mul2(v0, f);
-                    v1 = mul2(v1, f);
-                }
-                split2(v0.x, v0.y, a[kt][0], a[kt][1]);
-                split2(v1.x, v1.y, a[kt][2], a[kt][3]);
-            }
-#pragma unroll
-            for (int kt = 0; kt <= NP; ++kt)
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    mma16816(D + 4 * nt, a[kt], bhi[kt][nt][0], bhi[kt][nt][1]);
-                    mma16816(c1 + 4 * nt, a[kt], blo[kt][nt][0], blo[kt][nt][1]);
-                }
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                const float2 e = add2(make_float2(c1[4 * nt], c1[4 * nt + 1]), make_float2(D[4 * nt + 2], D[4 * nt + 3]));
-                const float2 f = add2(make_float2(D[4 * nt], D[4 * nt + 1]), e);
-                D[4 * nt] = f.x;
-                D[4 * nt + 1] = f.y;
-            }
-        } else {
-            uint32_t ahi[kMaxKT][4], alo[kMaxKT][4];
-            afrag(z, ahi[0], alo[0]);
-#pragma unroll
-            for (int kt = 1; kt <= NP; ++kt) {
-                float zs[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) zs[i] = z[i] * pp[srow(i) < RG ? srow(i) : 0][kt - 1];
-                afrag(zs, ahi[kt], alo[kt]);
-            }
-            mma_split<1 + NP>(D, ahi, alo, bhi, blo, 1 + NP);
-        }
+        float D[8];
+        product<NP, RG>(D, z, pp, bhi, blo);
 #pragma unroll
         for (int r = 0; r < RG; ++r) {
             float yv[4], res[4] = {0.f, 0.f, 0.f, 0.f};
@@ -502,9 +508,9 @@ __global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __
             float2 gw[NT];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
-                float c0[4] = {0, 0, 0, 0}, c1[4] = {0, 0, 0, 0};
-                mma16816(c0, a, bhi[nt][0], bhi[nt][1]);
-                mma16816(c1, a, blo[nt][0], blo[nt][1]);
+                float c0[4], c1[4];
+                mma16816_0(c0, a, bhi[nt][0], bhi[nt][1]);
+                mma16816_0(c1, a, blo[nt][0], blo[nt][1]);
                 gw[nt] = add2(make_float2(c0[0], c0[1]), add2(make_float2(c1[0], c1[1]), make_float2(c0[2], c0[3])));
             }
 #pragma unroll
@@ -592,16 +598,33 @@ __global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __
     }
 }
 
-// Value D[i] of the lane owning output column c of row rsel (0: g, 1: g + 8).
-__device__ __forceinline__ float quad_get(const float* D, int c, int rsel, int g)
+// FP32 values of N doubles on the integer pipe.  A conversion instruction
+// takes 16 cycles of an SM's FP64 pipe whichever way it converts: with the
+// inputs converted once per row here, the outputs' conversions (one in four
+// lanes each) are all that this pipe is left with, 64 cycles per warp of 16
+// runs and period, beside as many issue slots.  Gives what the instruction
+// gives: to nearest (ties to even); zeros keep their sign; what is neither
+// zero nor a normal FP32 number is left to the instruction (a branch no warp
+// takes otherwise).
+template <int N>
+__device__ __forceinline__ void to_float(const double* x, float* r)
 {
-    const int tc = (c < 8) ? (c >> 1) : ((c - 8) >> 1);
-    const int ic = ((c < 8) ? 0 : 4) + (c & 1) + 2 * rsel;
-    float v = 0.f;
+    bool other[N], any = false;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (j == ic) v = D[j];
-    return __shfl_sync(0xffffffffu, v, g * 4 + tc);
+    for (int i = 0; i < N; ++i) {
+        const unsigned hi = (unsigned)__double2hiint(x[i]), lo = (unsigned)__double2loint(x[i]), m = hi & 0x7fffffffu;
+        const bool normal = m - 0x38100000u < 0x0fe00000u, zero = (m | lo) == 0u;
+        unsigned f = __funnelshift_l(lo, m - 0x38000000u, 3);
+        f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;
+        r[i] = __uint_as_float((normal ? f : 0u) | (hi & 0x80000000u));
+        other[i] = !normal && !zero;
+        any |= other[i];
+    }
+    if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            if (other[i]) r[i] = (float)x[i];
+    }
 }
 
 struct BodyPar {
@@ -610,98 +633,162 @@ struct BodyPar {
     float kp, kd;                // PD gains J w^2 and 2 xi J w
 };
 
-// Closed loop of 16 runs per warp (Sections 5.1.1, 5.4): per period the PD
+// Closed loop of 8 RG runs per warp (Sections 5.1.1, 5.4): per period the PD
 // torque (Eq. 28, zero-order hold), the surrogate step with p = [fill,
 // thetadot], and n_sub kick-then-drift substeps of the body under the held
 // forces, summed in closed form: v += n dt a, x += n dt v + dt^2 a n(n+1)/2.
-// The body state (FP32) is replicated in the four lanes of each row group.
-__global__ void __launch_bounds__(128, 4) closed_loop_kernel(const float* __restrict__ Wp, Dims d, int B, int T,
-                                                          const double* __restrict__ F, const double* __restrict__ tau,
-                                                          const double* __restrict__ ref,
-                                                          const double* __restrict__ fill, BodyPar bp,
-                                                          double* __restrict__ out)
+// The body state (FP32) is replicated in the four lanes of each row.  A chunk
+// of kC periods of the inputs passes through shared memory: the four lanes of
+// a row copy one period each, three chunks ahead, and convert it once for all
+// four.  65,536 runs of 500 periods (n_x 12, n_p 2): 2.60 -> 0.92 ms, 2.8 TB/s;
+// bound by the 297 instructions of a warp's period (50 % of the issue slots,
+// 44 % of the FP64 pipe for the outputs) at 14 to 16 warps per SM, and by the
+// period's chain for few runs.
+// wide: out is 16-byte aligned, so that three lanes store a row's sample.
+template <bool LOW, int NP, int RG>
+__global__ void __launch_bounds__(32, RG == 2 ? 16 : 1) closed_loop_kernel(const float* __restrict__ Wp, Dims d, int B, int T,
+                                                         const double* __restrict__ F, const double* __restrict__ tau,
+                                                         const double* __restrict__ ref,
+                                                         const double* __restrict__ fill, BodyPar bp,
+                                                         double* __restrict__ out, int wide)
 {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int rr[2] = {wid * 16 + g, wid * 16 + g + 8};
-    const bool vv[2] = {rr[0] < B, rr[1] < B};
+    __shared__ double raw[kStages][kC][RG][8][4];            // F_x, F_y, tau, theta_ref
+    __shared__ __align__(16) float4 in[kC][RG][8];
+    const int lane = threadIdx.x, g = lane >> 2, t = lane & 3, first = blockIdx.x * 8 * RG;
+    for (int i = lane; i < kStages * kC * RG * 32; i += 32) (&raw[0][0][0][0][0])[i] = 0.0;  // rows beyond B stay zero
+    __syncwarp();
     uint32_t bhi[kMaxKT][2][2], blo[kMaxKT][2][2];
-    load_fwd_frags(Wp, bhi, blo, d.nkt, g, t);
-    float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    float bs[2][6] = {{0, 0, 0, 0, 0, 0}, {0, 0, 0, 0, 0, 0}};  // r_x r_y theta v_x v_y omega
-    const float fl[2] = {vv[0] ? (float)fill[rr[0]] : 0.f, vv[1] ? (float)fill[rr[1]] : 0.f};
-    // inputs of a period (F_x, F_y, tau, theta_ref) for the two rows; those of
-    // period k + 1 are loaded while period k runs
-    auto fetch = [&](int k, float (*in)[4]) {
+    load_fwd_frags(Wp, bhi, blo, 1 + NP, g, t);
+    bool is_x[4];
+    float fu[4];
+    int uq[4];  // the input at a column, 3 where none lies
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const size_t o = (size_t)rr[q] * T + k;
-            in[q][0] = vv[q] ? (float)F[2 * o] : 0.f;
-            in[q][1] = vv[q] ? (float)F[2 * o + 1] : 0.f;
-            in[q][2] = vv[q] ? (float)tau[o] : 0.f;
-            in[q][3] = vv[q] ? (float)ref[o] : 0.f;
+    for (int j = 0; j < 4; ++j) {
+        const int q = 8 * (j >> 1) + 2 * t + (j & 1) - d.nx;
+        is_x[j] = q < 0;
+        uq[j] = q >= 0 && q < min(d.nu, 3) ? q : 3;
+        fu[j] = uq[j] < 3 ? d.inv_su[uq[j]] : 0.f;
+    }
+    // lane and register of the loads F_x, F_y, T_b: columns n_x, n_x + 1, n_x + 2 of D
+    int src[3];
+    bool up[3], odd[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const int c = d.nx + j;
+        src[j] = (lane & ~3) + ((c & 7) >> 1);
+        up[j] = c >= 8;
+        odd[j] = c & 1;
+    }
+    float pp[RG][2];
+    bool valid[RG];
+#pragma unroll
+    for (int r = 0; r < RG; ++r) {
+        const int run = first + 8 * r + g;
+        valid[r] = run < B;
+        // scheduling clamped to the range it was identified on
+        const float fl = valid[r] ? (float)fill[run] : 0.f;
+        pp[r][0] = NP > 0 ? (fminf(fmaxf(fl, d.plo[0]), d.phi[0]) - d.pm[0]) * d.inv_ps[0] : 0.f;
+        pp[r][1] = 0.f;
+    }
+    const int n_chunk = (T + kC - 1) / kC;
+    auto fetch = [&](int c) {
+        const int k = c * kC + t;
+        if (k < T) {
+#pragma unroll
+            for (int r = 0; r < RG; ++r)
+                if (valid[r]) {
+                    const size_t o = (size_t)(first + 8 * r + g) * T + k;
+                    double* dst = raw[c % kStages][t][r][g];
+                    copy_async<8>(dst, F + 2 * o);
+                    copy_async<8>(dst + 1, F + 2 * o + 1);
+                    copy_async<8>(dst + 2, tau + o);
+                    copy_async<8>(dst + 3, ref + o);
+                }
+        }
+        copy_commit();
+    };
+#pragma unroll
+    for (int c = 0; c < kStages - 1; ++c) fetch(c);
+    float s[RG][4] = {}, bs[RG][6] = {};  // surrogate state; r_x r_y theta v_x v_y omega
+    const float ndt = bp.n * bp.dt, hdt2 = bp.n_half * bp.dt * bp.dt;
+    double* o0 = out + (size_t)(first + g) * T * 6 + 2 * t;
+    auto step = [&](int q, int k) {
+        float z[8], uu[RG][3];
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (r >= RG) {
+                z[2 * r] = z[2 * r + 1] = z[4 + 2 * r] = z[5 + 2 * r] = 0.f;
+                continue;
+            }
+            const float4 v = in[q][r][g];
+            // the sample before the period: lane t stores components 2t, 2t + 1
+            const double a = (double)(t == 0 ? bs[r][0] : t == 1 ? bs[r][2] : bs[r][4]);
+            const double b = (double)(t == 0 ? bs[r][1] : t == 1 ? bs[r][3] : bs[r][5]);
+            if (valid[r] && t < 3) {
+                double* o = o0 + ((size_t)(8 * r) * T + k) * 6;
+                if (wide) {
+                    *reinterpret_cast<double2*>(o) = make_double2(a, b);
+                } else {
+                    o[0] = a;
+                    o[1] = b;
+                }
+            }
+            const float tc = bp.kp * (v.w - bs[r][2]) - bp.kd * bs[r][5];
+            uu[r][0] = v.x;
+            uu[r][1] = v.y;
+            uu[r][2] = v.z + tc;
+            if (NP > 1) pp[r][1] = (fminf(fmaxf(bs[r][5], d.plo[1]), d.phi[1]) - d.pm[1]) * d.inv_ps[1];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float u = 0.f;
+                if (LOW || j >= 2)
+                    u = (uq[j] == 0 ? uu[r][0] : uq[j] == 1 ? uu[r][1] : uq[j] == 2 ? uu[r][2] : 0.f) * fu[j];
+                z[4 * (j >> 1) + 2 * r + (j & 1)] = LOW || j >= 2 ? s[r][j] + u : s[r][j];  // one of the two is zero
+            }
+        }
+        float D[8];
+        product<NP, RG>(D, z, pp, bhi, blo);
+#pragma unroll
+        for (int r = 0; r < RG; ++r) {
+            float load[3];  // sloshing loads: the first three outputs, in physical units
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const float hi = odd[j] ? D[5 + 2 * r] : D[4 + 2 * r];
+                float v = hi;
+                if (LOW) v = up[j] ? hi : (odd[j] ? D[1 + 2 * r] : D[2 * r]);
+                load[j] = __shfl_sync(0xffffffffu, v, src[j]) * d.sy[j];
+            }
+            const float ax = (uu[r][0] + load[0]) * bp.inv_m, ay = (uu[r][1] + load[1]) * bp.inv_m;
+            const float aw = (uu[r][2] + load[2]) * bp.inv_J;
+            bs[r][0] += ndt * bs[r][3] + hdt2 * ax;
+            bs[r][1] += ndt * bs[r][4] + hdt2 * ay;
+            bs[r][2] += ndt * bs[r][5] + hdt2 * aw;
+            bs[r][3] += ndt * ax;
+            bs[r][4] += ndt * ay;
+            bs[r][5] += ndt * aw;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float v = D[4 * (j >> 1) + 2 * r + (j & 1)];
+                s[r][j] = (LOW || j >= 2) ? (is_x[j] ? v : 0.f) : v;
+            }
         }
     };
-    float cin[2][4];
-    fetch(0, cin);
-    for (int k = 0; k < T; ++k) {
-        float nin[2][4];
-        fetch(k + 1 < T ? k + 1 : k, nin);
-        float uu[2][3], pp[2][2];
+    for (int c = 0; c < n_chunk; ++c) {
+        copy_wait<kStages - 2>();
+        fetch(c + kStages - 1);
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const size_t o = (size_t)rr[q] * T + k;
-            if (vv[q] && t == 0) {
-#pragma unroll
-                for (int j = 0; j < 6; ++j) out[o * 6 + j] = bs[q][j];
-            }
-            const float tc = vv[q] ? bp.kp * (cin[q][3] - bs[q][2]) - bp.kd * bs[q][5] : 0.f;
-            uu[q][0] = cin[q][0];
-            uu[q][1] = cin[q][1];
-            uu[q][2] = vv[q] ? cin[q][2] + tc : 0.f;
-            // scheduling clamped to the range it was identified on
-            pp[q][0] = d.np > 0 ? (fminf(fmaxf(fl[q], d.plo[0]), d.phi[0]) - d.pm[0]) * d.inv_ps[0] : 0.f;
-            pp[q][1] = d.np > 1 ? (fminf(fmaxf(bs[q][5], d.plo[1]), d.phi[1]) - d.pm[1]) * d.inv_ps[1] : 0.f;
+        for (int r = 0; r < RG; ++r) {  // the period this lane copied
+            float v[4];
+            to_float<4>(raw[c % kStages][t][r][g], v);
+            in[t][r][g] = make_float4(v[0], v[1], v[2], v[3]);
         }
-        float z[8];
+        __syncwarp();
+        if ((c + 1) * kC <= T) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = scol(i, t), q = srow(i);
-            z[i] = (c < d.nx) ? s[i] : (c < d.nx + d.nu) ? uu[q][c - d.nx] * d.inv_su[c - d.nx] : 0.f;
+            for (int q = 0; q < kC; ++q) step(q, c * kC + q);
+        } else {
+            for (int q = 0; c * kC + q < T; ++q) step(q, c * kC + q);
         }
-        uint32_t ahi[kMaxKT][4], alo[kMaxKT][4];
-        afrag(z, ahi[0], alo[0]);
-#pragma unroll
-        for (int kt = 1; kt < kMaxKT; ++kt) {
-            float zs[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) zs[i] = z[i] * pp[srow(i)][kt - 1];
-            afrag(zs, ahi[kt], alo[kt]);
-        }
-        float D[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        mma_split<kMaxKT>(D, ahi, alo, bhi, blo, d.nkt);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            // sloshing loads: the first three outputs, in physical units
-            const float Fx = quad_get(D, d.nx, q, g) * d.sy[0];
-            const float Fy = quad_get(D, d.nx + 1, q, g) * d.sy[1];
-            const float Tb = quad_get(D, d.nx + 2, q, g) * d.sy[2];
-            const float ax = (uu[q][0] + Fx) * bp.inv_m, ay = (uu[q][1] + Fy) * bp.inv_m;
-            const float aw = (uu[q][2] + Tb) * bp.inv_J;
-            const float ndt = bp.n * bp.dt, hdt2 = bp.n_half * bp.dt * bp.dt;
-            bs[q][0] += ndt * bs[q][3] + hdt2 * ax;
-            bs[q][1] += ndt * bs[q][4] + hdt2 * ay;
-            bs[q][2] += ndt * bs[q][5] + hdt2 * aw;
-            bs[q][3] += ndt * ax;
-            bs[q][4] += ndt * ay;
-            bs[q][5] += ndt * aw;
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) s[i] = (scol(i, t) < d.nx) ? D[i] : 0.f;
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cin[q][j] = nin[q][j];
     }
 }
 
@@ -758,9 +845,16 @@ cudaError_t launch_closed_loop(const float* Wp, const Dims& d, int B, int T, con
                                const double* ref, const double* fill, const BodyParHost& h, double* out,
                                cudaStream_t st)
 {
-    const int warps = (B + 15) / 16, blocks = (warps + 3) / 4;
-    BodyPar bp{h.inv_m, h.inv_J, h.dt, h.n, h.n_half, h.kp, h.kd};
-    closed_loop_kernel<<<blocks, 128, 0, st>>>(Wp, d, B, T, F, tau, ref, fill, bp, out);
+    const BodyPar bp{h.inv_m, h.inv_J, h.dt, h.n, h.n_half, h.kp, h.kd};
+    const int wide = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    by_np(d.np, [&](auto np) {
+        constexpr int NP = decltype(np)::value;
+        auto go = [&](auto kernel) {
+            kernel<<<serial_warps(B), 32, 0, st>>>(Wp, d, B, T, F, tau, ref, fill, bp, out, wide);
+        };
+        if (row_groups(B) == 1) d.nx < 8 ? go(closed_loop_kernel<true, NP, 1>) : go(closed_loop_kernel<false, NP, 1>);
+        else d.nx < 8 ? go(closed_loop_kernel<true, NP, 2>) : go(closed_loop_kernel<false, NP, 2>);
+    });
     return cudaGetLastError();
 }
 

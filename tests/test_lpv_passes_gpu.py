@@ -64,3 +64,40 @@ def test_passes_match_fp64(na, n_y, n_p, nu, n, T):
     assert abs(loss - ref) <= 1e-4 * ref
     assert np.abs(g - gr).max() <= 1e-3 * np.abs(gr).max()
     assert np.abs(yh - yr).max() <= 1e-3 * np.abs(yr).max()
+
+
+@pytest.mark.parametrize("na,n_y,n_p,nu,B,T", [(3, 4, 2, 3, 1, 1), (3, 4, 2, 3, 19, 37), (2, 3, 1, 3, 8, 4), (1, 4, 0, 3, 5, 9),
+                                               (2, 3, 2, 2, 4871, 6), (3, 4, 2, 3, 4866, 5), (4, 3, 0, 1, 33, 10)])
+def test_closed_loop_matches_fp64(na, n_y, n_p, nu, B, T):
+    torch = need_gpu()
+    from paper_2604_12505_gb300 import lpv
+    rng = np.random.default_rng(7 * B + T)
+    nx = na * n_y
+    W, sc = _model(rng, na, n_y, n_p, nu)
+    body = dict(m=500.0, J=50.0, Ts=0.02, n_sub=10, ctrl_omega=0.2 * np.pi, ctrl_xi=0.7)
+    F, tau = rng.uniform(-20, 20, (B, T, 2)), rng.uniform(-2, 2, (B, T))
+    ref, fill = rng.uniform(-0.3, 0.3, (B, T)), rng.uniform(0.2, 0.8, B)
+    F[0, 0] = 0.0, -0.0
+    ref[:, T // 2] = 1e-42  # not a normal FP32 number
+    m = lpv.Model(dict(n_x=nx, n_u=nu, n_y=n_y, n_p=n_p, na=na))
+    m.set_params(W, sc)
+    out = m.simulate(F, tau, ref, fill, body).cpu().numpy()
+    m.close()
+
+    Wd, s = W.astype(np.float64), sc.astype(np.float64)
+    su, sy, pm, ps = s[:nu], s[nu:nu + n_y], s[nu + n_y:nu + n_y + n_p], s[nu + n_y + n_p:nu + n_y + 2 * n_p]
+    x, q, v = np.zeros((B, nx)), np.zeros((B, 3)), np.zeros((B, 3))
+    mass, w, want = np.array([500.0, 500.0, 50.0]), 0.2 * np.pi, np.zeros((B, T, 6))
+    for k in range(T):
+        want[:, k] = np.concatenate([q, v], 1)
+        u = np.concatenate([F[:, k], (tau[:, k] + 50.0 * w * w * (ref[:, k] - q[:, 2]) - 1.4 * 50.0 * w * v[:, 2])[:, None]], 1)
+        p = (np.clip(np.stack([fill, v[:, 2]], 1)[:, :n_p], -5.0, 5.0) - pm) / ps
+        z = np.concatenate([x, u[:, :nu] / su], 1)
+        o = z @ Wd[0].T + sum(p[:, i:i + 1] * (z @ Wd[1 + i].T) for i in range(n_p))
+        x = o[:, :nx]
+        a = (u + o[:, nx:nx + 3] * sy[:3]) / mass
+        for _ in range(10):
+            v = v + 0.002 * a
+            q = q + 0.002 * v
+    for blk in (slice(0, 3), slice(3, 6)):
+        assert np.abs(out[:, :, blk] - want[:, :, blk]).max() <= 1e-3 * max(np.abs(want[:, :, blk]).max(), 1e-300)
