@@ -43,3 +43,25 @@ def test_passes_match_oracle(nx, n, T, copies):
     assert np.abs(g - ref_g).max() <= 1e-3 * np.abs(ref_g).max()
     assert abs(float(alone.item()) - loss) <= 1e-12 * loss
     m.close()
+
+
+@pytest.mark.parametrize("nx,B,T", [(2, 1, 1), (4, 33, 5), (4, 64, 8), (6, 31, 7), (8, 40, 3)])
+def test_closed_loop_matches_oracle_at_edge_sizes(nx, B, T):
+    torch = need_gpu()
+    from paper_2604_12505_gb300.slpv import VelocityModel
+    th64, th32 = _theta(nx, 21, m1=0.2)
+    rng = np.random.default_rng(B + T)
+    F, tau, ref = rng.uniform(-20, 20, (B, T, 2)), rng.uniform(-2, 2, (B, T)), rng.uniform(-0.3, 0.3, (B, T))
+    pd = dict(J=133.84, omega=0.2 * np.pi, xi=0.7)
+    m = VelocityModel(nx=nx)
+    m.set_params(th32, SC)
+    # the second time from buffers that are 8-byte but not 16-byte aligned
+    odd = torch.empty(2 * B * T + 1, dtype=torch.float64, device="cuda")[1:].view(B, T, 2)
+    odd.copy_(torch.tensor(F))
+    for f in (F, odd):
+        out = m.simulate(f, tau, ref, 0.05, pd["J"], pd["omega"], pd["xi"]).cpu().numpy()
+        want = np.stack([S.closed_loop(th64, nx, dict(u=SC[:3].astype(np.float64), y=SC[3:].astype(np.float64)), F[b],
+                                       tau[b], ref[b], 0.05, pd) for b in range(B)])
+        for blk in (slice(0, 3), slice(3, 6)):
+            assert np.abs(out[:, :, blk] - want[:, :, blk]).max() <= 1e-3 * np.abs(want[:, :, blk]).max() + 1e-12
+    m.close()
