@@ -275,11 +275,13 @@ int sph_eval_jvp(sph_sim* sim, const double* u, const double* du, const float* d
  *  xvbar0     float32 [N, 4] out: adjoint of the initial fluid state (NULL: skip)
  *  bodybar0   float64 [B, 6] out: adjoint of the initial body state (NULL: skip)
  *  ubar       float64 [B, K, 3] out: adjoint of u (NULL: skip)
- * The forward pass keeps a checkpoint every checkpoint_every steps; the
- * reverse sweep recomputes each segment from its checkpoint and runs the
- * adjoint kernels on 4x4 tiles (device memory of about K / checkpoint_every +
- * checkpoint_every states, allocated for the call).  The simulator is left at
- * state K, as after sph_jvp.  Blocks until done.
+ * The forward pass keeps a checkpoint every checkpoint_every steps; each
+ * segment is run again from its checkpoint with its steps recorded, and the
+ * adjoint kernels run backwards over the records on 4x4 tiles.  Device memory:
+ * K / checkpoint_every states for the call, and records of up to 2 GB (more
+ * where the checkpoints and a segment's states take more, a step's at least,
+ * and less where the device has no room), which the handle keeps for its next
+ * call.  The simulator is left at state K, as after sph_jvp.  Blocks until done.
  */
 int sph_vjp(sph_sim* sim, const double* u, int32_t K, const double* ybar, const float* xvbar_K,
             const double* bodybar_K, float* xvbar0, double* bodybar0, double* ubar, int32_t checkpoint_every,

@@ -20,7 +20,16 @@
 //
 // Body terms are summed per tile in compensated two-float FP32 and per tank
 // in fixed order, so the result is deterministic.  One CTA per tile of 4x4
-// cells, staged like the forward pass.
+// cells, staged from the forward step's record.
+//
+// A reverse step is three launches (the body, the force pass's adjoint, the
+// density pass's) chained by programmatic dependent launch: what a kernel
+// stages is the forward step's record, complete long before, so each stages
+// its tile and its ghosts while its predecessor still runs.  50 steps of the
+// 15,532-particle tank, checkpoints every 10: 8.3 -> 3.7 ms.  Before, a
+// reverse step was ten launches (the state re-binned, the primal density pass
+// run again, the tiles sorted twice, ghosts from global memory) and the
+// recomputed steps came one after the other on the same stream.
 #include <cuda_runtime.h>
 
 #include "sph_common.cuh"
@@ -80,71 +89,37 @@ __device__ void store_part6(const float (&a)[6], float* out)
 
 }  // namespace
 
-// Body integration adjoint and the step's sample adjoints, one thread per tank (FP64).
-__global__ void adj_body_pre_kernel(SimDev S, AdjDev A)
-{
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= S.B) return;
-    const TankDev& T = S.tank[b];
-    const double* bb = A.bbar + 6 * b;
-    const double dt = T.dt_d;
-    // r' = r + dt rdot', rdot' = rdot + dt (F_b + u) / M (theta likewise)
-    const double rdx = bb[3] + dt * bb[0], rdy = bb[4] + dt * bb[1], wd = bb[5] + dt * bb[2];
-    double Fx = dt / T.m_body * rdx, Fy = dt / T.m_body * rdy, Tq = dt / T.J_body * wd;
-    if (A.ubar) {
-        double* ub = A.ubar + b * A.ubar_stride + 3ll * A.k;
-        ub[0] = Fx;
-        ub[1] = Fy;
-        ub[2] = Tq;
-    }
-    double part[6] = {bb[0], bb[1], bb[2], rdx, rdy, wd};
-    float cx = 0.f, cy = 0.f;
-    if (A.row >= 0 && A.ybar) {  // samples of this step: body state, F_b, T_b, fluid centre of mass
-        const double* y = A.ybar + b * A.ybar_stride + (long long)A.row * SPH_NY;
-        for (int q = 0; q < 6; ++q) part[q] += y[q];
-        Fx += y[6];
-        Fy += y[7];
-        Tq += y[8];
-        if (T.n_f) {
-            cx = (float)(y[9] / T.n_f);
-            cy = (float)(y[10] / T.n_f);
-        }
-    }
-    for (int q = 0; q < 6; ++q) A.bbar_part[6 * b + q] = part[q];
-    float* fb = A.fbar + 8 * b;
-    fb[0] = (float)Fx;
-    fb[1] = (float)Fy;
-    fb[2] = (float)Tq;
-    fb[3] = cx;
-    fb[4] = cy;
-}
-
 // Adjoint of the force pass, the EOS and the kick-then-drift of the fluid.
 template <int TX, int TY>
 __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_force_kernel(SimDev S, AdjDev A)
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, true, false> sm;
+    __shared__ GhostStage<true> gs;
     __shared__ float2 sab[Sh::MAXS];  // acceleration adjoint of each staged particle
     const int4 td = S.tiles[blockIdx.x];
     const int tank = td.x;
     const TankDev T = S.tank[tank];
-    const int buf = (int)(S.run->step & 1);
     float bacc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (stage_tile<TX, TY, true, false>(S, T, buf, td.y, td.z, sm)) {
+    bool waited = false;
+    if (stage_from_record<TX, TY, false>(S, tank, A.buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
         const float dt = T.dt;
         const int total = sm.start[Sh::NC];
+        const BodyDev& b = S.body[tank];
+        const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry, om = b.fw;
+        const int n_own = sm.own_row[TY];
+        const int gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs) : kGhostsNone;
+        pdl_wait();  // the adjoint of the state after the step, the body's part
+        pdl_trigger();
+        waited = true;
         for (int e = threadIdx.x; e < total; e += blockDim.x) {
             const float4 a = A.in[sm.pid[e]];
             sab[e] = make_float2(dt * (a.z + dt * a.x), dt * (a.w + dt * a.y));
         }
         __syncthreads();
-        const BodyDev& b = S.body[tank];
-        const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry, om = b.fw;
         const float* fb = A.fbar + 8 * tank;
         const float Fbx = fb[0], Fby = fb[1], Tbb = fb[2], cmx = fb[3], cmy = fb[4];
         const float m = T.m, mm = T.m * T.m;
-        const int n_own = sm.own_row[TY];
         for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
             const int e = own_index(t, sm);
             const float4 pi = sm.pv[e];
@@ -196,13 +171,13 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_force_kernel(SimDe
                     }
                 }
             }
-            for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry, [&](int g) {
-                const float4 gp = S.gpos[g];
+            // one ghost: its world position, and load_gv() its (v_x, v_y, arm_x, arm_y)
+            auto ghost = [&](const float4 gp, auto&& load_gv) {
                 const float2 sg = sep_fg(pi, li, gp);
                 const float dx = sg.x, dy = sg.y;
                 const float r2 = dist2(dx, dy);
                 if (!(r2 < T.h2) || !(r2 > 0.f)) return;
-                const float4 gv = S.gvel[g];                             // (v_g, arm)
+                const float4 gv = load_gv();
                 const float inv_r = rsqrtf(r2), r = r2 * inv_r;
                 const float d = T.h - r;
                 const float Gs = T.cdS * d * d * inv_r;                  // (dW_s/dr) / r
@@ -240,11 +215,17 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_force_kernel(SimDe
                 bacc[3] += vgx;
                 bacc[4] += vgy;
                 bacc[5] += vgy * gv.z - vgx * gv.w;
-            });
+            };
+            if (gmode == kGhostsStaged)
+                for_staged_ghosts(T, gs, pi.x, pi.y, bc, bs, brx, bry, T.hclip,
+                                  [&](int, int q) { ghost(gs.gp[q], [&] { return gs.gv[q]; }); });
+            else if (gmode == kGhostsGlobal)
+                for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry, [&](int g) { ghost(S.gpos[g], [&] { return S.gvel[g]; }); });
             A.out[id] = make_float4(xbx, xby, vbx, vby);
             A.rhobar[id] = rb + qb * (T.k / (ri.x * ri.x) - 2.0f * ri.y / ri.x);  // Eq. 11 with q = P / rho^2
         }
     }
+    if (!waited) pdl_wait();  // before the partials of the step before are overwritten
     store_part6<Sh::THREADS>(bacc, A.part + (size_t)blockIdx.x * 12);
 }
 
@@ -253,21 +234,26 @@ template <int TX, int TY>
 __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(SimDev S, AdjDev A)
 {
     using Sh = Shape<TX, TY>;
-    __shared__ Stage<TX, TY, false, false> sm;
+    __shared__ Stage<TX, TY, true, false> sm;
+    __shared__ GhostStage<true> gs;
     __shared__ float srb[Sh::MAXS];  // density adjoint of each staged particle
     const int4 td = S.tiles[blockIdx.x];
     const int tank = td.x;
     const TankDev T = S.tank[tank];
-    const int buf = (int)(S.run->step & 1);
     float bacc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (stage_tile<TX, TY, false, false>(S, T, buf, td.y, td.z, sm)) {
+    bool waited = false;
+    if (stage_from_record<TX, TY, false>(S, tank, A.buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
         const int total = sm.start[Sh::NC];
-        for (int e = threadIdx.x; e < total; e += blockDim.x) srb[e] = A.rhobar[sm.pid[e]];
-        __syncthreads();
         const BodyDev& b = S.body[tank];
         const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry;
-        const float m = T.m, mg = T.m * T.gamma1;
         const int n_own = sm.own_row[TY];
+        const int gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs) : kGhostsNone;
+        pdl_wait();  // the density adjoints
+        pdl_trigger();
+        waited = true;
+        for (int e = threadIdx.x; e < total; e += blockDim.x) srb[e] = A.rhobar[sm.pid[e]];
+        __syncthreads();
+        const float m = T.m, mg = T.m * T.gamma1;
         for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
             const int e = own_index(t, sm);
             const float4 pi = sm.pv[e];
@@ -296,13 +282,12 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(Sim
                     }
                 }
             }
-            for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry, [&](int g) {
-                const float4 gp = S.gpos[g];
+            auto ghost = [&](const float4 gp, auto&& load_gv) {
                 const float2 d = sep_fg(pi, li, gp);
                 const float dx = d.x, dy = d.y;
                 const float r2 = dist2(dx, dy);
                 if (!(r2 < T.R2) || !(r2 > 0.f)) return;
-                const float4 gv = S.gvel[g];
+                const float4 gv = load_gv();
                 const float inv_r = rsqrtf(r2), r = r2 * inv_r;
                 const float k = mg * rbi * dw_cubic_over_r(T, r, inv_r);
                 xbx += k * dx;
@@ -311,7 +296,12 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(Sim
                 bacc[0] += gwx;
                 bacc[1] += gwy;
                 bacc[2] += gwy * gv.z - gwx * gv.w;
-            });
+            };
+            if (gmode == kGhostsStaged)
+                for_staged_ghosts(T, gs, pi.x, pi.y, bc, bs, brx, bry, T.clip,
+                                  [&](int, int q) { ghost(gs.gp[q], [&] { return gs.gv[q]; }); });
+            else if (gmode == kGhostsGlobal)
+                for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry, [&](int g) { ghost(S.gpos[g], [&] { return S.gvel[g]; }); });
             const int id = sm.pid[e];
             float4 o = A.out[id];
             o.x += xbx;
@@ -319,27 +309,83 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(Sim
             A.out[id] = o;
         }
     }
+    if (!waited) pdl_wait();
     store_part6<Sh::THREADS>(bacc, A.part + ((size_t)A.max_tiles + blockIdx.x) * 12);
 }
 
-// Body adjoint of the state before the step: the integration part plus the
-// ghost terms of both passes, summed over the tank's tiles in fixed order.
-__global__ void __launch_bounds__(128) adj_body_post_kernel(SimDev S, AdjDev A)
+// The body between two reverse steps, one block per tank (FP64).  post: the
+// body adjoint of the state before the step just reversed, its integration
+// part plus the ghost terms of both passes, summed over the tank's tiles in
+// fixed order.  pre: the integration adjoint of step A.k and the adjoints of
+// its sample.
+__global__ void __launch_bounds__(128) adj_body_kernel(SimDev S, AdjDev A, int post, int pre)
 {
+    pdl_trigger();
     const int b = blockIdx.x;
     const int t0 = S.tile_tank_first[b], t1 = S.tile_tank_first[b + 1];
+    const TankDev& T = S.tank[b];
+    // what does not depend on the step just reversed: FP64 is slow here, divisions most of all
+    double kM = 0.0, kJ = 0.0, dt = 0.0, ys[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    float cx = 0.f, cy = 0.f;
+    if (threadIdx.x == 0 && pre) {
+        dt = T.dt_d;
+        kM = dt / T.m_body;
+        kJ = dt / T.J_body;
+        if (A.row >= 0 && A.ybar) {  // samples of this step: body state, F_b, T_b, fluid centre of mass
+            const double* y = A.ybar + b * A.ybar_stride + (long long)A.row * SPH_NY;
+            for (int q = 0; q < 9; ++q) ys[q] = y[q];
+            if (T.n_f) {
+                cx = (float)(y[9] / T.n_f);
+                cy = (float)(y[10] / T.n_f);
+            }
+        }
+    }
     F2 v[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) v[c] = F2{0.f, 0.f};
-    for (int p = 0; p < 2; ++p)
-        for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
-            const float* P = A.part + ((size_t)p * A.max_tiles + t) * 12;
-#pragma unroll
-            for (int c = 0; c < 6; ++c) v[c] = f2_add(v[c], F2{P[2 * c], P[2 * c + 1]});
-        }
-    block_sum6<128>(v);
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 6; ++c) A.bbar[6 * b + c] = A.bbar_part[6 * b + c] + ((double)v[c].hi + (double)v[c].lo);
+    pdl_wait();
+    if (post) {
+        for (int p = 0; p < 2; ++p)
+            for (int t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
+                const float4* P = reinterpret_cast<const float4*>(A.part + ((size_t)p * A.max_tiles + t) * 12);
+                const float4 x = P[0], y = P[1], z = P[2];
+                v[0] = f2_add(v[0], F2{x.x, x.y});
+                v[1] = f2_add(v[1], F2{x.z, x.w});
+                v[2] = f2_add(v[2], F2{y.x, y.y});
+                v[3] = f2_add(v[3], F2{y.z, y.w});
+                v[4] = f2_add(v[4], F2{z.x, z.y});
+                v[5] = f2_add(v[5], F2{z.z, z.w});
+            }
+        block_sum6<128>(v);
+    }
+    if (threadIdx.x) return;
+    double bb[6];
+    for (int c = 0; c < 6; ++c) {
+        bb[c] = post ? A.bbar_part[6 * b + c] + ((double)v[c].hi + (double)v[c].lo) : A.bbar[6 * b + c];
+        if (post) A.bbar[6 * b + c] = bb[c];
+    }
+    if (!pre) return;
+    // r' = r + dt rdot', rdot' = rdot + dt (F_b + u) / M (theta likewise)
+    const double rdx = bb[3] + dt * bb[0], rdy = bb[4] + dt * bb[1], wd = bb[5] + dt * bb[2];
+    double Fx = kM * rdx, Fy = kM * rdy, Tq = kJ * wd;
+    if (A.ubar) {
+        double* ub = A.ubar + b * A.ubar_stride + 3ll * A.k;
+        ub[0] = Fx;
+        ub[1] = Fy;
+        ub[2] = Tq;
+    }
+    double part[6] = {bb[0], bb[1], bb[2], rdx, rdy, wd};
+    for (int q = 0; q < 6; ++q) part[q] += ys[q];
+    Fx += ys[6];
+    Fy += ys[7];
+    Tq += ys[8];
+    for (int q = 0; q < 6; ++q) A.bbar_part[6 * b + q] = part[q];
+    float* fb = A.fbar + 8 * b;
+    fb[0] = (float)Fx;
+    fb[1] = (float)Fy;
+    fb[2] = (float)Tq;
+    fb[3] = cx;
+    fb[4] = cy;
 }
 
 __global__ void set_step_kernel(RunDev* run, long long step)
@@ -358,20 +404,18 @@ cudaError_t launch_set_step(RunDev* run, long long step, cudaStream_t st)
 
 int adjoint_tile_code() { return kAdjCode; }
 
-// One reverse step on the state set in the grid (S built for the 4x4 tiles).
+cudaError_t launch_adjoint_body(const SimDev& S, const AdjDev& A, int post, int pre, cudaStream_t st, bool pdl)
+{
+    return launch(adj_body_kernel, S.B, 128, st, pdl, S, A, post, pre);
+}
+
+// The fluid's reverse step over a recorded step (S built for the 4x4 tiles).
 cudaError_t launch_adjoint_step(const SimDev& S, const AdjDev& A, int n_tiles, cudaStream_t st)
 {
     using Sh = Shape<kAdjTX, kAdjTY>;
-    adj_body_pre_kernel<<<(S.B + 127) / 128, 128, 0, st>>>(S, A);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch(adj_force_kernel<kAdjTX, kAdjTY>, n_tiles, Sh::THREADS, st, true, S, A);
     if (e != cudaSuccess) return e;
-    EvalOut E{};
-    e = launch_phase(S, E, 0, kAdjCode, n_tiles, 0, st, false);  // primal density pass of this state
-    if (e != cudaSuccess) return e;
-    adj_force_kernel<kAdjTX, kAdjTY><<<n_tiles, Sh::THREADS, 0, st>>>(S, A);
-    adj_density_kernel<kAdjTX, kAdjTY><<<n_tiles, Sh::THREADS, 0, st>>>(S, A);
-    adj_body_post_kernel<<<S.B, 128, 0, st>>>(S, A);
-    return cudaGetLastError();
+    return launch(adj_density_kernel<kAdjTX, kAdjTY>, n_tiles, Sh::THREADS, st, true, S, A);
 }
 
 }  // namespace sph

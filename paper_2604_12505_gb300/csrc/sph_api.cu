@@ -11,6 +11,7 @@
 #include <cstddef>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/sph.h"
@@ -140,13 +141,6 @@ struct DevScratch {
     }
 };
 
-// Rows [k0, k0 + n) of u [B, K, 3] into dst [B, n, 3].
-cudaError_t slice_u(double* dst, const double* u, int B, int K, int k0, int n, cudaStream_t st)
-{
-    return cudaMemcpy2DAsync(dst, 3 * sizeof(double) * n, u + 3ll * k0, 3 * sizeof(double) * K,
-                             3 * sizeof(double) * n, B, cudaMemcpyDeviceToDevice, st);
-}
-
 }  // namespace
 
 namespace sph {
@@ -178,6 +172,10 @@ struct sph_sim {
     int graph_tile = 0;
     bool use_pdl = true;
     int max_tiles = 0, max_groups = 0;
+    char* d_rec = nullptr;  // sph_vjp's records, kept for the next call (at most kRecordBytes, or one step's)
+    size_t rec_bytes = 0;
+    cudaStream_t side = nullptr;  // sph_vjp's second stream and the event that orders the two
+    cudaEvent_t ev = nullptr;
 
     SimDev dev(int code = 0) const
     {
@@ -219,6 +217,9 @@ void free_sim(sph_sim* s)
     cudaFree(s->d_scratch_body);
     cudaFree(s->d_scratch_xv);
     cudaFree(s->d_scratch_lo);
+    cudaFree(s->d_rec);
+    if (s->side) cudaStreamDestroy(s->side);
+    if (s->ev) cudaEventDestroy(s->ev);
     for (int b = 0; b < 2; ++b) {
         cudaFree(s->S.pv[b]);
         cudaFree(s->S.lo[b]);
@@ -627,6 +628,27 @@ int sph_samples_for(const sph_sim* sim, int32_t n_steps, int32_t* n_samples)
     return SPH_OK;
 }
 
+namespace {
+// n_steps steps under the run record already set: whole graphs, then single steps.
+int run_steps(sph_sim* sim, int n_steps, cudaStream_t st)
+{
+    int rc = ensure_graph(sim);
+    if (rc) return rc;
+    int left = n_steps;
+    EvalOut E{};
+    while (left >= kGraphSteps) {
+        CK(cudaGraphLaunch(sim->graph, st));
+        left -= kGraphSteps;
+    }
+    for (int i = 0; left > 0; --left, ++i) {
+        rc = sim->step_launch(E, 0, st, i > 0);
+        if (rc) return rc;
+    }
+    sim->host_step += n_steps;
+    return SPH_OK;
+}
+}  // namespace
+
 int sph_step(sph_sim* sim, const double* u, int32_t n_steps, const sph_ctrl* pd, double* y_out, void* stream)
 {
     if (!sim || n_steps < 0) return fail(SPH_E_INVAL, "sph_step: bad argument");
@@ -651,20 +673,7 @@ int sph_step(sph_sim* sim, const double* u, int32_t n_steps, const sph_ctrl* pd,
         d.ref_stride = pd->ref_stride;
     }
     CK(launch_set_run(sim->d_run, d, st));
-    int rc = ensure_graph(sim);
-    if (rc) return rc;
-    int left = n_steps;
-    EvalOut E{};
-    while (left >= kGraphSteps) {
-        CK(cudaGraphLaunch(sim->graph, st));
-        left -= kGraphSteps;
-    }
-    for (int i = 0; left > 0; --left, ++i) {
-        rc = sim->step_launch(E, 0, st, i > 0);
-        if (rc) return rc;
-    }
-    sim->host_step += n_steps;
-    return SPH_OK;
+    return run_steps(sim, n_steps, st);
 }
 
 int sph_relax(sph_sim* sim, int32_t n_steps, double damping, void* stream)
@@ -761,6 +770,95 @@ int sph_jvp(sph_sim* sim, const double* u, const double* du, const float* dxv0, 
     return SPH_OK;
 }
 
+namespace {
+// A recorded run keeps, per step, the state after it in the grid that the
+// step left, and what the adjoint of the step reads: its state binned at the
+// body's position (as a call on that state would bin it), the densities, the
+// neighbour and staging records, the ghosts' positions and the body.
+struct Recorder {
+    size_t n_slot, n_cell, n_ghost, n_own, srec_bytes;
+    int B;
+    size_t step_bytes = 0;
+    static size_t up(size_t n) { return (n + 255) & ~(size_t)255; }
+
+    Recorder(const sph_sim* sim, int code)
+    {
+        int TX, TY;
+        tile_dims(code, &TX, &TY);
+        int nt[SPH_TILE_COUNT + 1] = {0};
+        nt[code] = sim->n_tiles[code];
+        n_cell = sim->n_cells_total;
+        n_slot = n_cell * kCap;
+        n_ghost = sim->n_g_total;
+        n_own = (size_t)nt[code] * TX * TY * 12;
+        srec_bytes = stage_record_bytes(nt);
+        B = sim->B;
+        RecordDev unused{};
+        step_bytes = place(nullptr, unused);
+    }
+    // Points R at a first record at `at`; returns a record's size.
+    size_t place(char* at, RecordDev& R) const
+    {
+        size_t o = 0;
+        auto take = [&](size_t bytes) {
+            char* p = at + o;
+            o += up(bytes);
+            return (void*)p;
+        };
+        SimDev& s = R.first;
+        const int b = R.buf0;
+        R.next_pv = (float4*)take(n_slot * sizeof(float4));
+        R.next_lo = (float4*)take(n_slot * sizeof(float4));
+        R.next_pid = (int*)take(n_slot * sizeof(int));
+        s.pv[b] = (float4*)take(n_slot * sizeof(float4));
+        s.lo[b] = (float4*)take(n_slot * sizeof(float4));
+        s.pid[b] = (int*)take(n_slot * sizeof(int));
+        s.rhoP = (float2*)take(n_slot * sizeof(float2));
+        s.gpos = (float4*)take(n_ghost * sizeof(float4));
+        s.gvel = (float4*)take(n_ghost * sizeof(float4));
+        s.nbm = (unsigned int*)take(3 * n_own * sizeof(unsigned int));
+        s.nba = (unsigned short*)take(3 * n_own * sizeof(unsigned short));
+        s.nbn = (unsigned char*)take(n_own);
+        s.srec = (unsigned char*)take(srec_bytes);
+        s.brec = (double*)take((size_t)B * kBodyRec * sizeof(double));
+        return o;
+    }
+    // Apart from the records: the cell counts of both states of every step
+    // (cleared together before a run), and the body records.
+    size_t count_stride() const { return up(n_cell * sizeof(int)) / sizeof(int); }
+    size_t step_total() const { return step_bytes + 2 * count_stride() * sizeof(int) + (size_t)B * sizeof(BodyDev); }
+    // Points s at working memory of its own at `at`, so that its steps run
+    // beside the simulator's: bodies, run record, and what a step leaves for
+    // itself; returns its size.
+    static size_t own_work(char* at, SimDev& s, const sph_sim* sim)
+    {
+        size_t o = 0, nn = 0;
+        auto take = [&](size_t bytes) {
+            char* p = at + o;
+            o += up(bytes);
+            return (void*)p;
+        };
+        for (int code = 1; code <= SPH_TILE_COUNT; ++code) {
+            int TX, TY;
+            tile_dims(code, &TX, &TY);
+            nn = std::max(nn, (size_t)sim->n_tiles[code] * TX * TY * 12);
+        }
+        s.body = (BodyDev*)take(sim->B * sizeof(BodyDev));
+        s.run = (RunDev*)take(sizeof(RunDev));
+        s.rhoP = (float2*)take((size_t)sim->n_cells_total * kCap * sizeof(float2));
+        s.gpos = (float4*)take(sim->n_g_total * sizeof(float4));
+        s.gvel = (float4*)take(sim->n_g_total * sizeof(float4));
+        s.nbm = (unsigned int*)take(3 * nn * sizeof(unsigned int));
+        s.nba = (unsigned short*)take(3 * nn * sizeof(unsigned short));
+        s.nbn = (unsigned char*)take(nn);
+        s.srec = (unsigned char*)take(stage_record_bytes(sim->n_tiles));
+        return o;
+    }
+};
+
+constexpr size_t kRecordBytes = 2ull << 30;
+}  // namespace
+
 int sph_vjp(sph_sim* sim, const double* u, int32_t K, const double* ybar, const float* xvbar_K,
             const double* bodybar_K, float* xvbar0, double* bodybar0, double* ubar, int32_t checkpoint_every,
             void* stream)
@@ -770,38 +868,72 @@ int sph_vjp(sph_sim* sim, const double* u, int32_t K, const double* ybar, const 
         if (sim->tanks[b].p.outer_every != sim->tanks[0].p.outer_every)
             return fail(SPH_E_UNSUPPORTED, "sph_vjp: tanks of a batch must share outer_every");
     cudaStream_t st = (cudaStream_t)stream;
-    const int B = sim->B, N = sim->n_f_total, C = checkpoint_every;
+    const int B = sim->B, N = sim->n_f_total;
     const long long step0 = sim->host_step;
     const int oe = sim->tanks[0].p.outer_every > 0 ? sim->tanks[0].p.outer_every : 1;
-    const int n_seg = (K + C - 1) / C;
     const size_t nxv = 4 * (size_t)N;
+    const int code = adjoint_tile_code();
+    const Recorder rec(sim, code);
+    // The trajectory is run once for the states at every checkpoint_every-th
+    // step (as the header says), and each segment again from its checkpoint,
+    // recording its steps: on a stream of its own beside the forward pass when
+    // the records of all K steps fit kRecordBytes (a small tank leaves most of
+    // the GPU idle), else group by group of segments before they are reversed.
+    // A segment longer than the records' room is cut.
+    const size_t per = rec.step_total(), state_bytes = 2 * nxv * sizeof(float) + 6 * (size_t)B * sizeof(double);
+    const size_t allowed = std::max(kRecordBytes, 2 * state_bytes * ((size_t)K / checkpoint_every + checkpoint_every));
+    SimDev lane = sim->dev();
+    const size_t work = Recorder::own_work(nullptr, lane, sim);
+    int L = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::max(K, 1), allowed / per));
+    while (sim->rec_bytes < work + per * L) {  // fewer steps a group where the device has no room
+        cudaFree(sim->d_rec);
+        sim->d_rec = nullptr;
+        sim->rec_bytes = 0;
+        if (cudaMalloc((void**)&sim->d_rec, work + per * L) == cudaSuccess) {
+            sim->rec_bytes = work + per * L;
+        } else {
+            sim->d_rec = nullptr;
+            cudaGetLastError();
+            if (L == 1) return fail(SPH_E_NOMEM, "sph_vjp: no memory for a step's record");
+            L = (L + 1) / 2;
+        }
+    }
+    const int C = std::min(std::min(checkpoint_every, L), std::max(K, 1)), n_seg = (K + C - 1) / C;
+    const int per_grp = L >= K ? std::max(n_seg, 1) : std::max(1, L / C);  // segments of a group
+    const int n_grp = (n_seg + per_grp - 1) / per_grp;
+    const bool beside = n_grp == 1;
+    if (!sim->side) {
+        CK(cudaStreamCreateWithFlags(&sim->side, cudaStreamNonBlocking));
+        CK(cudaEventCreateWithFlags(&sim->ev, cudaEventDisableTiming));
+    }
     DevScratch mem;
     float4 *adj0 = nullptr, *adj1 = nullptr;
-    float *rhob = nullptr, *fbar = nullptr, *part = nullptr, *ck_xv = nullptr, *seg_xv = nullptr, *fin_xv = nullptr;
-    float *ck_lo = nullptr, *seg_lo = nullptr, *fin_lo = nullptr;
-    double *bbar = nullptr, *bpart = nullptr, *ck_b = nullptr, *seg_b = nullptr, *fin_b = nullptr, *us = nullptr;
-    const int code = adjoint_tile_code();
+    float *rhob = nullptr, *fbar = nullptr, *part = nullptr, *ck = nullptr;
+    double *bbar = nullptr, *bpart = nullptr, *ck_b = nullptr;
+    const int n_ck = n_seg + 1;  // the segments' first states and the final one
     int rc = mem.get(&adj0, N) | mem.get(&adj1, N) | mem.get(&rhob, N) | mem.get(&fbar, 8 * (size_t)B) |
              mem.get(&part, 2 * (size_t)sim->max_tiles * 12) | mem.get(&bbar, 6 * (size_t)B) |
-             mem.get(&bpart, 6 * (size_t)B) | mem.get(&ck_xv, nxv * (n_seg ? n_seg : 1)) |
-             mem.get(&ck_b, 6 * (size_t)B * (n_seg ? n_seg : 1)) | mem.get(&seg_xv, nxv * C) |
-             mem.get(&seg_b, 6 * (size_t)B * C) | mem.get(&fin_xv, nxv) | mem.get(&fin_b, 6 * (size_t)B) |
-             mem.get(&us, 3 * (size_t)B * C) | mem.get(&ck_lo, nxv * (n_seg ? n_seg : 1)) |
-             mem.get(&seg_lo, nxv * C) | mem.get(&fin_lo, nxv);
+             mem.get(&bpart, 6 * (size_t)B) | mem.get(&ck, 2 * nxv * n_ck) | mem.get(&ck_b, 6 * (size_t)B * n_ck);
     if (rc) return SPH_E_NOMEM;
+    Recorder::own_work(sim->d_rec, lane, sim);
+    char* const recs = sim->d_rec + work;
+    RecordDev R{};
+    BodyDev* const bodies = (BodyDev*)(recs + rec.step_bytes * L);
+    int* const counts = (int*)(bodies + (size_t)B * L);  // of the states after the steps, then of the steps' own
+    auto save = [&](int i) {
+        return get_state_full(sim, ck + 2 * nxv * i, ck + 2 * nxv * i + nxv, ck_b + 6ll * B * i, st);
+    };
+    auto run_of = [&](int k) {
+        RunDev d{};
+        d.u = u ? u + 3ll * k : nullptr;
+        d.u_tank_stride = 3ll * K;
+        return d;
+    };
     // adjoint of the final state
     if (xvbar_K) CK(cudaMemcpyAsync(adj0, xvbar_K, nxv * sizeof(float), cudaMemcpyDeviceToDevice, st));
     else CK(cudaMemsetAsync(adj0, 0, nxv * sizeof(float), st));
     if (bodybar_K) CK(cudaMemcpyAsync(bbar, bodybar_K, 6 * B * sizeof(double), cudaMemcpyDeviceToDevice, st));
     else CK(cudaMemsetAsync(bbar, 0, 6 * B * sizeof(double), st));
-    // forward: a checkpoint every C steps, then the final state
-    for (int sgi = 0; sgi < n_seg; ++sgi) {
-        const int k0 = sgi * C, n = std::min(C, K - k0);
-        if ((rc = get_state_full(sim, ck_xv + nxv * sgi, ck_lo + nxv * sgi, ck_b + 6ll * B * sgi, st))) return rc;
-        if (u) CK(slice_u(us, u, B, K, k0, n, st));
-        if ((rc = sph_step(sim, u ? us : nullptr, n, nullptr, nullptr, stream))) return rc;
-    }
-    if ((rc = get_state_full(sim, fin_xv, fin_lo, fin_b, st))) return rc;
     AdjDev A{};
     A.rhobar = rhob;
     A.bbar = bbar;
@@ -810,53 +942,124 @@ int sph_vjp(sph_sim* sim, const double* u, int32_t K, const double* ybar, const 
     A.part = part;
     A.max_tiles = sim->max_tiles;
     A.ybar = ybar;
-    int32_t ns = 0;
-    {   // samples of the forward call
-        long long first = (step0 + oe - 1) / oe, last = (step0 + K + oe - 1) / oe;
-        ns = (int32_t)(last - first);
-    }
-    A.ybar_stride = (long long)ns * SPH_NY;
+    const long long first_row = (step0 + oe - 1) / oe;
+    A.ybar_stride = ((step0 + K + oe - 1) / oe - first_row) * SPH_NY;  // the samples of the forward call
     A.ubar = ubar;
     A.ubar_stride = 3ll * K;
-    const SimDev S = sim->dev(code);
     float4* cur = adj0;
     float4* nxt = adj1;
-    for (int sgi = n_seg - 1; sgi >= 0; --sgi) {
-        const int k0 = sgi * C, n1 = std::min(K, k0 + C);
-        // recompute the states of the segment from its checkpoint
-        sim->host_step = step0 + k0;
-        CK(launch_set_step(sim->d_run, sim->host_step, st));
-        if ((rc = set_state_full(sim, ck_xv + nxv * sgi, ck_lo + nxv * sgi, ck_b + 6ll * B * sgi, st))) return rc;
-        for (int k = k0; k < n1; ++k) {
-            if ((rc = get_state_full(sim, seg_xv + nxv * (k - k0), seg_lo + nxv * (k - k0), seg_b + 6ll * B * (k - k0),
-                                     st)))
-                return rc;
-            if (k + 1 < n1) {
-                if (u) CK(slice_u(us, u, B, K, k, 1, st));
-                if ((rc = sph_step(sim, u ? us : nullptr, 1, nullptr, nullptr, stream))) return rc;
-            }
+    auto at = [&](auto* p, int i) { return (std::remove_const_t<std::remove_pointer_t<decltype(p)>>*)((char*)p + rec.step_bytes * i); };
+    // the records of a group whose first step is k0
+    auto begin = [&](int k0, cudaStream_t q) {
+        R = RecordDev{};
+        R.first = sim->dev(code);
+        R.buf0 = (int)((step0 + k0) & 1);
+        R.seg = C;
+        rec.place(recs, R);
+        R.step_bytes = rec.step_bytes;
+        R.count_stride = rec.count_stride();
+        R.first.count[R.buf0] = counts + rec.count_stride() * L;
+        R.first.body = bodies;
+        R.next_count = counts;
+        R.flags = &sim->d_body->flags;
+        R.flags_stride = (int)(sizeof(BodyDev) / sizeof(int));
+        CK(cudaMemsetAsync(counts, 0, 2 * rec.count_stride() * L * sizeof(int), q));
+        CK(cudaMemsetAsync(lane.body, 0, B * sizeof(BodyDev), q));
+        return (int)SPH_OK;
+    };
+    // runs segment s again from its checkpoint; its first step is step i0 of the group
+    auto record = [&](int s, int i0, cudaStream_t q) {
+        const int k0 = s * C, n = std::min(C, K - k0);
+        SimDev cur = lane;  // reads the state before the step, writes the state after it into the step's record
+        int buf = (R.buf0 + i0) & 1;
+        cur.pv[buf] = at(R.first.pv[R.buf0], i0);
+        cur.lo[buf] = at(R.first.lo[R.buf0], i0);
+        cur.pid[buf] = at(R.first.pid[R.buf0], i0);
+        cur.count[buf] = R.first.count[R.buf0] + rec.count_stride() * i0;
+        CK(launch_set_step(lane.run, step0 + k0, q));
+        CK(launch_set_body(cur, ck_b + 6ll * B * s, buf, q));
+        CK(launch_bin_flat(cur, ck + 2 * nxv * s, ck + 2 * nxv * s + nxv, sim->d_part_tank, N, buf, q));
+        CK(launch_set_run(lane.run, run_of(k0), q));
+        EvalOut E{};
+        for (int i = i0; i < i0 + n; ++i, buf ^= 1) {
+            cur.pv[buf ^ 1] = at(R.next_pv, i);
+            cur.lo[buf ^ 1] = at(R.next_lo, i);
+            cur.pid[buf ^ 1] = at(R.next_pid, i);
+            cur.count[buf ^ 1] = counts + rec.count_stride() * i;
+            cur.brec = at(R.first.brec, i);
+            CK(launch_step(cur, E, 0, sim->tile_code, sim->n_tiles[sim->tile_code], q, sim->use_pdl, false, i > i0));
         }
-        for (int k = n1 - 1; k >= k0; --k) {
-            sim->host_step = step0 + k;
-            CK(launch_set_step(sim->d_run, sim->host_step, st));
-            if ((rc = set_state_full(sim, seg_xv + nxv * (k - k0), seg_lo + nxv * (k - k0), seg_b + 6ll * B * (k - k0),
-                                     st)))
-                return rc;
+        return (int)SPH_OK;
+    };
+    // S of the recorded step i, for its adjoint
+    auto step_of = [&](int i) {
+        const int b0 = R.buf0, b = (b0 + i) & 1;
+        SimDev s = R.first;
+        s.pv[b] = at(R.first.pv[b0], i);
+        s.lo[b] = at(R.first.lo[b0], i);
+        s.pid[b] = at(R.first.pid[b0], i);
+        s.rhoP = at(s.rhoP, i);
+        s.gpos = at(s.gpos, i);
+        s.gvel = at(s.gvel, i);
+        s.nbm = at(s.nbm, i);
+        s.nba = at(s.nba, i);
+        s.nbn = at(s.nbn, i);
+        s.srec = at(s.srec, i);
+        s.body = bodies + (size_t)B * i;
+        return s;
+    };
+    auto reverse = [&](int k0, int k1) {
+        for (int k = k1 - 1; k >= k0; --k) {
             const long long g = step0 + k;
+            const SimDev s = step_of(k - k0);
             A.k = k;
-            A.row = (g % oe == 0) ? (int)(g / oe - (step0 + oe - 1) / oe) : -1;
+            A.row = (g % oe == 0) ? (int)(g / oe - first_row) : -1;
+            A.buf = (int)(g & 1);
             A.in = cur;
             A.out = nxt;
-            CK(launch_adjoint_step(S, A, sim->n_tiles[code], st));
+            CK(launch_adjoint_body(s, A, k < K - 1, 1, st, k < k1 - 1));
+            CK(launch_adjoint_step(s, A, sim->n_tiles[code], st));
             std::swap(cur, nxt);
         }
+        return (int)SPH_OK;
+    };
+    if (beside && K > 0) {
+        CK(cudaEventRecord(sim->ev, st));  // after whatever used the records and the inputs before
+        CK(cudaStreamWaitEvent(sim->side, sim->ev, 0));
+        if ((rc = begin(0, sim->side))) return rc;
+    }
+    for (int s = 0; s < n_seg; ++s) {
+        if ((rc = save(s))) return rc;
+        if (beside) {
+            CK(cudaEventRecord(sim->ev, st));
+            CK(cudaStreamWaitEvent(sim->side, sim->ev, 0));
+        }
+        CK(launch_set_run(sim->d_run, run_of(s * C), st));
+        if ((rc = run_steps(sim, std::min(C, K - s * C), st))) return rc;
+        if (beside && (rc = record(s, s * C, sim->side))) return rc;
+    }
+    if ((rc = save(n_seg))) return rc;
+    if (beside && K > 0) {
+        CK(cudaEventRecord(sim->ev, sim->side));
+        CK(cudaStreamWaitEvent(st, sim->ev, 0));
+    }
+    for (int g = n_grp - 1; g >= 0 && K > 0; --g) {
+        const int s0 = g * per_grp, s1 = std::min(n_seg, s0 + per_grp), k0 = s0 * C, k1 = std::min(K, s1 * C);
+        if (!beside) {
+            if ((rc = begin(k0, st))) return rc;
+            for (int s = s0; s < s1; ++s)
+                if ((rc = record(s, (s - s0) * C, st))) return rc;
+        }
+        CK(launch_recorded(R, sim->d_part_tank, sim->n_cells_total, sim->n_tiles[code], k1 - k0, st));
+        if ((rc = reverse(k0, k1))) return rc;
+    }
+    if (K > 0) {  // leave the simulator at the final state, as sph_jvp does
+        CK(launch_adjoint_body(R.first, A, 1, 0, st, true));
+        CK(launch_set_step(sim->d_run, sim->host_step, st));
+        if ((rc = set_state_full(sim, ck + 2 * nxv * n_seg, ck + 2 * nxv * n_seg + nxv, ck_b + 6ll * B * n_seg, st))) return rc;
     }
     if (xvbar0) CK(cudaMemcpyAsync(xvbar0, cur, nxv * sizeof(float), cudaMemcpyDeviceToDevice, st));
     if (bodybar0) CK(cudaMemcpyAsync(bodybar0, bbar, 6 * B * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    // leave the simulator at the final state, as sph_jvp does
-    sim->host_step = step0 + K;
-    CK(launch_set_step(sim->d_run, sim->host_step, st));
-    if ((rc = set_state_full(sim, fin_xv, fin_lo, fin_b, st))) return rc;
     CK(cudaStreamSynchronize(st));  // the scratch buffers are freed on return
     return SPH_OK;
 }

@@ -205,6 +205,8 @@ constexpr int kOneLevelLoads = 8; // one-level reduction up to this many partial
 constexpr int kNbrRowBits = 32;   // candidates of one stencil row the density pass can record as a bit mask
 constexpr unsigned char kNbrNone = 255;  // neighbour count marking a particle whose rows were not recorded
 
+constexpr int kBodyRec = 6;       // r_x, r_y, theta, rdot_x, rdot_y, thetadot
+
 // Optional per-particle outputs of an evaluation pass (indexed by particle).
 struct EvalOut {
     float* rho;
@@ -247,6 +249,7 @@ struct SimDev {
     float4* tgh;                  // per ghost (d r_g, d v_g)
     TilePartial* tpartials;       // tangent partials per tile / group
     TilePartial* tgpartials;
+    double* brec;                 // recorded run: per tank kBodyRec doubles, the body before the step (else NULL)
     int B;
     int n_tiles;
 };

@@ -36,9 +36,10 @@ namespace sph {
 // ---------------------------------------------------------------------------
 // TAN: also the forward-mode tangent d rho (Eq. 14 differentiated along the
 // tangent of positions and of the body pose) and d(P / rho^2).
-template <int TX, int TY, bool TAN>
-__global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY>::DENSITY_MIN_CTAS)
-    density_kernel(SimDev S, EvalOut E, int eval, int chained)
+// RECORDED: the pass over a recorded state, in buffer rbuf of S (nothing else
+// of the buffers is touched, and no dependency is waited for).
+template <int TX, int TY, bool TAN, bool RECORDED>
+__device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, int eval, int chained, int rbuf)
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, false, TAN> sm;
@@ -51,9 +52,11 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
     // that pass completed before the body update passed its dependency, so
     // they run before this pass's dependency on the body update (through L2:
     // the staging loads bypass L1); the ghosts wait for the body
-    const bool early = !TAN && chained;
+    const bool early = !TAN && !RECORDED && chained;
     int buf;
-    if (early) {
+    if (RECORDED) {
+        buf = rbuf;
+    } else if (early) {
         buf = __ldcg(&S.run->next_buf);
     } else {
         pdl_wait();
@@ -62,10 +65,11 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
     const int nbuf = buf ^ 1;
 
     // clear the other buffer's counts of the own cells (it is re-filled by the force pass)
-    for (int c = threadIdx.x; c < TX * TY; c += blockDim.x) {
-        int ix = cx0 + c % TX, iy = cy0 + c / TX;
-        if (ix < T.G && iy < T.G) S.count[nbuf][T.cell_base + iy * T.G + ix] = 0;
-    }
+    if (!RECORDED)
+        for (int c = threadIdx.x; c < TX * TY; c += blockDim.x) {
+            int ix = cx0 + c % TX, iy = cy0 + c / TX;
+            if (ix < T.G && iy < T.G) S.count[nbuf][T.cell_base + iy * T.G + ix] = 0;
+        }
     const bool staged = stage_tile<TX, TY, false, TAN>(S, T, buf, cx0, cy0, sm);
     save_stage(sm, staged, stage_record<TX, TY>(S, blockIdx.x));
     const int n_own = staged ? sm.own_row[TY] : 0;
@@ -168,7 +172,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
     GhostFrame fr{};
     float t_rx = 0.f, t_ry = 0.f, t_th = 0.f, t_vx = 0.f, t_vy = 0.f, t_w = 0.f;
     auto body_frame = [&]() {
-        if constexpr (!TAN) gmode = stage_ghosts<true>(S, T, b, sm, n_own, gs);
+        if constexpr (!TAN) gmode = stage_ghosts<true>(S, T, b.fc, b.fs, b.frx, b.fry, ghost_frame(b), sm, n_own, gs);
         bc = b.fc;
         bs = b.fs;
         brx = b.frx;
@@ -275,7 +279,130 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
     // the successor's CTAs may be placed once every CTA of this pass is past
     // its particle loop (or has exited): placed earlier, they would wait in
     // griddepcontrol.wait on SM slots that tiles of this pass still need
-    pdl_trigger();
+    if (!RECORDED) pdl_trigger();
+}
+
+template <int TX, int TY, bool TAN>
+__global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY>::DENSITY_MIN_CTAS)
+    density_kernel(SimDev S, EvalOut E, int eval, int chained)
+{
+    density_pass<TX, TY, TAN, false>(S, E, eval, chained, 0);
+}
+
+// ---------------------------------------------------------------------------
+// Recorded steps (the adjoint): the body records, the re-binned states and
+// the density passes of all steps of a run, each in one launch (blockIdx.y is
+// the step).  Step by step, the density passes alone took as long as the
+// forward steps; together they fill the GPU.
+// ---------------------------------------------------------------------------
+// S of step i of the run: the first step's, its own arrays moved on by i records.
+__device__ __forceinline__ SimDev recorded(const RecordDev& R, int i)
+{
+    SimDev s = R.first;
+    const int buf = (R.buf0 + i) & 1;
+    auto at = [&](auto* p) { return reinterpret_cast<decltype(p)>(reinterpret_cast<char*>(p) + (size_t)i * R.step_bytes); };
+    s.pv[buf] = at(R.first.pv[R.buf0]);
+    s.lo[buf] = at(R.first.lo[R.buf0]);
+    s.pid[buf] = at(R.first.pid[R.buf0]);
+    s.count[buf] = R.first.count[R.buf0] + (size_t)i * R.count_stride;
+    s.rhoP = at(R.first.rhoP);
+    s.gpos = at(R.first.gpos);
+    s.gvel = at(R.first.gvel);
+    s.nbm = at(R.first.nbm);
+    s.nba = at(R.first.nba);
+    s.nbn = at(R.first.nbn);
+    s.srec = at(R.first.srec);
+    s.brec = at(R.first.brec);
+    s.body = R.first.body + (size_t)i * s.B;
+    return s;
+}
+
+// The body record of a state (what set_body_kernel gives for it).
+__device__ void write_body(BodyDev& b, const TankDev& T, const double* s, int buf)
+{
+    b.r[0] = s[0];
+    b.r[1] = s[1];
+    b.th = s[2];
+    b.v[0] = s[3];
+    b.v[1] = s[4];
+    b.w = s[5];
+    sincos(b.th, &b.s, &b.c);
+    b.anchor[buf][0] = s[0];
+    b.anchor[buf][1] = s[1];
+    b.tau_c = 0.0;
+    b.done = 0;
+    for (int q = 0; q < 5; ++q) b.acc[q] = 0ull;
+    b.dc = df_split(b.c);
+    b.ds = df_split(b.s);
+    b.drx = df_split(b.r[0]);
+    b.dry = df_split(b.r[1]);
+    b.fvx = (float)b.v[0];
+    b.fvy = (float)b.v[1];
+    b.fw = (float)b.w;
+    b.fc = (float)b.c;
+    b.fs = (float)b.s;
+    b.frx = (float)b.r[0];
+    b.fry = (float)b.r[1];
+    b.fo_next[0] = (float)(b.r[0] - T.W);
+    b.fo_next[1] = (float)(b.r[1] - T.W);
+}
+
+__global__ void rec_body_kernel(RecordDev R)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= R.first.B) return;
+    const SimDev S = recorded(R, blockIdx.y);
+    S.body[t].flags = 0;
+    write_body(S.body[t], S.tank[t], S.brec + t * kBodyRec, (R.buf0 + (int)blockIdx.y) & 1);
+}
+
+// Cell of a position in the grid of buffer buf, and the flags of a position
+// off the grid or the cover disc.
+__device__ __forceinline__ int bin_cell(const TankDev& T, const BodyDev& b, int buf, float x, float y, int* flags)
+{
+    const float ox = (float)(b.anchor[buf][0] - T.W), oy = (float)(b.anchor[buf][1] - T.W);
+    bool out = false;
+    const int cx = cell_coord(x, ox, T.inv_cell, T.G, &out), cy = cell_coord(y, oy, T.inv_cell, T.G, &out);
+    const float ex = x - (ox + T.Wf), ey = y - (oy + T.Wf);
+    if (out || fmaf(ex, ex, ey * ey) > T.cover2) *flags |= SPH_FLAG_ESCAPED;
+    return T.cell_base + cy * T.G + cx;
+}
+
+// One warp per cell of the grid that the step before left (anchored where the
+// body was then): its particles into the grid anchored at the body's position,
+// the one that a call on this state bins into.
+__global__ void rec_bin_kernel(RecordDev R, const int* __restrict__ part_tank, int n_cells_total)
+{
+    const int cell = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), i = blockIdx.y;
+    const int lane = threadIdx.x & 31;
+    if (cell >= n_cells_total || i % R.seg == 0) return;
+    const size_t off = (size_t)(i - 1) * R.step_bytes;
+    const int n = min(max(R.next_count[(size_t)(i - 1) * R.count_stride + cell], 0), kCap);
+    if (lane >= n) return;
+    const SimDev S = recorded(R, i);
+    const int buf = (R.buf0 + i) & 1, gs = cell * kCap + lane;
+    auto from = [&](auto* p) { return ((decltype(p))((const char*)p + off))[gs]; };
+    const int id = from(R.next_pid);
+    const float4 p = from(R.next_pv), lo = from(R.next_lo);
+    const int t = part_tank[id];
+    int flags = 0;
+    const int c = bin_cell(S.tank[t], S.body[t], buf, p.x, p.y, &flags);
+    const int slot = atomicAdd(&S.count[buf][c], 1);
+    if ((unsigned)slot < (unsigned)kCap) {
+        S.pv[buf][c * kCap + slot] = p;
+        S.lo[buf][c * kCap + slot] = lo;
+        S.pid[buf][c * kCap + slot] = id;
+    } else {
+        flags |= SPH_FLAG_CELL_FULL;
+    }
+    if (flags) atomicOr(R.flags + t * R.flags_stride, flags);
+}
+
+template <int TX, int TY>
+__global__ void __launch_bounds__(Shape<TX, TY>::THREADS, Shape<TX, TY>::DENSITY_MIN_CTAS) rec_density_kernel(RecordDev R)
+{
+    const SimDev S = recorded(R, blockIdx.y);
+    density_pass<TX, TY, false, true>(S, EvalOut{}, 0, 0, (R.buf0 + (int)blockIdx.y) & 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -695,8 +822,9 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
         const int n_own = sm.own_row[TY];
         own = n_own;
         int gmode = kGhostsGlobal;  // the tangent variant visits the ghosts through global memory
-        if constexpr (!TAN) gmode = n_own > 0 ? stage_ghosts<false>(S, T, b, sm, n_own, gs) : kGhostsNone;
         const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry;
+        if constexpr (!TAN)
+            gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs) : kGhostsNone;
         const float ox = b.fo_next[0], oy = b.fo_next[1];  // origin of the next grid
         const float mm = T.m * T.m;
         float wfx = 0.f, wfy = 0.f, wt = 0.f, cxs = 0.f, cys = 0.f;
@@ -1049,6 +1177,7 @@ __global__ void __launch_bounds__(32 * kBodyWarps) body_kernel(SimDev S, EvalOut
         }
         if (y && lane < 6) y[lane] = pick(lane, 0, rx, ry, th, vx, vy, w);
     }
+    if (S.brec && lane < kBodyRec) S.brec[tank * kBodyRec + lane] = pre;  // the state before the step, for the adjoint
     const double tau = ut + (ctrl_on ? tau_c : 0.0);
     // output l = A + B F_which: 0..5 r', theta', rdot', thetadot'; 6, 7 r' - W
     // (the origin of the next grid); in an evaluation 0..5 are F_b, T_b and
@@ -1170,16 +1299,10 @@ __global__ void bin_flat_kernel(SimDev S, const float4* __restrict__ xv, const f
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int t = part_tank[i];
-    const TankDev& T = S.tank[t];
-    const BodyDev& b = S.body[t];
     const float4 p = xv[i];
-    const float ox = (float)(b.anchor[buf][0] - T.W), oy = (float)(b.anchor[buf][1] - T.W);
-    bool out = false;
-    const int cx = cell_coord(p.x, ox, T.inv_cell, T.G, &out), cy = cell_coord(p.y, oy, T.inv_cell, T.G, &out);
-    const float ex = p.x - (ox + T.Wf), ey = p.y - (oy + T.Wf);
-    int flags = (out || fmaf(ex, ex, ey * ey) > T.cover2) ? SPH_FLAG_ESCAPED : 0;
+    int flags = 0;
+    const int cell = bin_cell(S.tank[t], S.body[t], buf, p.x, p.y, &flags);
     if (!(isfinite(p.x) && isfinite(p.y) && isfinite(p.z) && isfinite(p.w))) flags |= SPH_FLAG_NAN;
-    const int cell = T.cell_base + cy * T.G + cx;
     const int slot = atomicAdd(&S.count[buf][cell], 1);
     if ((unsigned)slot < (unsigned)kCap) {
         S.pv[buf][cell * kCap + slot] = p;
@@ -1196,34 +1319,7 @@ __global__ void set_body_kernel(SimDev S, const double* __restrict__ body, int b
 {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= S.B) return;
-    BodyDev& b = S.body[t];
-    const TankDev& T = S.tank[t];
-    const double* s = body + 6 * t;
-    b.r[0] = s[0];
-    b.r[1] = s[1];
-    b.th = s[2];
-    b.v[0] = s[3];
-    b.v[1] = s[4];
-    b.w = s[5];
-    sincos(b.th, &b.s, &b.c);
-    b.anchor[buf][0] = s[0];
-    b.anchor[buf][1] = s[1];
-    b.tau_c = 0.0;
-    b.done = 0;
-    for (int q = 0; q < 5; ++q) b.acc[q] = 0ull;
-    b.dc = df_split(b.c);
-    b.ds = df_split(b.s);
-    b.drx = df_split(b.r[0]);
-    b.dry = df_split(b.r[1]);
-    b.fvx = (float)b.v[0];
-    b.fvy = (float)b.v[1];
-    b.fw = (float)b.w;
-    b.fc = (float)b.c;
-    b.fs = (float)b.s;
-    b.frx = (float)b.r[0];
-    b.fry = (float)b.r[1];
-    b.fo_next[0] = (float)(b.r[0] - T.W);
-    b.fo_next[1] = (float)(b.r[1] - T.W);
+    write_body(S.body[t], S.tank[t], body + 6 * t, buf);
 }
 
 __global__ void get_body_kernel(SimDev S, double* __restrict__ body)
@@ -1326,22 +1422,6 @@ __global__ void set_run_kernel(RunDev* run, RunDev desc)
 // ---------------------------------------------------------------------------
 // Host-side launchers
 // ---------------------------------------------------------------------------
-template <typename... KArgs, typename... Args>
-static cudaError_t launch(void (*k)(KArgs...), int grid, int block, cudaStream_t st, bool pdl, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = pdl ? at : nullptr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 template <int TX, int TY>
 static cudaError_t launch_tile_phase(const SimDev& S, const EvalOut& E, int eval, int n_tiles, int phase,
                                      cudaStream_t st, bool pdl, bool tan, bool chained)
@@ -1406,6 +1486,16 @@ cudaError_t launch_step(const SimDev& S, const EvalOut& E, int eval, int tile_co
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+cudaError_t launch_recorded(const RecordDev& R, const int* part_tank, int n_cells_total, int n_tiles, int steps,
+                            cudaStream_t st)
+{
+    using Sh = Shape<4, 4>;
+    rec_body_kernel<<<dim3((R.first.B + 127) / 128, steps), 128, 0, st>>>(R);
+    rec_bin_kernel<<<dim3((n_cells_total + 7) / 8, steps), 256, 0, st>>>(R, part_tank, n_cells_total);
+    rec_density_kernel<4, 4><<<dim3(n_tiles, steps), Sh::THREADS, 0, st>>>(R);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_bin_flat(const SimDev& S, const float* xv, const float* lo, const int* part_tank, int n, int buf,

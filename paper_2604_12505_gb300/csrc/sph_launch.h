@@ -6,6 +6,23 @@
 
 namespace sph {
 
+// Launch with or without programmatic stream serialization.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch(void (*k)(KArgs...), int grid, int block, cudaStream_t st, bool pdl, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = 0;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = pdl ? at : nullptr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 void tile_dims(int code, int* tx, int* ty);
 // Bytes of the per-tile staging records for the tile counts of every shape
 // (n_tiles indexed by tile code 1..SPH_TILE_COUNT).
@@ -38,9 +55,28 @@ cudaError_t launch_tangent_state(const SimDev& S, const float* txv_in, float* tx
                                  double* tb_out, int n_cells_total, int buf, cudaStream_t st);
 cudaError_t launch_set_run(RunDev* run, const RunDev& desc, cudaStream_t st);
 
-// Reverse-mode step (sph_adjoint.cu).  Adjoint arrays are indexed by particle
-// index (the order of sph_get_state); body adjoints are (r_x, r_y, theta,
-// rdot_x, rdot_y, thetadot).
+// Recorded steps: their records lie step_bytes apart, their counts
+// count_stride integers.  first: the SimDev of the first step, its arrays (of
+// buffer buf0: the state binned at the body's position) in the first record.
+// next_*: the state after the first step in the grid that the step left, in
+// the first record (the state after step i, i records on).  Every `seg`th step
+// starts a run: its state is already binned.
+struct RecordDev {
+    SimDev first;
+    int buf0, seg;
+    size_t step_bytes, count_stride;
+    const float4 *next_pv, *next_lo;
+    const int *next_pid, *next_count;
+    int* flags;              // health flags of the tanks
+    int flags_stride;        // integers between them
+};
+// The body records, re-binned states and density passes (4x4 tiles) of `steps` recorded steps.
+cudaError_t launch_recorded(const RecordDev& R, const int* part_tank, int n_cells_total, int n_tiles, int steps,
+                            cudaStream_t st);
+
+// Reverse-mode step (sph_adjoint.cu) over a recorded step: S points at its
+// records (launch_recorded), buf is the buffer of its state.  Adjoint arrays are indexed by particle index (the order of sph_get_state); body
+// adjoints are (r_x, r_y, theta, rdot_x, rdot_y, thetadot).
 struct AdjDev {
     const float4* in;        // [N] adjoint of (x, v) after the step
     float4* out;             // [N] adjoint of (x, v) before the step
@@ -54,10 +90,16 @@ struct AdjDev {
     long long ybar_stride;   // doubles between tanks
     double* ubar;            // [B, K, 3] input adjoints (NULL: not written)
     long long ubar_stride;
+    int buf;                 // buffer of the state before the step
     int k;                   // step index within the call
     int row;                 // sample row of this step, -1: not sampled
 };
 int adjoint_tile_code();
+// The body's part around a step: post finishes the step just reversed (its
+// tile partials), pre begins step A.k (bbar, the samples and u of the step).
+// pdl: the previous launch on st is a reverse step's too (the kernels stage
+// from the records before they wait for it).
+cudaError_t launch_adjoint_body(const SimDev& S, const AdjDev& A, int post, int pre, cudaStream_t st, bool pdl);
 cudaError_t launch_adjoint_step(const SimDev& S, const AdjDev& A, int n_tiles, cudaStream_t st);
 cudaError_t launch_set_step(RunDev* run, long long step, cudaStream_t st);
 

@@ -424,10 +424,12 @@ enum { kGhostsNone = 0, kGhostsStaged = 1, kGhostsGlobal = 2 };
 // stores them to S.gpos / S.gvel for the force pass and the adjoint;
 // otherwise loads them from there.  Returns (uniformly) kGhostsNone when no
 // own particle reaches a ghost, kGhostsGlobal when the box does not fit
-// (the caller then visits the ghosts through global memory).
+// (the caller then visits the ghosts through global memory).  (bc, bs, brx,
+// bry): the body frame that selects ghost cells; fr: the frame of Eq. 21 (FILL).
 template <bool FILL, int TX, int TY, bool RHO, bool TAN>
-__device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, const BodyDev& b, const Stage<TX, TY, RHO, TAN>& sm,
-                            int n_own, GhostStage<true>& gs)
+__device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, float bc, float bs, float brx, float bry,
+                                            const GhostFrame& fr, const Stage<TX, TY, RHO, TAN>& sm, int n_own,
+                                            GhostStage<true>& gs)
 {
     if (threadIdx.x == 0) {
         gs.box[0] = INT_MAX;
@@ -436,7 +438,6 @@ __device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, c
         gs.box[3] = INT_MIN;
     }
     __syncthreads();
-    const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry;
     int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
     for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
         const float4 pi = sm.pv[own_index(t, sm)];
@@ -481,7 +482,6 @@ __device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, c
     __syncthreads();
     const int total = gs.pre[nr];
     if (total > kGhostMax) return kGhostsGlobal;
-    const GhostFrame fr = ghost_frame(b);
     for (int s = threadIdx.x; s < total; s += blockDim.x) {
         int r = 0;
         while (s >= gs.pre[r + 1]) ++r;
