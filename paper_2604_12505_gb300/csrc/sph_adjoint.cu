@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_force_kernel(SimDe
         const BodyDev& b = S.body[tank];
         const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry, om = b.fw;
         const int n_own = sm.own_row[TY];
-        const int gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs) : kGhostsNone;
+        const int gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs, NoTangent{}) : kGhostsNone;
         pdl_wait();  // the adjoint of the state after the step, the body's part
         pdl_trigger();
         waited = true;
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(Sim
         const BodyDev& b = S.body[tank];
         const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry;
         const int n_own = sm.own_row[TY];
-        const int gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs) : kGhostsNone;
+        const int gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs, NoTangent{}) : kGhostsNone;
         pdl_wait();  // the density adjoints
         pdl_trigger();
         waited = true;

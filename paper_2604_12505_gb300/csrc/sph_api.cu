@@ -238,7 +238,6 @@ void free_sim(sph_sim* s)
     cudaFree(s->S.tgh);
     cudaFree(s->S.tpartials);
     cudaFree(s->S.tgpartials);
-    cudaFree(s->S.gdone);
     cudaFree((void*)s->S.gB);
     cudaFree((void*)s->S.gstart);
     cudaFree(s->S.gpos);
@@ -457,7 +456,6 @@ int create_impl(const sph_params* p, int B, cudaStream_t st, sph_sim** out)
         rc |= dalloc(&s->S.nba, 3 * nn);
         rc |= dalloc(&s->S.nbn, nn);
     }
-    rc |= dalloc(&s->S.gdone, max_groups);
     rc |= dalloc(&s->S.srec, stage_record_bytes(s->n_tiles));
     float4* gB_d;
     int* gstart_d;
@@ -488,7 +486,6 @@ int create_impl(const sph_params* p, int B, cudaStream_t st, sph_sim** out)
     CKF(cudaMemcpy(s->d_tank, td.data(), B * sizeof(TankDev), cudaMemcpyHostToDevice));
     CKF(cudaMemset(s->d_body, 0, B * sizeof(BodyDev)));
     CKF(cudaMemset(s->d_run, 0, sizeof(RunDev)));
-    CKF(cudaMemset(s->S.gdone, 0, max_groups * sizeof(unsigned int)));
     for (int code = 1; code <= SPH_TILE_COUNT; ++code) {
         CKF(cudaMemcpy(s->d_tiles[code], tiles[code].data(), tiles[code].size() * sizeof(int4), cudaMemcpyHostToDevice));
         CKF(cudaMemcpy(s->d_tile_first[code], first[code].data(), first[code].size() * sizeof(int), cudaMemcpyHostToDevice));
@@ -759,7 +756,7 @@ int sph_jvp(sph_sim* sim, const double* u, const double* du, const float* dxv0, 
     CK(launch_set_run(sim->d_run, d, st));
     EvalOut E{};
     for (int i = 0; i < K; ++i) {
-        cudaError_t e = launch_step(S, E, 0, code, sim->n_tiles[code], st, sim->use_pdl, true);
+        cudaError_t e = launch_step(S, E, 0, code, sim->n_tiles[code], st, sim->use_pdl, true, i > 0);
         if (e != cudaSuccess) return fail(SPH_E_CUDA, std::string("sph_jvp launch: ") + cudaGetErrorString(e));
     }
     sim->host_step += K;

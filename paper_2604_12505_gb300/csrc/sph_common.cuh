@@ -81,9 +81,8 @@ struct BodyDev {
     // fluid force, torque and particle-position sums of the current force
     // pass as 64-bit fixed point (units of 2^-32, two's complement): the
     // tiles add them with integer atomics, whose sum does not depend on the
-    // order of the additions, and the tank's last tile reads and clears them
+    // order of the additions, and the body kernel reads and clears them
     unsigned long long acc[5];    // F_x, F_y, T, sum x, sum y
-    unsigned int done;            // tiles (reduction groups in the tangent variant) finished in the current force pass
     int flags;                    // SPH_FLAG_* bits
 };
 // the body update stores these fields by lane (consecutive fields of one type)
@@ -234,7 +233,6 @@ struct SimDev {
     const int* group_first;       // per tank: first reduction group (size B + 1)
     TilePartial* partials;        // per tile
     TilePartial* gpartials;       // per group of kTileGroup tiles
-    unsigned int* gdone;          // per group: tiles finished in the current force pass
     const float4* gB;             // body-frame ghost positions as two-float (x_hi, x_lo, y_hi, y_lo), sorted by ghost cell
     const int* gstart;            // per tank (G*G + 1) ghost-cell starts (global ghost index)
     float4* gpos;                 // per step: (hi_x, hi_y, lo_x, lo_y) world position, written by the density pass

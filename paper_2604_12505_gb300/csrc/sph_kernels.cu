@@ -43,7 +43,7 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, false, TAN> sm;
-    __shared__ GhostStage<!TAN> gs;
+    __shared__ GhostStage<true, TAN> gs;
     const int4 td = S.tiles[blockIdx.x];
     const TankDev T = S.tank[td.x];  // by value: the constants live in registers
     const int cx0 = td.y, cy0 = td.z;
@@ -52,7 +52,7 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
     // that pass completed before the body update passed its dependency, so
     // they run before this pass's dependency on the body update (through L2:
     // the staging loads bypass L1); the ghosts wait for the body
-    const bool early = !TAN && !RECORDED && chained;
+    const bool early = !RECORDED && chained;
     int buf;
     if (RECORDED) {
         buf = rbuf;
@@ -167,12 +167,17 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
 
     // after the body update: the ghosts of Eqs. 14 and 21, then rho and P
     const BodyDev& b = S.body[td.x];
-    int gmode = kGhostsGlobal;  // the tangent variant visits the ghosts through global memory
+    int gmode = kGhostsNone;
     float bc = 0.f, bs = 0.f, brx = 0.f, bry = 0.f, fw = 0.f;
     GhostFrame fr{};
     float t_rx = 0.f, t_ry = 0.f, t_th = 0.f, t_vx = 0.f, t_vy = 0.f, t_w = 0.f;
+    // d r_g = d r + d theta z x arm, d v_g likewise (Eq. 21)
+    auto ghost_tangent = [&](const float4& gv) {
+        const float armx = gv.z, army = gv.w;
+        return make_float4(t_rx - t_th * army, t_ry + t_th * armx, t_vx - t_w * army - fw * t_th * armx,
+                           t_vy + t_w * armx - fw * t_th * army);
+    };
     auto body_frame = [&]() {
-        if constexpr (!TAN) gmode = stage_ghosts<true>(S, T, b.fc, b.fs, b.frx, b.fry, ghost_frame(b), sm, n_own, gs);
         bc = b.fc;
         bs = b.fs;
         brx = b.frx;
@@ -187,6 +192,7 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
             t_vy = b.ftv[1];
             t_w = b.ftw;
         }
+        gmode = stage_ghosts<true>(S, T, bc, bs, brx, bry, fr, sm, n_own, gs, ghost_tangent);
     };
     auto ghost_part = [&](int t, float Sf, float Df, float dRf) {
         const int e = own_index(t, sm);
@@ -216,9 +222,10 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
             }
         };
         if (gmode == kGhostsStaged) {
-            if constexpr (!TAN)
-                for_staged_ghosts(T, gs, pi.x, pi.y, bc, bs, brx, bry, T.clip,
-                                  [&](int, int sg) { ghost(gs.gp[sg], gs.gv[sg], 0.f, 0.f); });
+            for_staged_ghosts(T, gs, pi.x, pi.y, bc, bs, brx, bry, T.clip, [&](int, int sg) {
+                if constexpr (TAN) ghost(gs.gp[sg], gs.gv[sg], gs.tg[sg].x, gs.tg[sg].y);
+                else ghost(gs.gp[sg], gs.gv[sg], 0.f, 0.f);
+            });
         } else if (gmode == kGhostsGlobal) {
             // Eq. 21 per visit, stored for the force pass and the adjoint
             for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry, [&](int g) {
@@ -227,12 +234,11 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
                 S.gpos[g] = gp;
                 S.gvel[g] = gv;
                 float tgx = 0.f, tgy = 0.f;
-                if constexpr (TAN) {  // d r_g = d r + d theta z x arm, d v_g likewise (Eq. 21)
-                    const float armx = gv.z, army = gv.w;
-                    tgx = t_rx - t_th * army;
-                    tgy = t_ry + t_th * armx;
-                    S.tgh[g] = make_float4(tgx, tgy, t_vx - t_w * army - fw * t_th * armx,
-                                           t_vy + t_w * armx - fw * t_th * army);
+                if constexpr (TAN) {
+                    const float4 tg = ghost_tangent(gv);
+                    tgx = tg.x;
+                    tgy = tg.y;
+                    S.tgh[g] = tg;
                 }
                 ghost(gp, gv, tgx, tgy);
             });
@@ -255,27 +261,19 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
         }
     };
 
-    if constexpr (TAN) {
-        body_frame();
-        for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
-            float Sf, Df, dRf;
-            fluid_part(t, Sf, Df, dRf);
-            ghost_part(t, Sf, Df, dRf);
-        }
-    } else {
-        // the fluid sums wait in the staging scratch (key_in, pid_in: free
-        // once the tile is staged), each read back by the thread that wrote it
-        for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
-            float Sf, Df, dRf;
-            fluid_part(t, Sf, Df, dRf);
-            sm.key_in[t] = __float_as_uint(Sf);
-            sm.pid_in[t] = __float_as_int(Df);
-        }
-        if (early) pdl_wait();
-        body_frame();
-        for (int t = threadIdx.x; t < n_own; t += blockDim.x)
-            ghost_part(t, __uint_as_float(sm.key_in[t]), __int_as_float(sm.pid_in[t]), 0.f);
+    // the fluid sums wait in the staging scratch (key_in, pid_in: free once the
+    // tile is staged), each read back by the thread that wrote it
+    for (int t = threadIdx.x; t < n_own; t += blockDim.x) {
+        float Sf, Df, dRf;
+        fluid_part(t, Sf, Df, dRf);
+        sm.key_in[t] = __float_as_uint(Sf);
+        sm.pid_in[t] = __float_as_int(Df);
+        if constexpr (TAN) sm.tsum[t] = dRf;
     }
+    if (early) pdl_wait();
+    body_frame();
+    for (int t = threadIdx.x; t < n_own; t += blockDim.x)
+        ghost_part(t, __uint_as_float(sm.key_in[t]), __int_as_float(sm.pid_in[t]), TAN ? sm.tsum[TAN ? t : 0] : 0.f);
     // the successor's CTAs may be placed once every CTA of this pass is past
     // its particle loop (or has exited): placed earlier, they would wait in
     // griddepcontrol.wait on SM slots that tiles of this pass still need
@@ -330,7 +328,6 @@ __device__ void write_body(BodyDev& b, const TankDev& T, const double* s, int bu
     b.anchor[buf][0] = s[0];
     b.anchor[buf][1] = s[1];
     b.tau_c = 0.0;
-    b.done = 0;
     for (int q = 0; q < 5; ++q) b.acc[q] = 0ull;
     b.dc = df_split(b.c);
     b.ds = df_split(b.s);
@@ -516,15 +513,14 @@ __device__ Red warp_reduce_partials(const TilePartial* P, int p0, int p1, bool c
 }
 
 // ---------------------------------------------------------------------------
-// Body update by the last CTA of a tank (Eq. 20, Eq. 28, outputs)
+// Body update of the tangent variant (Eq. 20, Eq. 28, outputs)
 // ---------------------------------------------------------------------------
-// Runs in warp 0 of the CTA that finished the tank's reduction, with the
-// reduced fluid force, torque and position sums as FP64 totals.  The FP64 pipe
-// of this GPU is narrow and every global access on the serial path costs an
-// L2 round trip, so warp 0 of every CTA loads the values the update reads
-// (finalize_preload) right after the grid dependency resolves, while the tile
-// is staged; the body is updated in registers and stored once, and the masses
-// enter as reciprocals.
+// Runs in warp 0 of the tank's block, with the reduced fluid force, torque and
+// position sums as FP64 totals.  The FP64 pipe of this GPU is narrow and every
+// global access on the serial path costs an L2 round trip, so the values the
+// update reads are loaded (finalize_preload) before the grid dependency; the
+// body is updated in registers and stored once, and the masses enter as
+// reciprocals.
 //
 // finalize_preload: lane l of warp 0 holds one value (as a double or as the
 // bits of one): the body's r, theta, rdot, thetadot, cos, sin (l < 8, the
@@ -762,7 +758,6 @@ __device__ void tank_finalize(const SimDev& S, const TankDev& T, int tank, int e
         if (lane == 0) bp->pairs += add_pairs;
     }
     if (lane != 0) return;
-    bp->done = 0;
     if (S.B == 1) {  // the only tank: its step is the pass's (visible when the kernel completes)
         if (!eval) run->step = step + 1;
         return;
@@ -793,13 +788,11 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, true, TAN> sm;
-    __shared__ GhostStage<!TAN> gs;
+    __shared__ GhostStage<true> gs;
     __shared__ Red scratch[32];
-    __shared__ int is_last;
     // the successor is the body update, a few warps: placed at once, it
-    // prepares its update during this pass (the tangent variant's successor
-    // is the next density pass, placed after the loop as there)
-    if constexpr (!TAN) pdl_trigger();
+    // prepares its update during this pass
+    pdl_trigger();
     const int4 td = S.tiles[blockIdx.x];
     const int tank = td.x;
     const TankDev T = S.tank[tank];  // by value: the constants live in registers
@@ -821,10 +814,9 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
         const BodyDev& b = S.body[tank];
         const int n_own = sm.own_row[TY];
         own = n_own;
-        int gmode = kGhostsGlobal;  // the tangent variant visits the ghosts through global memory
         const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry;
-        if constexpr (!TAN)
-            gmode = n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs) : kGhostsNone;
+        const int gmode =
+            n_own > 0 ? stage_ghosts<false>(S, T, bc, bs, brx, bry, GhostFrame{}, sm, n_own, gs, NoTangent{}) : kGhostsNone;
         const float ox = b.fo_next[0], oy = b.fo_next[1];  // origin of the next grid
         const float mm = T.m * T.m;
         float wfx = 0.f, wfy = 0.f, wt = 0.f, cxs = 0.f, cys = 0.f;
@@ -897,8 +889,9 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
             // P_i / rho_i^2 in Eq. 16: clamped at zero when the wall only pushes
             const float qg = T.gp_clamp ? fmaxf(ri.y, 0.f) : ri.y;
             // one ghost: gp its world position (x_hi, y_hi, x_lo, y_lo), load_gv()
-            // its (v_x, v_y, arm_x, arm_y), read only for a pair within reach
-            auto ghost = [&](int g, const float4 gp, auto&& load_gv) {
+            // its (v_x, v_y, arm_x, arm_y) and load_tg() its tangent, read only
+            // for a pair within reach
+            auto ghost = [&](const float4 gp, auto&& load_gv, auto&& load_tg) {
                 const float2 d = sep_fg(pi, li, gp);
                 const float ddx = d.x, ddy = d.y;
                 const float r2 = dist2(ddx, ddy);
@@ -921,7 +914,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
                         wfy -= fy;
                         wt -= gv.z * fy - gv.w * fx;                                     // Eq. 20 torque
                         if constexpr (TAN) {
-                            const float4 tg = __ldg(S.tgh + g);                           // (d r_g, d v_g)
+                            const float4 tg = load_tg();                                  // (d r_g, d v_g)
                             const float tdx = ti.x - tg.x, tdy = ti.y - tg.y;
                             const float rd = ddx * tdx + ddy * tdy;
                             const float tGs = -T.cdS * d * (T.h + r) * inv_r * inv_r * rd * inv_r;  // d(Gs)
@@ -949,12 +942,13 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
                 }
             };
             if (gmode == kGhostsStaged) {
-                if constexpr (!TAN)
-                    for_staged_ghosts(T, gs, pi.x, pi.y, bc, bs, brx, bry, T.hclip,
-                                      [&](int g, int sg) { ghost(g, gs.gp[sg], [&] { return gs.gv[sg]; }); });
+                for_staged_ghosts(T, gs, pi.x, pi.y, bc, bs, brx, bry, T.hclip, [&](int g, int sg) {
+                    ghost(gs.gp[sg], [&] { return gs.gv[sg]; }, [&] { return __ldcg(S.tgh + g); });
+                });
             } else if (gmode == kGhostsGlobal) {
-                for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry,
-                           [&](int g) { ghost(g, __ldg(S.gpos + g), [&] { return __ldg(S.gvel + g); }); });
+                for_ghosts(S, T, pi.x, pi.y, bc, bs, brx, bry, [&](int g) {
+                    ghost(__ldg(S.gpos + g), [&] { return __ldg(S.gvel + g); }, [&] { return __ldcg(S.tgh + g); });
+                });
             }
             wall |= (nfg > 0);
             acc.pairs += (unsigned long long)(nff + nfg);
@@ -1027,7 +1021,6 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
         tacc.cx = F2{tcxs, 0.f};
         tacc.cy = F2{tcys, 0.f};
     }
-    if constexpr (TAN) pdl_trigger();  // past the particle loop (see the density pass)
     if (flags) atomicOr(&S.body[tank].flags, flags);
     if constexpr (!TAN) {
         // The tile's sums go into the tank's fixed-point accumulators by
@@ -1050,74 +1043,67 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
         if (lane == 5 && !eval && pairs) atomicAdd(&bp->pairs, pairs);
         return;
     } else {
-        // what the body update reads, in flight during the tile's reduction
-        // (only the tank's last tile uses it)
-        double pre = 0.0;
-        if (threadIdx.x < 32) pre = finalize_preload(S, T, tank);
-        const int t0 = S.tile_tank_first[tank], t1 = S.tile_tank_first[tank + 1];
+        // the tile's partials, which the tangent's body kernel sums in fixed order
         const bool any_wall = __syncthreads_or(wall) != 0;
-        Red r = block_reduce(acc, any_wall, sample, scratch);
-        // Tangent variant: fixed-order reduction of the tile partials (the
-        // tangent's scale is the caller's, unsuited to a fixed point).  One
-        // level when the tank's last tile can fetch them with at most
-        // kOneLevelLoads loads per thread: the last tile (by a counter of
-        // finished tiles) sums them with the whole block.  Otherwise two
-        // levels: the last tile of each group of kTileGroup tiles sums the
-        // group, the last group of the tank sums the groups.
-        Red tr = block_reduce(tacc, any_wall, sample, scratch);
-        // called by all of warp 0 with the sums valid in lane 0: every lane
-        // of the body update needs them
-        auto finish = [&](const Red& rt, const Red& trt) {
-            auto all = [](F2 v) { return __shfl_sync(0xffffffffu, (double)v.hi + (double)v.lo, 0); };
-            tank_finalize(S, T, tank, eval, E, nbuf, step, sample, true, all(rt.fx), all(rt.fy), all(rt.t),
-                          all(rt.cx), all(rt.cy), rt.pairs, trt, pre);
-        };
-        if (t1 - t0 <= kOneLevelLoads * (int)blockDim.x) {
-            if (threadIdx.x == 0) {
-                store_partial(S.partials + blockIdx.x, r, any_wall ? 1 : 0);
-                store_partial(S.tpartials + blockIdx.x, tr, any_wall ? 1 : 0);
-                fence_acq_rel();
-                is_last = (atomicAdd(&S.body[tank].done, 1u) == (unsigned)(t1 - t0 - 1));
-            }
-            __syncthreads();
-            if (!is_last) return;
-            fence_acq_rel();
-            const Red rt = block_reduce_partials(S.partials, t0, t1, sample, scratch);
-            const Red trt = block_reduce_partials(S.tpartials, t0, t1, sample, scratch);
-            if (threadIdx.x < 32) finish(rt, trt);
-            return;
-        }
-        const int gi = (blockIdx.x - t0) / kTileGroup;
-        const int gt0 = t0 + gi * kTileGroup, gt1 = min(gt0 + kTileGroup, t1);
-        const int g = S.group_first[tank] + gi;
+        const Red r = block_reduce(acc, any_wall, sample, scratch);
+        const Red tr = block_reduce(tacc, any_wall, sample, scratch);
         if (threadIdx.x == 0) {
             store_partial(S.partials + blockIdx.x, r, any_wall ? 1 : 0);
             store_partial(S.tpartials + blockIdx.x, tr, any_wall ? 1 : 0);
-            fence_acq_rel();
-            is_last = (atomicAdd(&S.gdone[g], 1u) == (unsigned)(gt1 - gt0 - 1));
         }
-        __syncthreads();
-        if (!is_last || threadIdx.x >= 32) return;  // warp 0 of the group's last tile goes on
-        fence_acq_rel();
-        int wall_g;
-        r = warp_reduce_partials(S.partials, gt0, gt1, sample, &wall_g);
-        tr = warp_reduce_partials(S.tpartials, gt0, gt1, sample, &wall_g);
-        unsigned prev = 0;
-        if (threadIdx.x == 0) {
-            store_partial(S.gpartials + g, r, wall_g);
-            store_partial(S.tgpartials + g, tr, wall_g);
-            S.gdone[g] = 0;
-            fence_acq_rel();
-            prev = atomicAdd(&S.body[tank].done, 1u);
-        }
-        const unsigned n_groups = (unsigned)(S.group_first[tank + 1] - S.group_first[tank]);
-        if (__shfl_sync(0xffffffffu, prev, 0) != n_groups - 1) return;
-        fence_acq_rel();
-        int wall_t;
-        const Red rt = warp_reduce_partials(S.gpartials, S.group_first[tank], S.group_first[tank + 1], sample, &wall_t);
-        const Red trt = warp_reduce_partials(S.tgpartials, S.group_first[tank], S.group_first[tank + 1], sample, &wall_t);
-        finish(rt, trt);
     }
+}
+
+// Body and tangent update of the tangent variant after its force pass, one
+// block of a tile's threads per tank: the sums of the tile partials in fixed
+// order (the tangent's scale is the caller's, unsuited to a fixed point), one
+// level when that is at most kOneLevelLoads loads per thread, otherwise by
+// groups of kTileGroup tiles; then the update in warp 0.  A kernel of its own,
+// as in the step: in the force pass's last CTA, behind counters of finished
+// tiles, the sums and the FP64 chain sat at the end of every pass.  With the
+// ghosts staged and the density pass ahead of its dependency, as in the step:
+// 49 -> 36 us a step of the 15,532-particle tank; 256 copies of the paper's
+// spacecraft in one evaluation 620 -> 473 us.
+__global__ void __launch_bounds__(256) tan_body_kernel(SimDev S, EvalOut E, int eval)
+{
+    __shared__ Red scratch[32];
+    const int tank = blockIdx.x, warp = threadIdx.x >> 5;
+    const TankDev T = S.tank[tank];
+    double pre = 0.0;
+    if (warp == 0) pre = finalize_preload(S, T, tank);
+    const long long step = S.run->step;
+    const int nbuf = (int)(step & 1) ^ 1;
+    const bool sample = !eval && (step % T.outer_every) == 0;
+    const int t0 = S.tile_tank_first[tank], t1 = S.tile_tank_first[tank + 1];
+    pdl_wait();
+    pdl_trigger();
+    Red r, tr;
+    if (t1 - t0 <= kOneLevelLoads * (int)blockDim.x) {
+        r = block_reduce_partials(S.partials, t0, t1, sample, scratch);
+        tr = block_reduce_partials(S.tpartials, t0, t1, sample, scratch);
+        if (warp) return;
+    } else {
+        int wall;
+        const int g0 = S.group_first[tank], g1 = S.group_first[tank + 1];
+        for (int g = g0 + warp; g < g1; g += (int)(blockDim.x >> 5)) {
+            const int gt0 = t0 + (g - g0) * kTileGroup, gt1 = min(gt0 + kTileGroup, t1);
+            r = warp_reduce_partials(S.partials, gt0, gt1, sample, &wall);
+            tr = warp_reduce_partials(S.tpartials, gt0, gt1, sample, &wall);
+            if ((threadIdx.x & 31) == 0) {
+                store_partial(S.gpartials + g, r, wall);
+                store_partial(S.tgpartials + g, tr, wall);
+            }
+        }
+        __threadfence();
+        __syncthreads();
+        if (warp) return;
+        r = warp_reduce_partials(S.gpartials, g0, g1, sample, &wall);
+        tr = warp_reduce_partials(S.tgpartials, g0, g1, sample, &wall);
+    }
+    // every lane of the body update needs the sums, valid in lane 0
+    auto all = [](F2 v) { return __shfl_sync(0xffffffffu, (double)v.hi + (double)v.lo, 0); };
+    tank_finalize(S, T, tank, eval, E, nbuf, step, sample, true, all(r.fx), all(r.fy), all(r.t), all(r.cx), all(r.cy),
+                  r.pairs, tr, pre);
 }
 
 // ---------------------------------------------------------------------------
@@ -1429,8 +1415,9 @@ static cudaError_t launch_tile_phase(const SimDev& S, const EvalOut& E, int eval
     using Sh = Shape<TX, TY>;
     if (tan) {
         if constexpr (TX * TY <= 32) {  // the tangent staging of 8x8 tiles exceeds static shared memory
-            if (phase == 0) return launch(density_kernel<TX, TY, true>, n_tiles, Sh::THREADS, st, pdl, S, E, eval, 0);
-            if (phase == 2) return cudaSuccess;  // the tangent force pass updates the body itself
+            if (phase == 0)
+                return launch(density_kernel<TX, TY, true>, n_tiles, Sh::THREADS, st, pdl, S, E, eval, (pdl && chained) ? 1 : 0);
+            if (phase == 2) return launch(tan_body_kernel, S.B, Sh::THREADS, st, pdl, S, E, eval);
             return launch(force_kernel<TX, TY, true>, n_tiles, Sh::THREADS, st, pdl, S, E, eval);
         } else {
             return cudaErrorInvalidValue;
@@ -1464,7 +1451,7 @@ void tile_dims(int code, int* tx, int* ty)
     *ty = T[code - 1][1];
 }
 
-// phase 0: density pass, 1: force pass, 2: body update (none in the tangent variant)
+// phase 0: density pass, 1: force pass, 2: body update
 cudaError_t launch_phase(const SimDev& S, const EvalOut& E, int eval, int tile_code, int n_tiles, int phase,
                          cudaStream_t st, bool pdl, bool tan, bool chained)
 {

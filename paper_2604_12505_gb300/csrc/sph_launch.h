@@ -30,8 +30,7 @@ size_t stage_record_bytes(const int* n_tiles);
 // pdl: launch with programmatic stream serialization (the kernels wait on
 // their predecessor with griddepcontrol before reading its results).
 // tan: the forward-mode tangent variants (tile codes 1..4 only).
-// Phases: 0 density pass, 1 force pass, 2 body update (the tangent variant's
-// force pass updates the body itself, its phase 2 launches nothing).
+// Phases: 0 density pass, 1 force pass, 2 body update.
 // chained: this step directly follows a step of the same launch sequence
 // (its density pass is the programmatic dependent of the previous step's
 // body update), so that pass may stage the tile and sum the fluid part of

@@ -53,6 +53,7 @@ struct Stage {
     float2 rho[RHO ? Sh::MAXS : 1];
     float2 vlo[RHO ? Sh::MAXS : 1];           // low parts (vx_lo, vy_lo) of the velocities (force pass)
     float4 tpv[TAN ? Sh::MAXS : 1];           // tangent (dx, dy, dvx, dvy)
+    float tsum[(TAN && !RHO) ? Sh::MAXS : 1];  // density pass: an own particle's fluid sum of the tangent
     float2 trho[(TAN && RHO) ? Sh::MAXS : 1];  // tangent (d rho, d(P / rho^2))
 };
 
@@ -167,7 +168,7 @@ __device__ bool stage_tile(const SimDev& S, const TankDev& T, int buf, int cx0, 
             sm.vlo[d] = make_float2(lo.z, lo.w);
         }
         if constexpr (TAN) {
-            sm.tpv[d] = S.tpv[buf][gs];
+            sm.tpv[d] = __ldcg(S.tpv[buf] + gs);
             if (RHO) sm.trho[d] = S.trho[gs];
         }
         sm.pid[d] = id;
@@ -405,10 +406,11 @@ __device__ __forceinline__ void ghost_world(const GhostFrame& f, float4 gb, floa
 constexpr int kGhostMax = 256;  // staged ghosts per tile
 constexpr int kGhostDim = 16;   // staged ghost-cell rows and columns per tile
 
-template <bool ON>
+template <bool ON, bool TAN = false>
 struct GhostStage {
     float4 gp[ON ? kGhostMax : 1];                    // world position (x_hi, y_hi, x_lo, y_lo)
     float4 gv[ON ? kGhostMax : 1];                    // (v_x, v_y, arm_x, arm_y)
+    float4 tg[TAN ? kGhostMax : 1];                   // tangent (d r_g, d v_g)
     float bx[ON ? kGhostMax : 1];                     // body-frame x (a row of cells is sorted by it)
     int tab[ON ? kGhostDim : 1][kGhostDim + 1];      // ghost-cell starts of the staged cells (global index)
     int base[kGhostDim];                             // staged index of ghost g of row r: base[r] + g
@@ -426,10 +428,11 @@ enum { kGhostsNone = 0, kGhostsStaged = 1, kGhostsGlobal = 2 };
 // own particle reaches a ghost, kGhostsGlobal when the box does not fit
 // (the caller then visits the ghosts through global memory).  (bc, bs, brx,
 // bry): the body frame that selects ghost cells; fr: the frame of Eq. 21 (FILL).
-template <bool FILL, int TX, int TY, bool RHO, bool TAN>
+// tangent(gv): the tangent of a ghost (FILL and a stage that holds tangents).
+template <bool FILL, int TX, int TY, bool RHO, bool TAN, bool GTAN, class Tangent>
 __device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, float bc, float bs, float brx, float bry,
                                             const GhostFrame& fr, const Stage<TX, TY, RHO, TAN>& sm, int n_own,
-                                            GhostStage<true>& gs)
+                                            GhostStage<true, GTAN>& gs, Tangent&& tangent)
 {
     if (threadIdx.x == 0) {
         gs.box[0] = INT_MAX;
@@ -495,6 +498,7 @@ __device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, f
             gs.gv[s] = gv;
             S.gpos[g] = gp;
             S.gvel[g] = gv;
+            if constexpr (GTAN) S.tgh[g] = gs.tg[s] = tangent(gv);
         } else {
             gs.gp[s] = __ldcg(S.gpos + g);
             gs.gv[s] = __ldcg(S.gvel + g);
@@ -504,8 +508,13 @@ __device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, f
     return kGhostsStaged;
 }
 
+struct NoTangent {
+    __device__ float4 operator()(const float4&) const { return make_float4(0.f, 0.f, 0.f, 0.f); }
+};
+
 // First staged ghost in [lo, hi) whose body-frame x is not below v.
-__device__ __forceinline__ int lower_bx(const GhostStage<true>& gs, int lo, int hi, float v)
+template <class Gst>
+__device__ __forceinline__ int lower_bx(const Gst& gs, int lo, int hi, float v)
 {
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
@@ -522,8 +531,8 @@ __device__ __forceinline__ int lower_bx(const GhostStage<true>& gs, int lo, int 
 // relative 1e-3, far above the FP32 error of the body-frame coordinates, so no
 // ghost within the support is skipped.  The edge rows and columns of the
 // grid, which may hold ghosts clamped into them, are not clipped.
-template <class F>
-__device__ __forceinline__ void for_staged_ghosts(const TankDev& T, const GhostStage<true>& gs, float xi, float yi,
+template <class Gst, class F>
+__device__ __forceinline__ void for_staged_ghosts(const TankDev& T, const Gst& gs, float xi, float yi,
                                                   float bc, float bs, float brx, float bry, float clip, F&& f)
 {
     int gx, gy;
