@@ -43,11 +43,6 @@ namespace {
 constexpr int kAdjCode = 3;  // 4x4 tiles
 constexpr int kAdjTX = 4, kAdjTY = 4;
 
-__device__ __forceinline__ F2 shfl_down_f2a(F2 v, int o)
-{
-    return F2{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
-}
-
 // Fixed-order block sum of six components (compensated two-float); the
 // result is valid in thread 0.
 template <int THREADS>
@@ -58,7 +53,7 @@ __device__ void block_sum6(F2 (&v)[6])
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-        for (int c = 0; c < 6; ++c) v[c] = f2_add(v[c], shfl_down_f2a(v[c], o));
+        for (int c = 0; c < 6; ++c) v[c] = f2_add(v[c], shfl_down_f2(v[c], o));
     __syncthreads();
     if (lane == 0)
 #pragma unroll

@@ -24,6 +24,7 @@
 #include <cfloat>
 #include <climits>
 
+#include "sph_body.cuh"
 #include "sph_common.cuh"
 #include "sph_launch.h"
 #include <type_traits>
@@ -410,36 +411,6 @@ __device__ __forceinline__ F2 shfl_f2(F2 v)
     return F2{__shfl_sync(0xffffffffu, v.hi, 0), __shfl_sync(0xffffffffu, v.lo, 0)};
 }
 
-__device__ __forceinline__ F2 shfl_down_f2(F2 v, int o)
-{
-    return F2{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
-}
-
-struct Red {
-    F2 fx, fy, t, cx, cy;
-    unsigned long long pairs;
-};
-
-// Sums over a warp (result valid in lane 0).  Only the parts flagged by the
-// uniform switches are reduced.
-__device__ __forceinline__ Red warp_reduce(Red r, bool forces, bool com, int first = 16)
-{
-#pragma unroll
-    for (int o = first; o > 0; o >>= 1) {
-        if (forces) {
-            r.fx = f2_add(r.fx, shfl_down_f2(r.fx, o));
-            r.fy = f2_add(r.fy, shfl_down_f2(r.fy, o));
-            r.t = f2_add(r.t, shfl_down_f2(r.t, o));
-        }
-        if (com) {
-            r.cx = f2_add(r.cx, shfl_down_f2(r.cx, o));
-            r.cy = f2_add(r.cy, shfl_down_f2(r.cy, o));
-        }
-        r.pairs += __shfl_down_sync(0xffffffffu, r.pairs, o);
-    }
-    return r;
-}
-
 // Sums over the block (result valid in thread 0): each warp's sum, then the
 // warps' sums by a fixed shuffle tree in warp 0 (blockDim a power-of-two
 // multiple of 32).
@@ -587,15 +558,6 @@ __device__ __forceinline__ void rotate(double dth, double th_new, double& c, dou
     const double f = 1.5 - 0.5 * (c1 * c1 + s1 * s1);
     c = c1 * f;
     s = s1 * f;
-}
-
-// The value at position `lane` of the list (0 past its end): nested selects,
-// so the lanes of a warp pick different values without diverging.
-__device__ __forceinline__ double pick(int, int) { return 0.0; }
-template <class... R>
-__device__ __forceinline__ double pick(int lane, int i, double x, R... rest)
-{
-    return lane == i ? x : pick(lane, i + 1, rest...);
 }
 
 // Fx, Fy, Tq: fluid force and torque on the body (Eq. 20); Cx, Cy: sums of the
@@ -1124,8 +1086,6 @@ __global__ void __launch_bounds__(256) tan_body_kernel(SimDev S, EvalOut E, int 
 // differ from it in the last bits only.
 constexpr int kBodyWarps = 4;  // tanks per CTA
 
-__device__ __forceinline__ double sel3(int i, double a, double b, double c) { return i == 0 ? a : (i == 1 ? b : c); }
-
 __global__ void __launch_bounds__(32 * kBodyWarps) body_kernel(SimDev S, EvalOut E, int eval)
 {
     const int tank = blockIdx.x * kBodyWarps + (int)(threadIdx.x >> 5);
@@ -1138,7 +1098,7 @@ __global__ void __launch_bounds__(32 * kBodyWarps) body_kernel(SimDev S, EvalOut
     const double rx = __shfl_sync(0xffffffffu, pre, 0), ry = __shfl_sync(0xffffffffu, pre, 1);
     const double th = __shfl_sync(0xffffffffu, pre, 2), vx = __shfl_sync(0xffffffffu, pre, 3);
     const double vy = __shfl_sync(0xffffffffu, pre, 4), w = __shfl_sync(0xffffffffu, pre, 5);
-    double c = __shfl_sync(0xffffffffu, pre, 6), sn = __shfl_sync(0xffffffffu, pre, 7);
+    const double c = __shfl_sync(0xffffffffu, pre, 6), sn = __shfl_sync(0xffffffffu, pre, 7);
     double tau_c = __shfl_sync(0xffffffffu, pre, 8);
     const double ux = __shfl_sync(0xffffffffu, pre, 9), uy = __shfl_sync(0xffffffffu, pre, 10);
     const double ut = __shfl_sync(0xffffffffu, pre, 11);
@@ -1165,39 +1125,7 @@ __global__ void __launch_bounds__(32 * kBodyWarps) body_kernel(SimDev S, EvalOut
     }
     if (S.brec && lane < kBodyRec) S.brec[tank * kBodyRec + lane] = pre;  // the state before the step, for the adjoint
     const double tau = ut + (ctrl_on ? tau_c : 0.0);
-    // output l = A + B F_which: 0..5 r', theta', rdot', thetadot'; 6, 7 r' - W
-    // (the origin of the next grid); in an evaluation 0..5 are F_b, T_b and
-    // the accelerations of Eq. 20
-    const double dt = T.dt_d, im = T.inv_m_body, iJ = T.inv_J_body;
-    const int comp = lane % 3;  // F_x, F_y or T_b for lanes 0..7 (0, 1, 2, 0, 1, 2, 0, 1)
-    const int k = lane < 8 ? lane : 0;
-    double A, B;
-    if (eval) {
-        const double u3 = sel3(comp, ux, uy, tau), i3 = comp == 2 ? iJ : im;
-        A = k < 3 ? 0.0 : u3 * i3;
-        B = k < 3 ? 1.0 : i3;
-    } else if (body_fixed) {
-        A = pick(k, 0, rx, ry, th, vx, vy, w, rx - T.W, ry - T.W);
-        B = 0.0;
-    } else {
-        const double x0 = sel3(comp, rx, ry, th), v0 = sel3(comp, vx, vy, w);
-        const double u3 = sel3(comp, ux, uy, tau), i3 = comp == 2 ? iJ : im;
-        const double Av = v0 + dt * (u3 * i3), Bv = dt * i3;  // velocity
-        const bool vel = (k >= 3 && k <= 5);
-        A = vel ? Av : x0 + dt * Av - (k >= 6 ? T.W : 0.0);
-        B = vel ? Bv : dt * Bv;
-    }
-    // rotation of (cos, sin) by dtheta = dt thetadot' = Ad + Bd T_b, with
-    // (cos, sin) first brought back to unit norm (off the dependent chain)
-    double Ad = 0.0, Bd = 0.0;
-    if (!eval && !body_fixed) {
-        Ad = dt * (w + dt * (tau * iJ));
-        Bd = dt * dt * iJ;
-        const double f = 1.5 - 0.5 * (c * c + sn * sn);
-        c *= f;
-        sn *= f;
-    }
-    const double X = lane == 9 ? sn : c, Yr = lane == 9 ? c : -sn;  // lane 8: cos', lane 9: sin'
+    const BodyPlan plan = body_plan(T, lane, eval, body_fixed, rx, ry, th, vx, vy, w, c, sn, ux, uy, tau);
 
     pdl_wait();
     // the next density pass may be placed now: every tile of the force pass
@@ -1211,27 +1139,7 @@ __global__ void __launch_bounds__(32 * kBodyWarps) body_kernel(SimDev S, EvalOut
     const double Fx = __shfl_sync(0xffffffffu, vq, 0), Fy = __shfl_sync(0xffffffffu, vq, 1);
     const double Tq = __shfl_sync(0xffffffffu, vq, 2), Cx = __shfl_sync(0xffffffffu, vq, 3);
     const double Cy = __shfl_sync(0xffffffffu, vq, 4);
-    const double lin = fma(B, sel3(comp, Fx, Fy, Tq), A);
-    double v = lin;
-    if (!eval && !body_fixed) {
-        const double d = fma(Bd, Tq, Ad), d2 = d * d;
-        double cd, sd;
-        if (fabs(d) <= 1e-4) {  // first omitted terms d^4 / 24, d^5 / 120 below 1e-16 relative
-            cd = fma(-0.5, d2, 1.0);
-            sd = fma(d * d2, -1.0 / 6.0, d);
-        } else if (fabs(d) <= 1e-2) {
-            cd = 1.0 - d2 * (0.5 - d2 * (1.0 / 24.0 - d2 * (1.0 / 720.0)));
-            sd = d * (1.0 - d2 * (1.0 / 6.0 - d2 * (1.0 / 120.0 - d2 * (1.0 / 5040.0))));
-        } else {
-            double s1, c1;
-            sincos(d, &s1, &c1);
-            cd = c1;
-            sd = s1;
-        }
-        if (lane == 8 || lane == 9) v = fma(X, cd, Yr * sd);
-    } else if (lane == 8 || lane == 9) {
-        v = X;  // unchanged angle
-    }
+    const double v = body_apply(plan, lane, eval, body_fixed, Fx, Fy, Tq);
     if (sample && y && lane >= 6 && lane < SPH_NY) {
         double o = sel3(lane - 6, Fx, Fy, Tq);
         if (lane == 9) o = T.n_f ? Cx / T.n_f : 0.0;

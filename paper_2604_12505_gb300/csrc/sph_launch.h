@@ -41,6 +41,13 @@ cudaError_t launch_phase(const SimDev& S, const EvalOut& E, int eval, int tile_c
                          cudaStream_t st, bool pdl, bool tan = false, bool chained = false);
 cudaError_t launch_step(const SimDev& S, const EvalOut& E, int eval, int tile_code, int n_tiles, cudaStream_t st,
                         bool pdl, bool tan = false, bool chained = false);
+// Steps of small tanks in one launch (sph_resident.cu): whether a tank fits a
+// cluster; the CTAs per tank for B tanks (0: not all at once), asked on the
+// device before the first launch; n_steps steps under the run record already
+// set, from the step that it stands at.
+bool resident_fits(int n_f, int n_g, int G);
+cudaError_t prepare_resident(int B, int& cluster);
+cudaError_t launch_resident(const SimDev& S, int cluster, int n_steps, cudaStream_t st);
 // State transfer: xv [N, 4] the hi parts of the particle state, lo [N, 4] its
 // low parts (NULL: zero on binning, not read back on gathering).
 cudaError_t launch_bin_flat(const SimDev& S, const float* xv, const float* lo, const int* part_tank, int n, int buf,

@@ -36,6 +36,39 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
+// Warp sums (fixed order: deterministic)
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ F2 shfl_down_f2(F2 v, int o)
+{
+    return F2{__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)};
+}
+
+struct Red {
+    F2 fx, fy, t, cx, cy;
+    unsigned long long pairs;
+};
+
+// Sums over a warp (result valid in lane 0).  Only the parts flagged by the
+// uniform switches are reduced.
+__device__ __forceinline__ Red warp_reduce(Red r, bool forces, bool com, int first = 16)
+{
+#pragma unroll
+    for (int o = first; o > 0; o >>= 1) {
+        if (forces) {
+            r.fx = f2_add(r.fx, shfl_down_f2(r.fx, o));
+            r.fy = f2_add(r.fy, shfl_down_f2(r.fy, o));
+            r.t = f2_add(r.t, shfl_down_f2(r.t, o));
+        }
+        if (com) {
+            r.cx = f2_add(r.cx, shfl_down_f2(r.cx, o));
+            r.cy = f2_add(r.cy, shfl_down_f2(r.cy, o));
+        }
+        r.pairs += __shfl_down_sync(0xffffffffu, r.pairs, o);
+    }
+    return r;
+}
+
+// ---------------------------------------------------------------------------
 // Shared-memory staging of a tile and its halo
 // ---------------------------------------------------------------------------
 template <int TX, int TY, bool RHO, bool TAN = false>
