@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_force_kernel(SimDe
     const TankDev T = S.tank[tank];
     float bacc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     bool waited = false;
-    if (stage_from_record<TX, TY, false>(S, tank, A.buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
+    if (stage_from_record<Sh::THREADS, TX, TY, false>(S, tank, A.buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
         const float dt = T.dt;
         const int total = sm.start[Sh::NC];
         const BodyDev& b = S.body[tank];
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(Sim
     const TankDev T = S.tank[tank];
     float bacc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     bool waited = false;
-    if (stage_from_record<TX, TY, false>(S, tank, A.buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
+    if (stage_from_record<Sh::THREADS, TX, TY, false>(S, tank, A.buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
         const int total = sm.start[Sh::NC];
         const BodyDev& b = S.body[tank];
         const float bc = b.fc, bs = b.fs, brx = b.frx, bry = b.fry;

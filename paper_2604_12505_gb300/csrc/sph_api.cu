@@ -177,11 +177,11 @@ struct sph_sim {
     cudaStream_t side = nullptr;  // sph_vjp's second stream and the event that orders the two
     cudaEvent_t ev = nullptr;
     int res_cluster = 0;  // CTAs per tank of the resident kernel, 0: some tank does not fit, or not all at once
-    // Two and more steps run in the resident kernel: one alone is quicker in three
-    // launches (938 particles: 39 us against 43; two steps 65 against 54).  Its
-    // sums are those of the 4x4 tiles (code 3, the default), so another tile
-    // shape is taken at its word.
-    bool resident(int n_steps) const { return n_steps > 1 && res_cluster != 0 && tile_code == 3; }
+    // Three and more steps run in the resident kernel: one or two are as quick in
+    // three launches each (938 particles: two steps 50 us against 51, five 107
+    // against 83, forty 742 against 431).  Its sums are those of the 4x4 tiles
+    // (code 3, the default), so another tile shape is taken at its word.
+    bool resident(int n_steps) const { return n_steps > 2 && res_cluster != 0 && tile_code == 3; }
 
     SimDev dev(int code = 0) const
     {
@@ -425,6 +425,17 @@ int create_impl(const sph_params* p, int B, cudaStream_t st, sph_sim** out)
         max_groups = std::max(max_groups, ng);
     }
     s->tile_code = 3;
+    // Four lanes per particle while the tiles are at most four to an SM: two
+    // 512-thread CTAs have a place there at once, and about half of the tiles
+    // hold fluid.  On 152 SMs, us a step against a thread per particle: 255
+    // tiles (17 tanks of 138 particles) 20.2 / 25.7, 263 (18,696 particles at
+    // the paper's h) 28.6 / 41.2, 551 (29,272) 22.7 / 27.7; more tiles wait for
+    // a second round: 701 (38,348) 31.9 / 27.8, 813 (three tanks) 30.3 / 30.1,
+    // 960 (64 tanks of 138) 30.1 / 27.9.
+    int sms = 0, device = 0;
+    cudaGetDevice(&device);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    s->S.lanes = s->n_tiles[3] <= 4 * sms;
     bool fits = true;
     for (const TankHost& t : s->tanks) fits = fits && resident_fits(t.n_f, t.n_g, t.G);
 

@@ -250,6 +250,7 @@ struct SimDev {
     double* brec;                 // recorded run: per tank kBodyRec doubles, the body before the step (else NULL)
     int B;
     int n_tiles;
+    int lanes;                    // 4x4 tiles step with four lanes per particle
 };
 
 // ---------------------------------------------------------------------------

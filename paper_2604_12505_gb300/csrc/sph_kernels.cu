@@ -732,13 +732,6 @@ __device__ void tank_finalize(const SimDev& S, const TankDev& T, int tank, int e
     }
 }
 
-// Adds a two-float sum to a fixed-point body accumulator (an integer
-// reduction: the total does not depend on the order of the tiles).
-__device__ __forceinline__ void fix_add(unsigned long long* a, F2 v)
-{
-    const long long q = __float2ll_rn(v.hi * kFixScale) + __float2ll_rn(v.lo * kFixScale);
-    atomicAdd(a, (unsigned long long)q);
-}
 // ---------------------------------------------------------------------------
 // Force pass: Eqs. 10, 12, 16-19, Algorithm 1, symplectic Euler, re-binning
 // ---------------------------------------------------------------------------
@@ -772,7 +765,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
     Red acc{z, z, z, z, z, 0ull};
     Red tacc{z, z, z, z, z, 0ull};
     int flags = 0, wall = 0, own = 0;
-    if (stage_from_record<TX, TY, TAN>(S, tank, buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
+    if (stage_from_record<Sh::THREADS, TX, TY, TAN>(S, tank, buf, stage_record<TX, TY>(S, blockIdx.x), sm)) {
         const BodyDev& b = S.body[tank];
         const int n_own = sm.own_row[TY];
         own = n_own;
@@ -1331,6 +1324,8 @@ static cudaError_t launch_tile_phase(const SimDev& S, const EvalOut& E, int eval
             return cudaErrorInvalidValue;
         }
     }
+    if constexpr (TX == 4 && TY == 4)
+        if (S.lanes && !eval && phase < 2) return launch_lanes(S, n_tiles, phase, st, pdl, (pdl && chained) ? 1 : 0);
     if (phase == 0)
         return launch(density_kernel<TX, TY, false>, n_tiles, Sh::THREADS, st, pdl, S, E, eval, (pdl && chained) ? 1 : 0);
     if (phase == 1) return launch(force_kernel<TX, TY, false>, n_tiles, Sh::THREADS, st, pdl, S, E, eval);

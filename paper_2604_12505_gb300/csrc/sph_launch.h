@@ -41,6 +41,8 @@ cudaError_t launch_phase(const SimDev& S, const EvalOut& E, int eval, int tile_c
                          cudaStream_t st, bool pdl, bool tan = false, bool chained = false);
 cudaError_t launch_step(const SimDev& S, const EvalOut& E, int eval, int tile_code, int n_tiles, cudaStream_t st,
                         bool pdl, bool tan = false, bool chained = false);
+// Phase 0 or 1 of a step on 4x4 tiles with four lanes per particle (sph_lanes.cu).
+cudaError_t launch_lanes(const SimDev& S, int n_tiles, int phase, cudaStream_t st, bool pdl, int chained);
 // Steps of small tanks in one launch (sph_resident.cu): whether a tank fits a
 // cluster; the CTAs per tank for B tanks (0: not all at once), asked on the
 // device before the first launch; n_steps steps under the run record already

@@ -1,10 +1,11 @@
 // sph_resident.cu -- many steps of small tanks in one launch.
 //
 // A tank of up to 2,128 particles leaves most of the GPU idle, and a step of
-// three launches is a chain of L2 round trips and of long loops of few warps
-// (25 us for 938 particles, 44 for the paper's 2,024).  Here a cluster of CTAs
-// keeps one tank's state in its shared memory from step to step, and four
-// lanes share a particle: 11 and 18 us.  The 4x4-cell tiles of the step kernels are
+// three launches is a chain of L2 round trips and, with a thread per particle,
+// of long loops in few warps (25 us for 938 particles, 44 for the paper's
+// 2,024; with four lanes per particle 19 and 25).  Here a cluster of CTAs
+// keeps one tank's state in its shared memory from step to step, with four
+// lanes per particle: 11 and 16 to 18 us.  The 4x4-cell tiles of the step kernels are
 // dealt out to the CTAs (by particle count, when the kernel starts); a CTA
 // holds the particles of its tiles and of the cells around them, sends a
 // particle's new state to every CTA that will need it, and its density to
@@ -46,6 +47,7 @@
 
 #include "sph_body.cuh"
 #include "sph_common.cuh"
+#include "sph_lanes.cuh"
 #include "sph_launch.h"
 #include "sph_tile.cuh"
 
@@ -55,8 +57,6 @@ namespace {
 
 constexpr int kThreads = 640, kWarps = kThreads / 32;
 constexpr int kLanes = 4;           // lanes per particle
-constexpr int kChunk = 4;           // candidates that a lane evaluates at once
-constexpr int kBlock = kLanes * kChunk;
 constexpr int kSlots = kThreads / kLanes;  // particles that a pass takes at once
 constexpr int kSortThreads = kThreads - 32;  // the last warp updates the body meanwhile
 constexpr int kTile = 4;            // cells per tile side, as the default tile of the step kernels
@@ -142,36 +142,6 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void sort_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSortThreads) : "memory"); }
-
-// Lane l's value, of the lanes of this lane's particle.
-struct From {
-    template <typename V>
-    __device__ V operator()(V v, int l) const { return __shfl_sync(0xffffffffu, v, l, kLanes); }
-};
-
-// Eqs. 17, 19 and the torque: a ghost's force over the distance, the distance
-// and its arm, rounded as in force_kernel; of(l) is lane l's sum.
-struct WallSum {
-    float fx, fy, t;
-    __device__ void add(float f, float2 d, float2 arm)
-    {
-        const float x = __fmul_rn(f, d.x), y = __fmul_rn(f, d.y);
-        fx = __fsub_rn(fx, x);
-        fy = __fsub_rn(fy, y);
-        t = __fsub_rn(t, fmaf(arm.x, y, -__fmul_rn(arm.y, x)));
-    }
-    __device__ WallSum of(int l) const { return {From()(fx, l), From()(fy, l), From()(t, l)}; }
-};
-struct BothSum : WallSum {  // and the acceleration of the particle
-    float ax, ay, inv_m;
-    __device__ void add(float f, float2 d, float2 arm)
-    {
-        ax = fmaf(__fmul_rn(f, d.x), inv_m, ax);
-        ay = fmaf(__fmul_rn(f, d.y), inv_m, ay);
-        WallSum::add(f, d, arm);
-    }
-    __device__ BothSum of(int l) const { return {WallSum::of(l), From()(ax, l), From()(ay, l), inv_m}; }
-};
 
 // First indices in [lo0, hi0) and [lo1, hi1) of a list sorted by x whose x is
 // not below v0, v1.
@@ -369,36 +339,6 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
         return (int)start[(int)sh.at[i] + q * P] + t - (int)r[q];
     };
     const int sub = lane & (kLanes - 1);
-    constexpr From from;
-    // Up to three runs of a sorted list, one after the other: entry k lies at
-    // at(k).  Lane r of a particle has found run r, from a to z.  A warp's
-    // particles are walked together, as far as the longest: `most`.
-    struct Runs {
-        int o0, o1, o2, n0, n1, n, most;
-        __device__ int at(int k) const { return k + (k < n0 ? o0 : k < n1 ? o1 : o2); }
-        __device__ void pack(unsigned* p) const  // start and length
-        {
-            p[0] = (unsigned)o0 | (unsigned)n0 << 16;
-            p[1] = (unsigned)(o1 + n0) | (unsigned)(n1 - n0) << 16;
-            p[2] = (unsigned)(o2 + n1) | (unsigned)(n - n1) << 16;
-        }
-    };
-    auto unpack = [](const unsigned* p) {
-        Runs R;
-        R.n0 = (int)(p[0] >> 16);
-        R.n1 = R.n0 + (int)(p[1] >> 16);
-        R.n = R.n1 + (int)(p[2] >> 16);
-        R.o0 = (int)(p[0] & 0xffffu);
-        R.o1 = (int)(p[1] & 0xffffu) - R.n0;
-        R.o2 = (int)(p[2] & 0xffffu) - R.n1;
-        R.most = __reduce_max_sync(0xffffffffu, R.n);
-        return R;
-    };
-    auto runs = [&](int a, int z) {
-        const unsigned mine = (unsigned)a | (unsigned)max(z - a, 0) << 16;
-        const unsigned p[3] = {from(mine, 0), from(mine, 1), from(mine, 2)};
-        return unpack(p);
-    };
     // The sorted particles around a particle in cell c, clipped to the support.
     auto stencil = [&](bool on, int c, float x) {
         int a = 0, z = 0;
@@ -408,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
             z = start[cl + 2];
             lower(s_pv, a, start[cl + 1], x - T.clip, z, start[cl + 3], x + T.clip);
         }
-        return runs(a, z);
+        return lane_runs<kLanes>(pack_run(a, z));
     };
     // The ghosts within clip, as for_staged_ghosts visits them.
     auto ghost_rows = [&](bool on, float xi, float yi, float clip) {
@@ -432,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
                 }
             }
         }
-        return runs(a, b);
+        return lane_runs<kLanes>(pack_run(a, b));
     };
 
     const unsigned a_pv = smem_addr(in_pv), a_lo = smem_addr(in_lo), a_cell = smem_addr(in_cell), a_rho = smem_addr(r_rho);
@@ -547,6 +487,11 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
         }
         const int first = warp * (32 / kLanes);  // the warp's first particle, and this lane's
         const int mine = tid / kLanes;
+        auto keep = [](unsigned* p, const Runs& R) {
+            p[0] = (unsigned)R.o0 | (unsigned)R.n0 << 16;
+            p[1] = (unsigned)(R.o1 + R.n0) | (unsigned)(R.n1 - R.n0) << 16;
+            p[2] = (unsigned)(R.o2 + R.n1) | (unsigned)(R.n - R.n1) << 16;
+        };
         unsigned kept[6];  // the first pass's runs, of particles and of ghosts, for the force
         for (int p = 0; first + p < n_own; p += kSlots) {  // by whole warps
             const bool on = mine + p < n_own;
@@ -555,54 +500,12 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
             const float4 pi = s_pv[e];
             const float2 li = s_plo[e];
             const Runs R = stencil(on, c, pi.x);
-            if (p == 0) R.pack(kept);
-            float Sf = 0.f;
-            for (int k0 = 0; k0 < R.most; k0 += kBlock) {
-                float f[kChunk];
-#pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    const int k = k0 + sub * kChunk + u;
-                    const int j = k < R.n ? R.at(k) : e;
-                    const float2 d = sep_ff(pi, li, s_pv[j], s_plo[j]);
-                    const float r2 = dist2(d.x, d.y);
-                    const float inv_r = rsqrtf(fmaxf(r2, FLT_MIN));
-                    const float q = r2 * inv_r * T.inv_h;
-                    const float qa = 2.0f - q, qb = fmaxf(1.0f - q, 0.0f);
-                    f[u] = r2 < T.R2 && k < R.n ? fmaf(-4.0f * qb * qb, qb, qa * qa * qa) : 0.0f;
-                }
-#pragma unroll
-                for (int l = 0; l < kLanes; ++l) {
-                    float t = Sf;
-#pragma unroll
-                    for (int u = 0; u < kChunk; ++u) t += f[u];
-                    Sf = from(t, l);
-                }
-            }
+            if (p == 0) keep(kept, R);
+            float Sf = fluid_sum<kLanes>(T, R, e, pi, li, s_pv, s_plo, sub);
             Sf = __fmul_rn(Sf, T.cW);
-            float Sg = 0.f;
             const Runs Q = ghost_rows(on, pi.x, pi.y, T.clip);
-            if (p == 0) Q.pack(kept + 3);
-            for (int k0 = 0; k0 < Q.most; k0 += kBlock) {
-                float f[kChunk];
-#pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    const int k = k0 + sub * kChunk + u;
-                    const float2 d = sep_fg(pi, li, g_p[k < Q.n ? Q.at(k) : 0]);
-                    const float r2 = dist2(d.x, d.y);
-                    // w_cubic as density_kernel rounds it, its factor cW with the sum
-                    const float inv_r = rsqrtf(fmaxf(r2, FLT_MIN));
-                    const float q = __fmul_rn(r2 * inv_r, T.inv_h);
-                    const float qa = __fsub_rn(2.0f, q), qb = fmaxf(__fsub_rn(1.0f, q), 0.0f);
-                    f[u] = k < Q.n && r2 < T.R2 ? fmaf(-4.0f * qb * qb, qb, qa * qa * qa) : 0.0f;
-                }
-#pragma unroll
-                for (int l = 0; l < kLanes; ++l) {
-                    float t = Sg;
-#pragma unroll
-                    for (int u = 0; u < kChunk; ++u) t = fmaf(T.cW, f[u], t);
-                    Sg = from(t, l);
-                }
-            }
+            if (p == 0) keep(kept + 3, Q);
+            const float Sg = ghost_sum<kLanes>(T, Q, pi, li, g_p, sub);
             const float rho = __fmul_rn(T.m, __fmaf_rn(T.gamma1, Sg, Sf));       // Eq. 14
             const float Pr = __fmul_rn(T.k, __fsub_rn(rho, T.rho0));              // Eq. 11
             const float2 v = make_float2(rho, __fdiv_rn(Pr, __fmul_rn(rho, rho)));
@@ -625,100 +528,17 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
         // --------------------------------------------------------------
         const float damp = sh.damp;
         int flags = 0;
-        // Eqs. 16-19 of own particle e with its ghosts, added to W ghost by ghost in their
-        // order; returns how many ghosts this lane found within reach.
-        auto ghost_forces = [&](int e, const Runs& Q, auto& W) {
-            const float4 pi = s_pv[e];
-            const float2 li = s_plo[e], ri = s_rho[e];
-            const float mm = T.m * T.m;
-            const float qg = T.gp_clamp ? fmaxf(ri.y, 0.f) : ri.y;
-            int n_met = 0;
-            for (int k0 = 0; k0 < Q.most; k0 += kBlock) {
-                float f[kChunk];
-                float2 d2[kChunk], arm[kChunk];
-                bool any = false;
-#pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    const int k = k0 + sub * kChunk + u, g = k < Q.n ? Q.at(k) : 0;
-                    d2[u] = sep_fg(pi, li, g_p[g]);
-                    const float ddx = d2[u].x, ddy = d2[u].y;
-                    const float r2 = dist2(ddx, ddy);
-                    const bool met = k < Q.n && r2 < T.h2;
-                    f[u] = 0.f;
-                    arm[u] = make_float2(0.f, 0.f);
-                    if (met && r2 > 0.f) {
-                        const float4 gv = g_v[g];
-                        const float inv_r = rsqrtf(r2);
-                        const float rr = r2 * inv_r;
-                        const float d = T.h - rr;
-                        const float gWs = T.cdS * d * d * inv_r;                         // (dW_s3/dr)/r
-                        const float fp = T.gp_sign * 2.0f * mm * qg * gWs;              // Eq. 16
-                        const float vr = (pi.z - gv.x) * ddx + (pi.w - gv.y) * ddy;
-                        const float fv = __fdividef(mm * T.beta2 * fminf(vr, 0.f), (ri.x + ri.x) * (r2 + T.epsh2)) * gWs;  // Eq. 18
-                        f[u] = fp + fv;
-                        arm[u] = make_float2(gv.z, gv.w);
-                    }
-                    n_met += met;
-                    any |= met;
-                }
-                const unsigned hit = __ballot_sync(0xffffffffu, any);
-#pragma unroll
-                for (int l = 0; l < kLanes; ++l)
-                    if (hit & (0x11111111u << l)) {
-                        auto V = W;
-#pragma unroll
-                        for (int u = 0; u < kChunk; ++u) V.add(f[u], d2[u], arm[u]);
-                        W = V.of(l);
-                    }
-            }
-            return n_met;
-        };
         for (int p = 0; first + p < n_own; p += kSlots) {
             const bool on = mine + p < n_own;
             const int e = on ? own[mine + p] : 0;
             const float4 pi = s_pv[e];
             const float2 li = s_plo[e], ri = s_rho[e];
-            const Runs R = p == 0 ? unpack(kept) : stencil(on, s_cell[e], pi.x);
+            const Runs R = p == 0 ? unpack_runs(kept[0], kept[1], kept[2]) : stencil(on, s_cell[e], pi.x);
             float ax = 0.f, ay = 0.f;
-            int nff = 0;
-            for (int k0 = 0; k0 < R.most; k0 += kBlock) {  // Eqs. 10 and 12
-                float sf[kChunk];
-                float2 d[kChunk];
-#pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    const int k = k0 + sub * kChunk + u;
-                    const int j = k < R.n ? R.at(k) : e;
-                    const float4 pj = s_pv[j];
-                    const float2 rj = s_rho[j];
-                    d[u] = sep_ff(pi, li, pj, s_plo[j]);
-                    const float ddx = d[u].x, ddy = d[u].y;
-                    const float r2 = dist2(ddx, ddy);
-                    const bool nb = r2 < T.R2 && j != e;
-                    const float inv_r = rsqrtf(fmaxf(r2, FLT_MIN));
-                    // dw_cubic_over_r and the rest as force_kernel rounds them
-                    const float q = __fmul_rn(r2 * inv_r, T.inv_h);
-                    const float qa = __fsub_rn(2.0f, q), qb = fmaxf(__fsub_rn(1.0f, q), 0.0f);
-                    const float gW = T.cdW * fmaf(12.0f * qb, qb, __fmul_rn(-3.0f * qa, qa)) * inv_r;
-                    const float press = -(ri.y + rj.y);                                  // Eq. 10
-                    const float vr = fmaf(pi.w - pj.w, ddy, __fmul_rn(pi.z - pj.z, ddx));
-                    const float visc = __fdividef(T.visc_a * vr, (ri.x + rj.x) * (r2 + T.epsh2));  // Eq. 12
-                    sf[u] = nb && r2 > 0.f ? T.m * (press + visc) * gW : 0.f;
-                    nff += nb;
-                }
-#pragma unroll
-                for (int l = 0; l < kLanes; ++l) {
-                    float tx = ax, ty = ay;
-#pragma unroll
-                    for (int u = 0; u < kChunk; ++u) {
-                        tx = fmaf(sf[u], d[u].x, tx);
-                        ty = fmaf(sf[u], d[u].y, ty);
-                    }
-                    ax = from(tx, l);
-                    ay = from(ty, l);
-                }
-            }
+            int nff = fluid_forces<kLanes>(T, R, e, pi, li, ri, s_pv, s_plo, s_rho, sub, ax, ay);
             BothSum W{{0.f, 0.f, 0.f}, ax, ay, T.inv_m};
-            nff += ghost_forces(e, p == 0 ? unpack(kept + 3) : ghost_rows(on, pi.x, pi.y, T.clip), W);
+            const Runs Q = p == 0 ? unpack_runs(kept[3], kept[4], kept[5]) : ghost_rows(on, pi.x, pi.y, T.clip);
+            nff += ghost_forces<kLanes>(T, Q, pi, li, ri, g_p, g_v, sub, W);
             ax = W.ax;
             ay = W.ay;
             pairs_sum += (unsigned)nff;
@@ -811,7 +631,8 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
                         on = W.fx != 0.f || W.fy != 0.f || W.t != 0.f;
                     }
                     if (!__any_sync(0xffffffffu, on)) continue;
-                    ghost_forces(e, ghost_rows(on, s_pv[e].x, s_pv[e].y, T.hclip), W);
+                    const float4 pi = s_pv[e];
+                    ghost_forces<kLanes>(T, ghost_rows(on, pi.x, pi.y, T.hclip), pi, s_plo[e], s_rho[e], g_p, g_v, sub, W);
                     if (on && sub == 0) {
                         w_xy[e] = make_float2(W.fx, W.fy);
                         w_t[e] = W.t;
@@ -971,7 +792,7 @@ struct Launch {
 
 // CTAs per tank: sixteen (the most a cluster can have) while the GPU holds all
 // tanks at once, else eight, else none: tanks that wait for a place lose to the
-// step kernels (64 of the paper's tanks take those 72 us a step; 12 tanks 36,
+// step kernels (64 of the paper's tanks take those 72 us a step, 12 tanks 35,
 // in clusters of eight 22).
 cudaError_t prepare_resident(int B, int& cluster)
 {

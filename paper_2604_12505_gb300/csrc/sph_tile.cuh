@@ -68,6 +68,14 @@ __device__ __forceinline__ Red warp_reduce(Red r, bool forces, bool com, int fir
     return r;
 }
 
+// Adds a two-float sum to a fixed-point body accumulator (an integer
+// reduction: the total does not depend on the order of the tiles).
+__device__ __forceinline__ void fix_add(unsigned long long* a, F2 v)
+{
+    const long long q = __float2ll_rn(v.hi * kFixScale) + __float2ll_rn(v.lo * kFixScale);
+    atomicAdd(a, (unsigned long long)q);
+}
+
 // ---------------------------------------------------------------------------
 // Shared-memory staging of a tile and its halo
 // ---------------------------------------------------------------------------
@@ -251,18 +259,18 @@ __device__ __forceinline__ void save_stage(const Stage<TX, TY, RHO, TAN>& sm, bo
 // Stages a tile from its record: one round of loads for the cell starts and
 // (speculatively, the whole list) the slots, one for the particle state.
 // Returns false (uniformly) if the density pass could not stage the tile.
-template <int TX, int TY, bool TAN>
+template <int THREADS, int TX, int TY, bool TAN>
 __device__ __forceinline__ bool stage_from_record(const SimDev& S, int tank, int buf, const StageRec<TX, TY>* rec,
                                                   Stage<TX, TY, true, TAN>& sm)
 {
     using Sh = Shape<TX, TY>;
-    constexpr int KPT = (Sh::MAXS + Sh::THREADS - 1) / Sh::THREADS;
+    constexpr int KPT = (Sh::MAXS + THREADS - 1) / THREADS;
     const int tid = threadIdx.x;
     int r_slot[KPT], r_cell[KPT];
-    for (int c = tid; c <= Sh::NC; c += Sh::THREADS) sm.start[c] = __ldcg(rec->start + c);
+    for (int c = tid; c <= Sh::NC; c += THREADS) sm.start[c] = __ldcg(rec->start + c);
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
-        const int i = tid + q * Sh::THREADS;
+        const int i = tid + q * THREADS;
         r_slot[q] = i < Sh::MAXS ? __ldcg(rec->slot + i) : 0;
         r_cell[q] = i < Sh::MAXS ? (int)__ldcg(rec->cell + i) : 0;
     }
@@ -286,7 +294,7 @@ __device__ __forceinline__ bool stage_from_record(const SimDev& S, int tank, int
     if (sm.own_row[TY] == 0) return true;  // no own particle: the slot list was not written
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
-        const int i = tid + q * Sh::THREADS;
+        const int i = tid + q * THREADS;
         if (i < total) {
             const int gs = r_slot[q];
             sm.pv[i] = S.pv[buf][gs];

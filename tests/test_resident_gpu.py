@@ -18,7 +18,7 @@ BASE = dict(W.BASE, dx=0.02)
 CASES = {
     # one tile's particles, on a few CTAs of the cluster; steps beyond one launch's
     "tiny": ([W.TINY], 1030, {}),
-    "one step and two": ([BASE], 3, dict(calls=(1, 2))),
+    "two steps and three": ([BASE], 5, dict(calls=(2, 3))),
     # tiles of more than 128 particles, whose threads sum two particles each
     "paper": ([PAPER], 60, {}),
     "clamped": ([dict(PAPER, ghost_pressure_clamp=1)], 60, {}),
