@@ -71,7 +71,7 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
             int ix = cx0 + c % TX, iy = cy0 + c / TX;
             if (ix < T.G && iy < T.G) S.count[nbuf][T.cell_base + iy * T.G + ix] = 0;
         }
-    const bool staged = stage_tile<TX, TY, false, TAN>(S, T, buf, cx0, cy0, sm);
+    const bool staged = stage_tile<TX, TY, TAN>(S, T, buf, cx0, cy0, sm);
     save_stage(sm, staged, stage_record<TX, TY>(S, blockIdx.x));
     const int n_own = staged ? sm.own_row[TY] : 0;
     if (n_own == 0) {
@@ -255,7 +255,7 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
             S.trho[sm.slot[e]] = make_float2(trh, trh * (T.k / (rho * rho) - 2.0f * pr2 / rho));
         }
         if (eval) {
-            const int id = sm.pid[e];
+            const int id = __ldcg(S.pid[buf] + sm.slot[e]);
             if (E.rho) E.rho[id] = rho;
             if (E.drho) E.drho[id] = T.m * (Df + T.gamma1 * Dg);
             if (E.nbr) E.nbr[3 * id + 1] = ng2;
@@ -933,7 +933,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
             } else {
                 // kick then drift (Section 3.4) on the two-float state, then bin
                 // into the next grid: v' = (v + dt a)(1 - c), x' = x + dt v'
-                const float2 vl = sm.vlo[e];
+                const float2 vl = velocity_lo(S, buf, sm, e);
                 float2 kx = two_sum(pi.z, fmaf(T.dt, ax, vl.x)), ky = two_sum(pi.w, fmaf(T.dt, ay, vl.y));
                 if (damp != 1.0f) {  // relaxation: scale the two-float velocity
                     const float hx = kx.x * damp, hy = ky.x * damp;

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kThreads, 2) density_lanes_kernel(SimDev S, in
         const int ix = cx0 + c % 4, iy = cy0 + c / 4;
         if (ix < T.G && iy < T.G) S.count[nbuf][T.cell_base + iy * T.G + ix] = 0;
     }
-    const bool staged = stage_tile<4, 4, false, false>(S, T, buf, cx0, cy0, sm);
+    const bool staged = stage_tile<4, 4, false>(S, T, buf, cx0, cy0, sm);
     save_stage(sm, staged, stage_record<4, 4>(S, blockIdx.x));
     const int n_own = staged ? sm.own_row[4] : 0;
     if (n_own == 0) {
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 2) force_lanes_kernel(SimDev S)
             ax = B.ax + T.grav_x;
             ay = B.ay + T.grav_y;
             // kick then drift, and the next grid, as in force_kernel
-            const float2 vl = sm.vlo[e];
+            const float2 vl = velocity_lo(S, buf, sm, e);
             float2 kx = two_sum(pi.z, fmaf(T.dt, ax, vl.x)), ky = two_sum(pi.w, fmaf(T.dt, ay, vl.y));
             if (damp != 1.0f) {
                 const float hx = kx.x * damp, hy = ky.x * damp;

@@ -86,13 +86,17 @@ struct Stage {
     int own_row[TY + 1];
     float4 pv[Sh::MAXS];
     float2 plo[Sh::MAXS];         // low parts (x_lo, y_lo) of the staged positions
-    int pid[Sh::MAXS];
-    int pid_in[Sh::MAXS];         // particle index in global slot order (before ordering)
-    unsigned int key_in[Sh::MAXS];  // ordering key of x in global slot order
+    // What only one of the passes reads takes no room in the other: it is shared
+    // memory that limits the CTAs of an SM (7 of the force pass, 8 of the density
+    // pass of 4x4 tiles; with all of it in both, and the low parts of the
+    // velocities, 6 and 7: 97,748 particles 36.3 -> 34.7 us a step, a batch of
+    // 64 tanks 256 -> 239).
+    int pid[RHO ? Sh::MAXS : 1];
+    int pid_in[RHO ? 1 : Sh::MAXS];         // particle index in global slot order (before ordering)
+    unsigned int key_in[RHO ? 1 : Sh::MAXS];  // ordering key of x in global slot order
     int slot[Sh::MAXS];
     unsigned char cell[Sh::MAXS];
     float2 rho[RHO ? Sh::MAXS : 1];
-    float2 vlo[RHO ? Sh::MAXS : 1];           // low parts (vx_lo, vy_lo) of the velocities (force pass)
     float4 tpv[TAN ? Sh::MAXS : 1];           // tangent (dx, dy, dvx, dvy)
     float tsum[(TAN && !RHO) ? Sh::MAXS : 1];  // density pass: an own particle's fluid sum of the tangent
     float2 trho[(TAN && RHO) ? Sh::MAXS : 1];  // tangent (d rho, d(P / rho^2))
@@ -114,8 +118,8 @@ __device__ __forceinline__ unsigned int order_key(float x)
 // does not fit.  The counts and the state are read through L2 (ld.global.cg):
 // the density pass may stage before its grid dependency, from data that an
 // earlier, completed grid wrote.
-template <int TX, int TY, bool RHO, bool TAN>
-__device__ bool stage_tile(const SimDev& S, const TankDev& T, int buf, int cx0, int cy0, Stage<TX, TY, RHO, TAN>& sm)
+template <int TX, int TY, bool TAN>
+__device__ bool stage_tile(const SimDev& S, const TankDev& T, int buf, int cx0, int cy0, Stage<TX, TY, false, TAN>& sm)
 {
     using Sh = Shape<TX, TY>;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -202,17 +206,8 @@ __device__ bool stage_tile(const SimDev& S, const TankDev& T, int buf, int cx0, 
         const int ix = cx0 - 1 + c % Sh::SX, iy = cy0 - 1 + c / Sh::SX;
         const int gs = (T.cell_base + iy * T.G + ix) * kCap + (e - a);
         sm.pv[d] = __ldcg(S.pv[buf] + gs);
-        const float4 lo = __ldcg(S.lo[buf] + gs);
-        sm.plo[d] = make_float2(lo.x, lo.y);
-        if (RHO) {
-            sm.rho[d] = S.rhoP[gs];
-            sm.vlo[d] = make_float2(lo.z, lo.w);
-        }
-        if constexpr (TAN) {
-            sm.tpv[d] = __ldcg(S.tpv[buf] + gs);
-            if (RHO) sm.trho[d] = S.trho[gs];
-        }
-        sm.pid[d] = id;
+        sm.plo[d] = __ldcg(reinterpret_cast<const float2*>(S.lo[buf] + gs));
+        if constexpr (TAN) sm.tpv[d] = __ldcg(S.tpv[buf] + gs);
         sm.slot[d] = gs;
     }
     __syncthreads();
@@ -298,9 +293,7 @@ __device__ __forceinline__ bool stage_from_record(const SimDev& S, int tank, int
         if (i < total) {
             const int gs = r_slot[q];
             sm.pv[i] = S.pv[buf][gs];
-            const float4 lo = S.lo[buf][gs];
-            sm.plo[i] = make_float2(lo.x, lo.y);
-            sm.vlo[i] = make_float2(lo.z, lo.w);
+            sm.plo[i] = *reinterpret_cast<const float2*>(S.lo[buf] + gs);
             sm.rho[i] = S.rhoP[gs];
             if constexpr (TAN) {
                 sm.tpv[i] = S.tpv[buf][gs];
@@ -313,6 +306,13 @@ __device__ __forceinline__ bool stage_from_record(const SimDev& S, int tank, int
     }
     __syncthreads();
     return true;
+}
+
+// The low parts of a staged particle's velocity, which only its own step needs.
+template <class Stg>
+__device__ __forceinline__ float2 velocity_lo(const SimDev& S, int buf, const Stg& sm, int e)
+{
+    return reinterpret_cast<const float2*>(S.lo[buf] + sm.slot[e])[1];
 }
 
 // First staged index in [lo, hi) whose x is not below v (a cell is sorted by
