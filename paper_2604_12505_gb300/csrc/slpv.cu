@@ -397,68 +397,97 @@ __global__ void __launch_bounds__(kSampleThreads)
 }
 
 // lambda_k = J_k^T lambda_{k+1} + c_k over the window, backwards from
-// carry[traj][NX] (last window: zero); lam[traj][ld][NX] receives lambda_{k+1}
-// at row k.  Lane j owns lambda_j: a step is NX shuffles and a chain of NX / 2
-// FMAs and an add.  The records pass through shared memory in chunks, copied
-// by the lanes of their own trajectory.
+// carry_in[traj][NX] (first, the last window: from zero); lam[traj][ld][NX]
+// receives lambda_{k+1} at row k, carry_out the window's first lambda.  Lane j
+// owns lambda_j: a step is NX shuffles and a chain of NX / 2 FMAs and an add.
+// The records pass through shared memory in chunks, copied by the lanes of
+// their own trajectory.
+//
+// The step is affine, so the time axis is cut into n_seg segments of seg_len
+// samples that run side by side: with MAP, each but the first takes the unit
+// vectors without and the zero vector with c_k from its end to its start, which
+// is its map (map[traj][seg][NX + 1][NX]); then each segment starts from what
+// the maps of the later ones give.  24 trajectories of 2,200 samples: 87 us in
+// one chain, 16 in 28 segments.
 template <int NX>
 constexpr int kAdjChunk = NX <= 4 ? 16 : 8;
 
-template <int NX>
-__global__ void __launch_bounds__(32) adjoint_kernel(const float* __restrict__ adj, int n_traj, int len, int ld,
-                                                     int first, float* __restrict__ carry, float* __restrict__ lam)
+template <int NX, bool MAP>
+__global__ void __launch_bounds__(32)
+    adjoint_kernel(const float* __restrict__ adj, int n_traj, int len, int ld, int n_seg, int seg_len, int first,
+                   const float* __restrict__ carry_in, float* __restrict__ carry_out, float* __restrict__ map,
+                   float* __restrict__ lam)
 {
     constexpr int L = kLanes<NX>, PER = 32 / L, C = kAdjChunk<NX>, R = kRec<NX>;
     // a trajectory's chunk padded by 4 floats: the groups of a warp read distinct banks
     __shared__ __align__(16) float sj[kStages][PER][C * R + 4];
     const int l = (int)threadIdx.x % L, j = l % NX, grp = (int)threadIdx.x / L;
-    const int tr = blockIdx.x * PER + grp;
+    const int g = blockIdx.x * PER + grp;
+    const int col = MAP ? g % (NX + 1) : NX;  // the map's column that this group computes
+    const int sg = MAP ? g / (NX + 1) : g, per_traj = MAP ? n_seg - 1 : n_seg;
+    const int tr = sg / per_traj, seg = sg % per_traj + (MAP ? 1 : 0);
     const bool own = tr < n_traj && l < NX;
     const size_t t = tr < n_traj ? tr : n_traj - 1;
-    float v = first ? 0.f : carry[t * NX + j];
-    float* lt = lam + t * ld * NX + j;
-    const float* at = adj + t * ld * R;
-    const int n_chunk = (len + C - 1) / C;
-    // chunk c holds steps [max(len - (c + 1) C, 0), len - c C), in order
+    const int k0 = seg * seg_len, n = min(len - k0, seg_len);  // the segment's samples
+    float v = MAP ? (j == col ? 1.f : 0.f) : first ? 0.f : carry_in[t * NX + j];
+    auto at_map = [&](int s, int c) { return map + ((t * n_seg + s) * (NX + 1) + c) * NX + j; };
+    if constexpr (!MAP) {
+#pragma unroll 4
+        for (int s = n_seg - 1; s >= 1; --s) {
+            float w = *at_map(s, NX);
+#pragma unroll
+            for (int r = 0; r < NX; ++r) w = fmaf(*at_map(s, r), __shfl_sync(0xffffffffu, v, r, L), w);
+            if (s > seg) v = w;
+        }
+    }
+    float* lt = lam + (t * ld + k0) * NX + j;
+    const float* at = adj + (t * ld + k0) * R;
+    const int n_chunk = (seg_len + C - 1) / C;  // the same in all groups of a warp
+    // chunk c holds steps n - (c + 1) C and on, C of them; those below 0 are not there
     auto fetch = [&](int c) {
-        const int lo = len - (c + 1) * C;
+        const int lo = n - (c + 1) * C;
         float* dst = &sj[c % kStages][grp][4 * l];
+        const float* src = at + (ptrdiff_t)lo * R + 4 * l;
         if (lo >= 0) {
-            const float* src = at + (size_t)lo * R + 4 * l;
 #pragma unroll
             for (int i = 0; i < C * R; i += 4 * L)
                 if (C * R % (4 * L) == 0 || i + 4 * l < C * R) copy_async<16>(dst + i, src + i);
         } else {
-            for (int i = 4 * l; i < (lo + C) * R; i += 4 * L) copy_async<16>(dst + (i - 4 * l), at + i);
+            for (int i = 0; i + 4 * l < C * R; i += 4 * L)
+                if (i + 4 * l >= -lo * R) copy_async<16>(dst + i, src + i);
         }
         copy_commit();
     };
-    auto step = [&](int k, const float* rec) {
-        if (own) lt[(size_t)k * NX] = v;
-        float J[NX], n = rec[NX * NX + j], m = 0.f;
+    auto step = [&](int k, const float* rec, bool in) {
+        if (!MAP && own && in) lt[(ptrdiff_t)k * NX] = v;
+        float J[NX], a = col == NX ? rec[NX * NX + j] : 0.f, m = 0.f;
         load_vec<NX>(rec + j * NX, J);
 #pragma unroll
         for (int r = 0; r < NX; r += 2) {
-            n = fmaf(J[r], __shfl_sync(0xffffffffu, v, r, L), n);
+            a = fmaf(J[r], __shfl_sync(0xffffffffu, v, r, L), a);
             m = fmaf(J[r + 1], __shfl_sync(0xffffffffu, v, r + 1, L), m);
         }
-        v = n + m;
+        v = in ? a + m : v;
     };
 #pragma unroll
     for (int c = 0; c < kStages - 1; ++c) fetch(c);
     for (int c = 0; c < n_chunk; ++c) {
         copy_wait<kStages - 2>();
         fetch(c + kStages - 1);
-        const int lo = len - (c + 1) * C;
+        const int lo = n - (c + 1) * C;
         const float* rec = sj[c % kStages][grp];
-        if (lo >= 0) {
+        if (__all_sync(0xffffffffu, lo >= 0)) {
 #pragma unroll
-            for (int q = C - 1; q >= 0; --q) step(lo + q, rec + q * R);
+            for (int q = C - 1; q >= 0; --q) step(lo + q, rec + q * R, true);
         } else {
-            for (int q = lo + C - 1; q >= 0; --q) step(q, rec + q * R);
+            for (int q = C - 1; q >= 0; --q) step(lo + q, rec + q * R, lo + q >= 0);
         }
     }
-    if (own) carry[t * NX + j] = v;
+    if constexpr (MAP) {
+        if (own) *at_map(seg, col) = v;
+    } else {
+        if (own && seg == 0) carry_out[t * NX + j] = v;
+    }
 }
 
 // The gradient's data term: every entry of theta is a sum over the samples of
@@ -1217,7 +1246,14 @@ int loss_grad_launch(slpv_model* m, const float* u, const float* y, int n_traj, 
     const size_t per = want ? (size_t)(nx * nx + nx + 3) / 4 * 4 + nx : (size_t)nx;  // floats of a sample in the window
     const int W = (int)std::min<size_t>((size_t)T, std::max<size_t>(kWindowBytes / 4 / per / (size_t)n_traj, 16));
     int rc = grow(&m->win, &m->win_cap, (size_t)n_traj * W * per);
-    if (!rc) rc = grow(&m->carry, &m->carry_cap, 2 * (size_t)n_traj * nx);
+    // The adjoint in segments of 64 samples and more, at most 32, while their
+    // maps are few enough to run at once; fewer than 4 do not pay for the maps
+    // (4 cut the time to about a half).
+    const int seg_most = std::min({W / 64, 32, 6144 / std::max(1, std::min(n_traj, 6144) * (nx + 1))});
+    const int n_seg_most = want && seg_most >= 4 ? seg_most : 1;
+    // state and adjoint between windows (the adjoint's read and written in turn), the maps
+    const size_t maps = (size_t)n_traj * n_seg_most * (nx + 1) * nx;
+    if (!rc) rc = grow(&m->carry, &m->carry_cap, 3 * (size_t)n_traj * nx + (n_seg_most > 1 ? maps : 0));
     if (!rc && want) rc = grow(&m->xh, &m->xh_cap, (size_t)n_traj * T * nx);
     if (rc) return rc;
     const double inv_nd = 1.0 / ((double)n_traj * T);
@@ -1257,8 +1293,17 @@ int loss_grad_launch(slpv_model* m, const float* u, const float* y, int n_traj, 
         for (int w = n_win - 1; w >= 0; --w) {
             const int k0 = w * W, len = std::min(W, T - k0), first = w == n_win - 1 ? 1 : 0;
             sample(w, m->xh, T, 0);
-            adjoint_kernel<NX><<<sgrid, 32, 0, st>>>(m->win, n_traj, len, W, first, m->carry + (size_t)n_traj * NX,
-                                                     lam);
+            const int want_len = (len + n_seg_most - 1) / n_seg_most;
+            const int seg_len = n_seg_most > 1 ? (want_len + kAdjChunk<NX> - 1) / kAdjChunk<NX> * kAdjChunk<NX> : len;
+            const int n_seg = (len + seg_len - 1) / seg_len;
+            float* carry[2] = {m->carry + (size_t)n_traj * NX, m->carry + 2 * (size_t)n_traj * NX};
+            float* map = m->carry + 3 * (size_t)n_traj * NX;
+            auto blocks = [&](long long groups) { return (unsigned)((groups * kLanes<NX> + 31) / 32); };
+            if (n_seg > 1)
+                adjoint_kernel<NX, true><<<blocks((long long)n_traj * (n_seg - 1) * (NX + 1)), 32, 0, st>>>(
+                    m->win, n_traj, len, W, n_seg, seg_len, first, nullptr, nullptr, map, nullptr);
+            adjoint_kernel<NX, false><<<blocks((long long)n_traj * n_seg), 32, 0, st>>>(
+                m->win, n_traj, len, W, n_seg, seg_len, first, carry[(w + 1) & 1], carry[w & 1], map, lam);
             outer_kernel<NX><<<oblk, Outer<NX>::kThreads, 0, st>>>(m->th, u, y, m->scales, n_traj, T, k0, len, W, inv_n,
                                                                    first, m->xh, lam, m->part);
         }

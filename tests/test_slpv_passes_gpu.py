@@ -22,7 +22,11 @@ SC = np.array([20.0, 20.0, 2.0, 0.1, 0.1, 0.05], dtype=np.float32)
 # cut into windows (the mean over them does not change)
 @pytest.mark.parametrize("nx,n,T,copies", [(2, 1, 1, 1), (2, 9, 32, 1), (4, 9, 33, 1), (4, 17, 127, 1), (6, 5, 64, 1),
                                            (6, 4, 9, 1), (8, 3, 31, 1), (8, 33, 8, 1), (4, 7, 40, 5000),
-                                           (8, 5, 50, 2000)])
+                                           (8, 5, 50, 2000),
+                                           # the adjoint in segments: 4, 5 and 10 of a ragged
+                                           # length, and of each of two windows
+                                           (2, 2, 257, 1), (4, 9, 321, 1), (6, 3, 650, 1), (8, 2, 333, 1),
+                                           (4, 2, 2500, 150)])
 def test_passes_match_oracle(nx, n, T, copies):
     torch = need_gpu()
     from paper_2604_12505_gb300.slpv import VelocityModel
