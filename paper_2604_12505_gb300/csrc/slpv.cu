@@ -102,19 +102,19 @@ __device__ __forceinline__ void mz(const float* th, float p, const float* z, flo
 // ---------------------------------------------------------------------------
 // Loss and gradient in four passes.
 //
-// Only two recurrences are serial in k: the state x_{k+1} and the adjoint
+// Only two recurrences run along k: the state x_{k+1} and the adjoint
 // lambda_k.  The adjoint's step is linear, lambda_k = J_k^T lambda_{k+1} +
 // c_k, with J_k and c_k functions of x_k alone, and so are every sample's
 // residual and its contribution to the gradient once lambda is known:
 //   state_kernel    x_k for all k (serial; NX lanes or more per trajectory)
 //   sample_kernel   squared errors, J_k and c_k (one thread per sample)
-//   adjoint_kernel  lambda_k (serial; one lane per state)
+//   adjoint_kernel  lambda_k (in segments of the time axis; one lane per state)
 //   outer_kernel    the gradient's outer products over all samples
 //   final_kernel    sums of the block partials, the l2 term, the mask
 // One thread per trajectory running both recurrences with everything on the
 // chain took 2,600 cycles per sample: 2.73 ms for 24 trajectories of 2,200
-// samples (n_x = 4), now 0.46 ms (state 339 us, adjoint 87, outer 12, sample
-// 10, final 7).  The state chain's latencies add up to 293 cycles of its 318
+// samples (n_x = 4), now 0.39 ms (state 339 us, adjoint 19, outer 11, sample
+// 9, final 6).  The state chain's latencies add up to 293 cycles of its 318
 // a sample: 7 FMAs, tanhf (62), a shuffle (26), 4 FMAs, tanhf, a shuffle, 4
 // FMAs, 8 FMAs and a shuffle.
 // ---------------------------------------------------------------------------
@@ -408,7 +408,8 @@ __global__ void __launch_bounds__(kSampleThreads)
 // vectors without and the zero vector with c_k from its end to its start, which
 // is its map (map[traj][seg][NX + 1][NX]); then each segment starts from what
 // the maps of the later ones give.  24 trajectories of 2,200 samples: 87 us in
-// one chain, 16 in 28 segments.
+// one chain, 19 in 28 segments (maps 7,
+// lambdas 12).
 template <int NX>
 constexpr int kAdjChunk = NX <= 4 ? 16 : 8;
 
