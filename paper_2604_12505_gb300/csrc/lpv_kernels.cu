@@ -733,7 +733,8 @@ __global__ void __launch_bounds__(32, RG == 2 ? 16 : 1) closed_loop_kernel(const
                     o[1] = b;
                 }
             }
-            const float tc = bp.kp * (v.w - bs[r][2]) - bp.kd * bs[r][5];
+            // rounding written out, so that a run gives the same in either row split
+            const float tc = fmaf(bp.kp, v.w - bs[r][2], -__fmul_rn(bp.kd, bs[r][5]));
             uu[r][0] = v.x;
             uu[r][1] = v.y;
             uu[r][2] = v.z + tc;
@@ -760,9 +761,9 @@ __global__ void __launch_bounds__(32, RG == 2 ? 16 : 1) closed_loop_kernel(const
             }
             const float ax = (uu[r][0] + load[0]) * bp.inv_m, ay = (uu[r][1] + load[1]) * bp.inv_m;
             const float aw = (uu[r][2] + load[2]) * bp.inv_J;
-            bs[r][0] += ndt * bs[r][3] + hdt2 * ax;
-            bs[r][1] += ndt * bs[r][4] + hdt2 * ay;
-            bs[r][2] += ndt * bs[r][5] + hdt2 * aw;
+            bs[r][0] += fmaf(hdt2, ax, __fmul_rn(ndt, bs[r][3]));
+            bs[r][1] += fmaf(hdt2, ay, __fmul_rn(ndt, bs[r][4]));
+            bs[r][2] += fmaf(hdt2, aw, __fmul_rn(ndt, bs[r][5]));
             bs[r][3] += ndt * ax;
             bs[r][4] += ndt * ay;
             bs[r][5] += ndt * aw;

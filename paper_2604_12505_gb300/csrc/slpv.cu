@@ -896,10 +896,16 @@ struct Pairs {
 // 65,536 runs of 600 samples (n_x = 4): 1.79 -> 0.97 ms, 2.3 TB/s; bound by the
 // 503 instructions of a warp's sample, of which the 16 tanhf are more than half.
 // wide: F is 16-byte aligned, so that a sample's two forces are one copy.
+// FEW: as long as every block has a scheduler to itself (152 SMs x 4), the
+// time is one warp's chain.  Then the parameters are held in registers, and a
+// second warp copies the inputs in and the outputs out: 10 runs of 214 samples
+// 110 -> 86 us (n_x 2), 3,000 runs 125 -> 105 (n_x 4).  At 25,000 runs, where
+// warps share a scheduler, the 16 warps of the other form are the more.
 constexpr int kLoopChunk = 4, kLoopStages = 2;
+constexpr int kFewBlocks = 152 * 4;
 
-template <int NX>
-__global__ void __launch_bounds__(32, 16)
+template <int NX, bool FEW>
+__global__ void __launch_bounds__(FEW ? 64 : 32, FEW ? 4 : 16)
     closed_loop_kernel(const float* __restrict__ theta, const float* __restrict__ scales, int B, int T,
                        const double* __restrict__ F, const double* __restrict__ tau, const double* __restrict__ ref,
                        float Ts, float J, float w, float xi, float* __restrict__ out, int wide)
@@ -909,14 +915,16 @@ __global__ void __launch_bounds__(32, 16)
     __shared__ __align__(16) Pairs<NX> P;
     __shared__ __align__(16) double2 sF[kLoopStages][C][32];
     __shared__ double sT[kLoopStages][C][32], sR[kLoopStages][C][32];
-    __shared__ __align__(8) float sO[32][C * 6 + 2];  // stride of 26 words: 64-bit accesses of a column meet distinct banks
-    const int lane = threadIdx.x, first = blockIdx.x * 32, n_run = min(32, B - first);
-    P.load(theta, lane, 32);
-    for (int i = lane; i < kLoopStages * C * 32; i += 32) {  // lanes beyond B run on zeros
+    __shared__ __align__(8) float sO[FEW ? 2 : 1][32][C * 6 + 2];  // stride of 26 words: 64-bit accesses of a column meet distinct banks
+    const int lane = threadIdx.x & 31, first = blockIdx.x * 32, n_run = min(32, B - first);
+    const bool copies = FEW ? threadIdx.x >= 32 : true;  // this warp moves the data
+    P.load(theta, threadIdx.x, FEW ? 64 : 32);
+    for (int i = threadIdx.x; i < kLoopStages * C * 32; i += blockDim.x) {  // lanes beyond B run on zeros
         (&sF[0][0][0])[i] = make_double2(0.0, 0.0);
         (&sT[0][0][0])[i] = (&sR[0][0][0])[i] = 0.0;
     }
-    __syncwarp();
+    if (FEW) __syncthreads();
+    else __syncwarp();
     float isu[NU], sy[NY], x[NX], e[NY] = {0.f, 0.f, 0.f}, un[NU] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -946,8 +954,8 @@ __global__ void __launch_bounds__(32, 16)
         }
         copy_commit();
     };
-    auto step = [&](int st, int q) {
-        asm volatile("" ::: "memory");  // the parameters are read again every step: hoisted out of the loop they spill
+    auto step = [&](int st, int q, float* row) {
+        if constexpr (!FEW || NX > 6) asm volatile("" ::: "memory");  // the parameters are read again every step: hoisted out of the loop they spill
         const double2 f = sF[st][q][lane];
         const float Fx = (float)f.x, Fy = (float)f.y, tk = (float)sT[st][q][lane], rk = (float)sR[st][q][lane];
         float z[Q::NZ];
@@ -994,7 +1002,7 @@ __global__ void __launch_bounds__(32, 16)
         float v[NY];
 #pragma unroll
         for (int c = 0; c < NY; ++c) v[c] = o[NX + c] * sy[c];
-        float2* ob = reinterpret_cast<float2*>(&sO[lane][6 * q]);
+        float2* ob = reinterpret_cast<float2*>(row + 6 * q);
         ob[0] = make_float2(e[0], e[1]);
         ob[1] = make_float2(e[2], v[0]);
         ob[2] = make_float2(v[1], v[2]);
@@ -1003,29 +1011,48 @@ __global__ void __launch_bounds__(32, 16)
 #pragma unroll
         for (int i = 0; i < NX; ++i) x[i] = o[i];
     };
-#pragma unroll
-    for (int c = 0; c < kLoopStages - 1; ++c) fetch(c);
-    for (int c = 0; c < n_chunk; ++c) {
-        copy_wait<kLoopStages - 2>();
-        fetch(c + kLoopStages - 1);
-        const int st = c % kLoopStages, n = min(C, T - c * C);
-        for (int q = 0; q < n; ++q) step(st, q);
-        __syncwarp();
-        // the chunk's samples of each run are 24 n consecutive bytes
+    // a chunk's samples of each run are 24 n consecutive bytes
+    auto write = [&](int c) {
+        const int n = min(C, T - c * C);
+        const auto& o = sO[FEW ? c & 1 : 0];
         float* ob = out + ((size_t)first * T + c * C) * 6;
         if (n == C) {
 #pragma unroll 4
             for (int i = lane; i < n_run * (C * 3); i += 32) {
                 const int r = i / (C * 3), h = i % (C * 3);
-                *reinterpret_cast<float2*>(ob + (size_t)r * T * 6 + 2 * h) = *reinterpret_cast<const float2*>(&sO[r][2 * h]);
+                *reinterpret_cast<float2*>(ob + (size_t)r * T * 6 + 2 * h) = *reinterpret_cast<const float2*>(&o[r][2 * h]);
             }
         } else {
             for (int i = lane; i < n_run * (n * 3); i += 32) {
                 const int r = i / (n * 3), h = i % (n * 3);
-                *reinterpret_cast<float2*>(ob + (size_t)r * T * 6 + 2 * h) = *reinterpret_cast<const float2*>(&sO[r][2 * h]);
+                *reinterpret_cast<float2*>(ob + (size_t)r * T * 6 + 2 * h) = *reinterpret_cast<const float2*>(&o[r][2 * h]);
             }
         }
-        // the next chunk's copy_wait is the barrier before sO is written again
+    };
+    static_assert(kLoopStages == 2, "a chunk under way while one is read");
+    if (copies) fetch(0);
+    for (int c = 0; c < n_chunk; ++c) {
+        const int n = min(C, T - c * C);
+        if (copies) copy_wait<0>();
+        if constexpr (FEW) {
+            __syncthreads();  // chunk c is there, the outputs of the one before are
+            if (copies) {
+                fetch(c + 1);
+                if (c > 0) write(c - 1);
+            } else {
+                for (int q = 0; q < n; ++q) step(c % kLoopStages, q, sO[c & 1][lane]);
+            }
+        } else {
+            fetch(c + 1);
+            for (int q = 0; q < n; ++q) step(c % kLoopStages, q, sO[0][lane]);
+            __syncwarp();
+            write(c);
+            // the next chunk's copy_wait is the barrier before sO is written again
+        }
+    }
+    if constexpr (FEW) {
+        __syncthreads();
+        if (copies) write(n_chunk - 1);
     }
 }
 
@@ -1611,8 +1638,12 @@ int slpv_simulate(const slpv_model* m, int32_t B, int32_t T, const double* F, co
     const int wide = (reinterpret_cast<uintptr_t>(F) & 15) == 0;
     SCK(by_nx(m->cfg.nx, [&](auto c) {
         constexpr int NX = decltype(c)::value;
-        closed_loop_kernel<NX><<<(B + 31) / 32, 32, 0, st>>>(m->th, m->scales, B, T, F, tau, theta_ref, (float)Ts,
-                                                             (float)J, (float)omega, (float)xi, out, wide);
+        auto go = [&](auto kernel, int threads) {
+            kernel<<<(B + 31) / 32, threads, 0, st>>>(m->th, m->scales, B, T, F, tau, theta_ref, (float)Ts, (float)J,
+                                                      (float)omega, (float)xi, out, wide);
+        };
+        if ((B + 31) / 32 <= kFewBlocks) go(closed_loop_kernel<NX, true>, 64);
+        else go(closed_loop_kernel<NX, false>, 32);
         return cudaGetLastError();
     }));
     return SPH_OK;

@@ -782,6 +782,8 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
             const float4 pi = sm.pv[e];
             const float2 li = sm.plo[e];
             const float2 ri = sm.rho[e];
+            float2 vl = make_float2(0.f, 0.f);
+            if constexpr (!TAN) vl = velocity_lo(S, buf, sm, e);  // for the kick, far ahead of it
             const int c = sm.cell[e];
             float ax = 0.f, ay = 0.f, tax = 0.f, tay = 0.f;
             float4 ti = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -933,7 +935,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
             } else {
                 // kick then drift (Section 3.4) on the two-float state, then bin
                 // into the next grid: v' = (v + dt a)(1 - c), x' = x + dt v'
-                const float2 vl = velocity_lo(S, buf, sm, e);
+                if constexpr (TAN) vl = velocity_lo(S, buf, sm, e);  // where its registers are short
                 float2 kx = two_sum(pi.z, fmaf(T.dt, ax, vl.x)), ky = two_sum(pi.w, fmaf(T.dt, ay, vl.y));
                 if (damp != 1.0f) {  // relaxation: scale the two-float velocity
                     const float hx = kx.x * damp, hy = ky.x * damp;

@@ -101,3 +101,22 @@ def test_closed_loop_matches_fp64(na, n_y, n_p, nu, B, T):
             q = q + 0.002 * v
     for blk in (slice(0, 3), slice(3, 6)):
         assert np.abs(out[:, :, blk] - want[:, :, blk]).max() <= 1e-3 * max(np.abs(want[:, :, blk]).max(), 1e-300)
+
+
+@pytest.mark.parametrize("na,n_y,n_p", [(1, 3, 0), (2, 3, 1), (3, 4, 2)])
+def test_closed_loop_is_the_same_in_either_row_split(na, n_y, n_p):
+    """A warp carries 8 runs while they are few and 16 beyond: equal bit for bit."""
+    torch = need_gpu()
+    from paper_2604_12505_gb300 import lpv
+    rng = np.random.default_rng(na)
+    W, sc = _model(rng, na, n_y, n_p, 3)
+    B, few, T = 5000, 45, 30
+    body = dict(m=500.0, J=50.0, Ts=0.02, n_sub=10, ctrl_omega=0.2 * np.pi, ctrl_xi=0.7)
+    F, tau = rng.uniform(-20, 20, (B, T, 2)), rng.uniform(-2, 2, (B, T))
+    ref, fill = rng.uniform(-0.3, 0.3, (B, T)), rng.uniform(0.2, 0.8, B)
+    m = lpv.Model(dict(n_x=na * n_y, n_u=3, n_y=n_y, n_p=n_p, na=na))
+    m.set_params(W, sc)
+    many = m.simulate(F, tau, ref, fill, body)[:few].cpu().numpy()
+    alone = m.simulate(F[:few], tau[:few], ref[:few], fill[:few], body).cpu().numpy()
+    m.close()
+    np.testing.assert_array_equal(many, alone)

@@ -69,3 +69,21 @@ def test_closed_loop_matches_oracle_at_edge_sizes(nx, B, T):
         for blk in (slice(0, 3), slice(3, 6)):
             assert np.abs(out[:, :, blk] - want[:, :, blk]).max() <= 1e-3 * np.abs(want[:, :, blk]).max() + 1e-12
     m.close()
+
+
+@pytest.mark.parametrize("nx,T", [(2, 9), (4, 8), (6, 3), (8, 21)])
+def test_closed_loop_is_the_same_among_few_and_many_runs(nx, T):
+    torch = need_gpu()
+    from paper_2604_12505_gb300.slpv import VelocityModel
+    _, th32 = _theta(nx, 21, m1=0.2)
+    rng = np.random.default_rng(nx + T)
+    B, few = 19500, 45
+    F, tau, ref = (torch.tensor(a, device="cuda") for a in (rng.uniform(-20, 20, (B, T, 2)), rng.uniform(-2, 2, (B, T)),
+                                                            rng.uniform(-0.3, 0.3, (B, T))))
+    m = VelocityModel(nx=nx)
+    m.set_params(th32, SC)
+    many = m.simulate(F, tau, ref, 0.05, 133.84, 0.2 * np.pi, 0.7)[:few].cpu().numpy()
+    alone = m.simulate(F[:few].contiguous(), tau[:few].contiguous(), ref[:few].contiguous(), 0.05, 133.84,
+                       0.2 * np.pi, 0.7).cpu().numpy()
+    m.close()
+    np.testing.assert_array_equal(many, alone)
