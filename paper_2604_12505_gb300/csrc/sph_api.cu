@@ -307,6 +307,16 @@ TankDev make_tank_dev(const TankHost& t)
     return d;
 }
 
+// 4x4 tiles of a tank that hold fluid at the start.
+int filled_tiles(const TankHost& t)
+{
+    const int nt = (t.G + 3) / 4;
+    std::vector<char> in((size_t)nt * nt, 0);
+    auto at = [&](double x) { return std::min(std::max((int)std::floor((x + t.W) / t.cell) / 4, 0), nt - 1); };
+    for (int i = 0; i < t.n_f; ++i) in[(size_t)at(t.xf[2 * i + 1]) * nt + at(t.xf[2 * i])] = 1;
+    return (int)std::count(in.begin(), in.end(), 1);
+}
+
 int create_impl(const sph_params* p, int B, cudaStream_t st, sph_sim** out)
 {
     if (!p || !out || B < 1) return fail(SPH_E_INVAL, "sph_create: NULL argument or B < 1");
@@ -425,17 +435,23 @@ int create_impl(const sph_params* p, int B, cudaStream_t st, sph_sim** out)
         max_groups = std::max(max_groups, ng);
     }
     s->tile_code = 3;
-    // Four lanes per particle while the tiles are at most four to an SM: two
-    // 512-thread CTAs have a place there at once, and about half of the tiles
-    // hold fluid.  On 152 SMs, us a step against a thread per particle: 255
-    // tiles (17 tanks of 138 particles) 20.2 / 25.7, 263 (18,696 particles at
-    // the paper's h) 28.6 / 41.2, 551 (29,272) 22.7 / 27.7; more tiles wait for
-    // a second round: 701 (38,348) 31.9 / 27.8, 813 (three tanks) 30.3 / 30.1,
-    // 960 (64 tanks of 138) 30.1 / 27.9.
+    // Four lanes per particle while all tiles that hold fluid (at the start) have
+    // a place at once, two 512-thread CTAs on an SM, and there are at most four
+    // tiles to an SM in all.  On 152 SMs, us a step against a thread per
+    // particle, by tiles (filled): 255 (17 tanks of 138 particles) 20.2 / 25.7;
+    // 263 (18,696 particles at the paper's h) 28.6 / 41.2; 551 (290; 29,272)
+    // 22.7 / 27.7.  The rest wait for a second round: 565 (395; 39,400) 10 steps
+    // 426 / 370, 701 (38,348) 31.9 / 27.8, 813 (three tanks) 30.3 / 30.1, 960
+    // (64 tanks of 138) 30.1 / 27.9.
     int sms = 0, device = 0;
     cudaGetDevice(&device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     s->S.lanes = s->n_tiles[3] <= 4 * sms;
+    if (s->S.lanes) {
+        int filled = 0;
+        for (const TankHost& t : s->tanks) filled += filled_tiles(t);
+        s->S.lanes = filled <= 2 * sms;
+    }
     bool fits = true;
     for (const TankHost& t : s->tanks) fits = fits && resident_fits(t.n_f, t.n_g, t.G);
 
