@@ -898,9 +898,10 @@ struct Pairs {
 // wide: F is 16-byte aligned, so that a sample's two forces are one copy.
 // FEW: as long as every block has a scheduler to itself (152 SMs x 4), the
 // time is one warp's chain.  Then the parameters are held in registers, and a
-// second warp copies the inputs in and the outputs out: 10 runs of 214 samples
-// 110 -> 86 us (n_x 2), 3,000 runs 125 -> 105 (n_x 4).  At 25,000 runs, where
-// warps share a scheduler, the 16 warps of the other form are the more.
+// second warp copies the inputs in, converts them, and copies the outputs
+// out: 10 runs of 214 samples 110 -> 72 us (n_x 2), 3,000 runs 125 -> 86 (n_x
+// 4).  At 25,000 runs, where warps share a scheduler, the 16 warps of the other
+// form are the more.
 constexpr int kLoopChunk = 4, kLoopStages = 2;
 constexpr int kFewBlocks = 152 * 4;
 
@@ -915,6 +916,7 @@ __global__ void __launch_bounds__(FEW ? 64 : 32, FEW ? 4 : 16)
     __shared__ __align__(16) Pairs<NX> P;
     __shared__ __align__(16) double2 sF[kLoopStages][C][32];
     __shared__ double sT[kLoopStages][C][32], sR[kLoopStages][C][32];
+    __shared__ __align__(16) float4 sI[FEW ? 2 : 1][FEW ? C : 1][32];  // FEW: the inputs as FP32
     __shared__ __align__(8) float sO[FEW ? 2 : 1][32][C * 6 + 2];  // stride of 26 words: 64-bit accesses of a column meet distinct banks
     const int lane = threadIdx.x & 31, first = blockIdx.x * 32, n_run = min(32, B - first);
     const bool copies = FEW ? threadIdx.x >= 32 : true;  // this warp moves the data
@@ -954,10 +956,17 @@ __global__ void __launch_bounds__(FEW ? 64 : 32, FEW ? 4 : 16)
         }
         copy_commit();
     };
-    auto step = [&](int st, int q, float* row) {
-        if constexpr (!FEW || NX > 6) asm volatile("" ::: "memory");  // the parameters are read again every step: hoisted out of the loop they spill
+    auto input = [&](int st, int q) {
         const double2 f = sF[st][q][lane];
-        const float Fx = (float)f.x, Fy = (float)f.y, tk = (float)sT[st][q][lane], rk = (float)sR[st][q][lane];
+        return make_float4((float)f.x, (float)f.y, (float)sT[st][q][lane], (float)sR[st][q][lane]);
+    };
+    auto convert = [&](int c) {
+#pragma unroll
+        for (int q = 0; q < C; ++q) sI[c & 1][q][lane] = input(c % kLoopStages, q);
+    };
+    auto step = [&](const float4& in, int q, float* row) {
+        if constexpr (!FEW || NX > 6) asm volatile("" ::: "memory");  // the parameters are read again every step: hoisted out of the loop they spill
+        const float Fx = in.x, Fy = in.y, tk = in.z, rk = in.w;
         float z[Q::NZ];
         float2 ax[NH / 2], a[NH / 2];
 #pragma unroll
@@ -1031,20 +1040,29 @@ __global__ void __launch_bounds__(FEW ? 64 : 32, FEW ? 4 : 16)
     };
     static_assert(kLoopStages == 2, "a chunk under way while one is read");
     if (copies) fetch(0);
+    if constexpr (FEW) {
+        if (copies) {
+            copy_wait<0>();
+            convert(0);
+            fetch(1);
+        }
+    }
     for (int c = 0; c < n_chunk; ++c) {
         const int n = min(C, T - c * C);
-        if (copies) copy_wait<0>();
         if constexpr (FEW) {
             __syncthreads();  // chunk c is there, the outputs of the one before are
             if (copies) {
-                fetch(c + 1);
+                copy_wait<0>();
+                convert(c + 1);
+                fetch(c + 2);
                 if (c > 0) write(c - 1);
             } else {
-                for (int q = 0; q < n; ++q) step(c % kLoopStages, q, sO[c & 1][lane]);
+                for (int q = 0; q < n; ++q) step(sI[c & 1][q][lane], q, sO[c & 1][lane]);
             }
         } else {
+            copy_wait<0>();
             fetch(c + 1);
-            for (int q = 0; q < n; ++q) step(c % kLoopStages, q, sO[0][lane]);
+            for (int q = 0; q < n; ++q) step(input(c % kLoopStages, q), q, sO[0][lane]);
             __syncwarp();
             write(c);
             // the next chunk's copy_wait is the barrier before sO is written again
