@@ -1102,6 +1102,7 @@ int sph_vjp(sph_sim* sim, const double* u, int32_t K, const double* ybar, const 
         }
         CK(launch_recorded(R, sim->d_part_tank, sim->n_cells_total, sim->n_tiles[code], k1 - k0, st));
         if ((rc = reverse(k0, k1))) return rc;
+        CK(launch_record_flags(R, lane.body, k1 - k0, st));
     }
     if (K > 0) {  // leave the simulator at the final state, as sph_jvp does
         CK(launch_adjoint_body(R.first, A, 1, 0, st, true));

@@ -403,6 +403,17 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, Shape<TX, TY>::DENSITY
     density_pass<TX, TY, false, true>(S, EvalOut{}, 0, 0, (R.buf0 + (int)blockIdx.y) & 1);
 }
 
+// The health flags that the recorded steps raised in body records of their own
+// (the densities' and the adjoint's passes in R's, the run that recorded them
+// in `lane`), to the simulator's.  One thread per body record.
+__global__ void rec_flags_kernel(RecordDev R, const BodyDev* __restrict__ lane, int steps)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, B = R.first.B;
+    if (i >= (steps + 1) * B) return;
+    const int f = i < steps * B ? R.first.body[i].flags : lane[i - steps * B].flags;
+    if (f) atomicOr(R.flags + (size_t)(i % B) * R.flags_stride, f);
+}
+
 // ---------------------------------------------------------------------------
 // Block reductions (fixed order: deterministic)
 // ---------------------------------------------------------------------------
@@ -1387,6 +1398,12 @@ cudaError_t launch_recorded(const RecordDev& R, const int* part_tank, int n_cell
     rec_body_kernel<<<dim3((R.first.B + 127) / 128, steps), 128, 0, st>>>(R);
     rec_bin_kernel<<<dim3((n_cells_total + 7) / 8, steps), 256, 0, st>>>(R, part_tank, n_cells_total);
     rec_density_kernel<4, 4><<<dim3(n_tiles, steps), Sh::THREADS, 0, st>>>(R);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_record_flags(const RecordDev& R, const BodyDev* lane, int steps, cudaStream_t st)
+{
+    rec_flags_kernel<<<((steps + 1) * R.first.B + 255) / 256, 256, 0, st>>>(R, lane, steps);
     return cudaGetLastError();
 }
 

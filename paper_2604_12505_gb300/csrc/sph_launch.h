@@ -81,6 +81,8 @@ struct RecordDev {
 // The body records, re-binned states and density passes (4x4 tiles) of `steps` recorded steps.
 cudaError_t launch_recorded(const RecordDev& R, const int* part_tank, int n_cells_total, int n_tiles, int steps,
                             cudaStream_t st);
+// The health flags of `steps` reversed steps, and of the run that recorded them, to R.flags.
+cudaError_t launch_record_flags(const RecordDev& R, const BodyDev* lane, int steps, cudaStream_t st);
 
 // Reverse-mode step (sph_adjoint.cu) over a recorded step: S points at its
 // records (launch_recorded), buf is the buffer of its state.  Adjoint arrays are indexed by particle index (the order of sph_get_state); body
