@@ -40,7 +40,9 @@
 //
 // Every buffer is sized for all of the tank's particles in one CTA: wherever
 // the fluid goes, nothing overflows.  That bounds the tanks this kernel takes
-// (resident_fits).
+// (resident_fits).  A tile with more particles around it than the step kernels
+// stage raises SPH_FLAG_STAGE_FULL as it does there, so that a tank is not
+// accepted or refused by the length of the call.
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -61,6 +63,7 @@ constexpr int kSlots = kThreads / kLanes;  // particles that a pass takes at onc
 constexpr int kSortThreads = kThreads - 32;  // the last warp updates the body meanwhile
 constexpr int kTile = 4;            // cells per tile side, as the default tile of the step kernels
 constexpr int kTileThreads = 128;   // threads that a tile has there: own particle t is summed by thread t % 128
+constexpr int kStage = Shape<kTile, kTile>::MAXS;  // particles that a tile stages there, with its halo
 constexpr int kMine = 4;            // particles of a sorting thread
 constexpr unsigned short kNone = 0xffff;
 constexpr unsigned kOwn = 1u << 31;
@@ -484,6 +487,13 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
             }
             sh.row[i][kTile] = (unsigned short)acc;
             if (acc > kTileThreads) atomicMax(&sh.most, acc);
+            // a tank that the step kernels cannot stage is refused here too
+            if (acc > 0 && n_in > kStage) {
+                const int first = (int)sh.at[i] - P - 1, wide = sh.across[i] + 2;
+                int around = 0;
+                for (int r = 0; r < sh.down[i] + 2; ++r) around += (int)start[first + r * P + wide] - (int)start[first + r * P];
+                if (around > kStage) atomicOr(&sh.flags, SPH_FLAG_STAGE_FULL);
+            }
         }
         const int first = warp * (32 / kLanes);  // the warp's first particle, and this lane's
         const int mine = tid / kLanes;
