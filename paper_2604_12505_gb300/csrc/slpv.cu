@@ -895,13 +895,15 @@ struct Pairs {
 // SM of 65,536 runs resident (in registers they allowed eight).
 // 65,536 runs of 600 samples (n_x = 4): 1.79 -> 0.97 ms, 2.3 TB/s; bound by the
 // 503 instructions of a warp's sample, of which the 16 tanhf are more than half.
-// wide: F is 16-byte aligned, so that a sample's two forces are one copy.
+// wide: kWideF, F is 16-byte aligned, so that a sample's two forces are one copy;
+// kWideOut, out is 8-byte aligned, so that two values are one store.
 // FEW: as long as every block has a scheduler to itself (152 SMs x 4), the
 // time is one warp's chain.  Then the parameters are held in registers, and a
 // second warp copies the inputs in, converts them, and copies the outputs
 // out: 10 runs of 214 samples 110 -> 72 us (n_x 2), 3,000 runs 125 -> 86 (n_x
 // 4).  At 25,000 runs, where warps share a scheduler, the 16 warps of the other
 // form are the more.
+enum { kWideF = 1, kWideOut = 2 };
 constexpr int kLoopChunk = 4, kLoopStages = 2;
 constexpr int kFewBlocks = 152 * 4;
 
@@ -944,7 +946,7 @@ __global__ void __launch_bounds__(FEW ? 64 : 32, FEW ? 4 : 16)
             for (int r = lane / C; r < 32; r += 32 / C)
                 if (r < n_run) {
                     const size_t o = (size_t)(first + r) * T + k;
-                    if (wide) {
+                    if (wide & kWideF) {
                         copy_async<16>(&sF[st][cs][r], F + 2 * o);
                     } else {
                         copy_async<8>(&sF[st][cs][r].x, F + 2 * o);
@@ -1025,16 +1027,16 @@ __global__ void __launch_bounds__(FEW ? 64 : 32, FEW ? 4 : 16)
         const int n = min(C, T - c * C);
         const auto& o = sO[FEW ? c & 1 : 0];
         float* ob = out + ((size_t)first * T + c * C) * 6;
-        if (n == C) {
+        if (n == C && (wide & kWideOut)) {
 #pragma unroll 4
             for (int i = lane; i < n_run * (C * 3); i += 32) {
                 const int r = i / (C * 3), h = i % (C * 3);
                 *reinterpret_cast<float2*>(ob + (size_t)r * T * 6 + 2 * h) = *reinterpret_cast<const float2*>(&o[r][2 * h]);
             }
         } else {
-            for (int i = lane; i < n_run * (n * 3); i += 32) {
-                const int r = i / (n * 3), h = i % (n * 3);
-                *reinterpret_cast<float2*>(ob + (size_t)r * T * 6 + 2 * h) = *reinterpret_cast<const float2*>(&o[r][2 * h]);
+            for (int i = lane; i < n_run * (n * 6); i += 32) {
+                const int r = i / (n * 6), h = i % (n * 6);
+                ob[(size_t)r * T * 6 + h] = o[r][h];
             }
         }
     };
@@ -1653,7 +1655,8 @@ int slpv_simulate(const slpv_model* m, int32_t B, int32_t T, const double* F, co
     if (!m || !F || !tau || !theta_ref || !out || B < 1 || T < 1) return inval("slpv_simulate: NULL pointer or empty");
     if (!(Ts > 0.0) || !(J > 0.0)) return inval("slpv_simulate: Ts and J must be > 0");
     cudaStream_t st = (cudaStream_t)stream;
-    const int wide = (reinterpret_cast<uintptr_t>(F) & 15) == 0;
+    const int wide = ((reinterpret_cast<uintptr_t>(F) & 15) == 0 ? kWideF : 0) |
+                     ((reinterpret_cast<uintptr_t>(out) & 7) == 0 ? kWideOut : 0);
     SCK(by_nx(m->cfg.nx, [&](auto c) {
         constexpr int NX = decltype(c)::value;
         auto go = [&](auto kernel, int threads) {
