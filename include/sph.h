@@ -278,10 +278,11 @@ int sph_eval_jvp(sph_sim* sim, const double* u, const double* du, const float* d
  * The forward pass keeps a checkpoint every checkpoint_every steps; each
  * segment is run again from its checkpoint with its steps recorded, and the
  * adjoint kernels run backwards over the records on 4x4 tiles.  Device memory:
- * K / checkpoint_every states for the call, and records of up to 2 GB (more
- * where the checkpoints and a segment's states take more, a step's at least,
- * and less where the device has no room), which the handle keeps for its next
- * call.  The simulator is left at state K, as after sph_jvp.  Blocks until done.
+ * K / checkpoint_every states for the call, and records of up to 2 GiB (a
+ * step's at least, and less where the device has no room).  The handle keeps
+ * the records for its next call, until it is destroyed, as far as those that
+ * all handles of the process keep come to 8 GiB together.  The simulator is
+ * left at state K, as after sph_jvp.  Blocks until done.
  */
 int sph_vjp(sph_sim* sim, const double* u, int32_t K, const double* ybar, const float* xvbar_K,
             const double* bodybar_K, float* xvbar0, double* bodybar0, double* ubar, int32_t checkpoint_every,
