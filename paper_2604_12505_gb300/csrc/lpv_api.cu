@@ -22,7 +22,7 @@ struct lpv_model {
     lpv_config cfg{};
     Dims d{};
     float *Wp = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
-    float* hist = nullptr;  // fragments of z_k and of G_k of every step (launch_forward)
+    float* hist = nullptr;  // state and residuals of every step (launch_forward)
     size_t hist_cap = 0;
     float* gpart = nullptr;
     double* loss_part = nullptr;
@@ -88,7 +88,7 @@ int workspace(lpv_model* M, int n_traj, int T)
             return err(SPH_E_NOMEM, "lpv: cudaMalloc failed");
         M->part_cap = parts;
     }
-    return grow(&M->hist, &M->hist_cap, 2 * frag_floats(n_traj, T));
+    return grow(&M->hist, &M->hist_cap, hist_floats(n_traj, T));
 }
 
 int check_data(const lpv_model* M, const float* u, const float* y, const float* p, int n_traj, int T)
@@ -277,9 +277,8 @@ int loss_grad_device(lpv_model* M, const float* u, const float* y, const float* 
     int rc = workspace(M, n_traj, T);
     if (rc) return rc;
     const double n = (double)n_traj * T;
-    float* gfrag = M->hist + frag_floats(n_traj, T);
-    LCK(launch_forward(1, M->Wp, M->d, u, p, y, n_traj, T, nullptr, M->hist, gfrag, M->loss_part, (float)(2.0 / n), st));
-    LCK(launch_backward(M->Wp, M->d, p, n_traj, T, M->hist, gfrag, M->gpart, st));
+    LCK(launch_forward(1, M->Wp, M->d, u, p, y, n_traj, T, nullptr, M->hist, M->loss_part, (float)(2.0 / n), st));
+    LCK(launch_backward(M->Wp, M->d, u, p, n_traj, T, M->hist, M->gpart, st));
     LCK(launch_reduce(M->gpart, grad_parts(n_traj), M->loss_part, serial_warps(n_traj), M->Wp, M->d, M->cfg.sigma2, n,
                       M->grad, M->d_loss, loss_hist, it, st));
     return SPH_OK;
@@ -514,8 +513,7 @@ int lpv_predict(const lpv_model* M, const float* u, const float* p, int32_t n_tr
                 void* stream)
 {
     if (!M || !u || !y_out || n_traj < 1 || T < 1 || (M->d.np > 0 && !p)) return err(SPH_E_INVAL, "lpv_predict: bad arguments");
-    LCK(launch_forward(0, M->Wp, M->d, u, p, nullptr, n_traj, T, y_out, nullptr, nullptr, nullptr, 0.f,
-                       (cudaStream_t)stream));
+    LCK(launch_forward(0, M->Wp, M->d, u, p, nullptr, n_traj, T, y_out, nullptr, nullptr, 0.f, (cudaStream_t)stream));
     return SPH_OK;
 }
 

@@ -21,6 +21,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
+#include <cstddef>
 #include <cstdint>
 #include <type_traits>
 
@@ -112,7 +114,7 @@ __device__ __forceinline__ void load_fwd_frags(const float* __restrict__ Wp, uin
 //
 // Serial in k are the state and its adjoint, each a product of the split
 // operands per step; everything else runs beside or after them:
-//   fwd_kernel     the free run: z_k fragments and residuals for the adjoint
+//   fwd_kernel     the free run: x_k and the residuals for the adjoint
 //   adj_kernel     lambda_k and, in other warps, sum_k G_k^T w_k with
 //                  G_k = [lambda_{k+1}; dJ/dy_k]
 // The serial passes are bound by the instructions of one warp's step, which
@@ -124,18 +126,21 @@ __device__ __forceinline__ void load_fwd_frags(const float* __restrict__ Wp, uin
 // but so is half of the work per step around the product, and a step is
 // shorter.  Runs that leave schedulers idle anyway take RG = 1
 // (row_groups).  820 trajectories of 1,000 samples (n_x 12, n_u 3, n_y 4,
-// n_p 2): 174 us forward, 189 us adjoint and gradient, 6 us reduction.  Four
+// n_p 2): 175 us forward, 173 us adjoint and gradient, 6 us reduction.  Four
 // warps to a block that loaded u, y and p from their rows (28 memory
 // instructions of up to 16 lines a step) and kept the weight gradient, with
 // its transposes through shared memory, on the adjoint's chain took 1,939 +
 // 1,469 + 31 us.
 //
-// Fragments in global memory: per group of 8 trajectories and step, [lane][4],
-// the values of columns 2t, 2t+1, 2t+8, 2t+9 of row g.
+// What the free run leaves for the adjoint is a row of 16 floats per trajectory
+// and step, hist[traj][k]: the state in the first n_x columns, the residuals'
+// part of G_k after it, the columns in the lanes' order (2t, 2t+1, 2t+8, 2t+9
+// at place 4t).  (As two fragments of 8 rows, z_k and G_k, it took twice the
+// room, 32 times for one trajectory, in the same time.)
 // ---------------------------------------------------------------------------
 constexpr int kC = 4;         // steps per chunk of staged inputs
 constexpr int kStages = 4;    // chunks in shared memory: one in use, three in flight
-constexpr int kFrag = kFragFloats;
+constexpr int kFrag = 128;    // floats of a step of 8 trajectories, [lane][4]
 
 template <int BYTES>
 __device__ __forceinline__ void copy_async(void* dst, const void* src)
@@ -261,14 +266,12 @@ __device__ __forceinline__ void product(float* D, const float* z, const float (*
 
 // Free-run simulation of 8 RG trajectories per warp.  MODE 0 writes the
 // prediction (physical units); MODE 1 accumulates the squared error of the
-// normalised outputs and records, per step, z_k and the residuals' part of
-// G_k as fragments.
+// normalised outputs and records x_k and the residuals' part of G_k.
 template <int MODE, bool LOW, int NP, int RG>
 __global__ void __launch_bounds__(32) fwd_kernel(const float* __restrict__ Wp, Dims d, const float* __restrict__ u,
                                                  const float* __restrict__ p, const float* __restrict__ y, int n_traj,
-                                                 int T, float* __restrict__ y_out, float* __restrict__ zfrag,
-                                                 float* __restrict__ gfrag, double* __restrict__ loss_part,
-                                                 float grad_scale)
+                                                 int T, float* __restrict__ y_out, float* __restrict__ hist,
+                                                 double* __restrict__ loss_part, float grad_scale)
 {
     __shared__ __align__(16) InStage<LOW, RG> sm[kStages];
     const int lane = threadIdx.x, g = lane >> 2, t = lane & 3, wid = blockIdx.x, first = wid * 8 * RG;
@@ -320,8 +323,14 @@ __global__ void __launch_bounds__(32) fwd_kernel(const float* __restrict__ Wp, D
     for (int c = 0; c < kStages - 1; ++c) fetch(c);
     float s[RG][4] = {};   // x_0 = 0; zero in the columns that hold no state
     float lsum_f = 0.f;    // widened to FP64 once, after the loop
-    float4* zo = reinterpret_cast<float4*>(zfrag) + (size_t)wid * RG * T * (kFrag / 4) + lane;
-    float4* go = reinterpret_cast<float4*>(gfrag) + (size_t)wid * RG * T * (kFrag / 4) + lane;
+    float* ho[RG];         // where this lane's part of the next row goes; beyond the data always the spare row
+    int h_step[RG];
+#pragma unroll
+    for (int r = 0; r < RG; ++r) {
+        const int tr = min(first + 8 * r + g, n_traj);
+        ho[r] = hist + (size_t)tr * T * 16 + 4 * t;
+        h_step[r] = tr < n_traj ? 16 : 0;
+    }
     auto step = [&](const InStage<LOW, RG>& S, int q, int k) {
         float z[8], pp[RG][2];
 #pragma unroll
@@ -338,8 +347,6 @@ __global__ void __launch_bounds__(32) fwd_kernel(const float* __restrict__ Wp, D
 #pragma unroll
             for (int j = 0; j < 4; ++j)  // at a column either the state or the input is zero: the sum is exact
                 z[4 * (j >> 1) + 2 * r + (j & 1)] = LOW || j >= 2 ? s[r][j] + uv[j] * fu[j] : s[r][j];
-            if (MODE == 1)
-                zo[((size_t)r * T + k) * 32] = make_float4(z[2 * r], z[2 * r + 1], z[4 + 2 * r], z[5 + 2 * r]);
         }
         float D[8];
         product<NP, RG>(D, z, pp, bhi, blo);
@@ -360,7 +367,13 @@ __global__ void __launch_bounds__(32) fwd_kernel(const float* __restrict__ Wp, D
                     res[j] *= grad_scale;
                 }
             }
-            if (MODE == 1) go[((size_t)r * T + k) * 32] = make_float4(res[0], res[1], res[2], res[3]);
+            if (MODE == 1) {
+                float h[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) h[j] = (LOW || j >= 2) && !is_x[j] ? res[j] : s[r][j];
+                *reinterpret_cast<float4*>(ho[r]) = make_float4(h[0], h[1], h[2], h[3]);
+                ho[r] += h_step[r];
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float o = D[4 * (j >> 1) + 2 * r + (j & 1)];
@@ -423,21 +436,24 @@ __device__ __forceinline__ uint32_t trans8(uint32_t a)
 // over all steps of the 16 trajectories (gpart[block][16][48], added up in
 // FP64 by launch_reduce): sums in other parts were measured and differ from
 // these by up to 7e-5, the rounding of a 1,000-step FP32 tensor-core sum.
+// One block per SM is asked for: the registers that the gradient's warps may
+// take then are what lets four steps overlap (820 trajectories of 1,000
+// samples 173 us, 201 with 79 registers).
 template <int NP>
 constexpr int kAdjWarps = 2 + 2 * (1 + NP);
 
 template <int NP>
 struct AdjStage {
-    float res[kC][2][kFrag];   // residuals' part of G_k (zero elsewhere)
-    float z[kC][2][kFrag];
+    float h[kC][2][kFrag];     // x_k and the residuals' part of G_k
+    float u[kC][16][16];       // inputs at their columns (zero elsewhere)
     float p[kC][16][2];
 };
 
 template <int NP>
-__global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __restrict__ Wp, Dims d,
+__global__ void __launch_bounds__(32 * kAdjWarps<NP>, 1) adj_kernel(const float* __restrict__ Wp, Dims d,
+                                                            const float* __restrict__ u,
                                                             const float* __restrict__ p, int n_traj, int T,
-                                                            const float* __restrict__ zfrag,
-                                                            const float* __restrict__ gfrag,
+                                                            const float* __restrict__ hist,
                                                             float* __restrict__ gpart)
 {
     __shared__ __align__(16) AdjStage<NP> sm[kStages];
@@ -445,33 +461,34 @@ __global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, wl = threadIdx.x >> 5;
     const int first = blockIdx.x * 16, n_chunk = (T + kC - 1) / kC;
     const bool is_adj = wl < 2;
-    const bool two = first + 8 < n_traj;  // the second group of 8 exists (its fragments are not written otherwise)
     {   // rows beyond the data stay zero
         float* z = reinterpret_cast<float*>(sm);
         for (int i = threadIdx.x; i < (int)(sizeof(sm) / sizeof(float)); i += blockDim.x) z[i] = 0.f;
     }
     __syncthreads();
-    const size_t grp = (size_t)blockIdx.x * 2;
-    // chunk c holds steps T - 1 - c kC - q for q = 0, 1, ..
+    // the inputs that this lane copies next, and down to which k0
+    const int u_row = min(first + 8 * ((wl - 2) & 1) + g, n_traj - 1);
+    const float* u_next = u + ((ptrdiff_t)u_row * T + (T - 1 - t)) * d.nu;
+    const int u_from = first + 8 * (wl - 2) + g < n_traj ? t : INT_MAX;
+    // chunk c holds steps T - 1 - c kC - q for q = 0, 1, ..; fetched in order
     auto fetch = [&](int c) {
         AdjStage<NP>& S = sm[c % kStages];
         const int k0 = T - 1 - c * kC;
-        if (is_adj) {  // a warp's residuals, and the p of its rows, a step per lane
-            const float* src = gfrag + ((grp + wl) * T + k0) * kFrag + 4 * lane;
-#pragma unroll
-            for (int q = 0; q < kC; ++q)
-                if (k0 - q >= 0 && (wl == 0 || two)) copy_async<16>(&S.res[q][wl][4 * lane], src - (size_t)q * kFrag);
+        if (is_adj) {  // the history of a warp's rows, and their p, a step per lane
             const int tr = first + 8 * wl + g;
-            if (k0 - t >= 0 && tr < n_traj)
+            if (tr < n_traj) {
+                const float* src = hist + ((size_t)tr * T + k0) * 16 + 4 * t;
 #pragma unroll
-                for (int j = 0; j < NP; ++j)
-                    copy_async<4>(&S.p[t][8 * wl + g][j], p + ((size_t)tr * T + (k0 - t)) * NP + j);
-        } else {
-            for (int i = wl - 2; i < 2 * kC; i += kAdjWarps<NP> - 2) {
-                const int q = i >> 1, r = i & 1;
-                if (k0 - q >= 0 && (r == 0 || two))
-                    copy_async<16>(&S.z[q][r][4 * lane], zfrag + ((grp + r) * T + (k0 - q)) * kFrag + 4 * lane);
+                for (int q = 0; q < kC; ++q)
+                    if (k0 - q >= 0) copy_async<16>(&S.h[q][wl][4 * lane], src - q * 16);
+                if (k0 - t >= 0)
+#pragma unroll
+                    for (int j = 0; j < NP; ++j)
+                        copy_async<4>(&S.p[t][8 * wl + g][j], p + ((size_t)tr * T + (k0 - t)) * NP + j);
             }
+        } else if (wl < 4) {  // the inputs of 8 rows, a step per lane
+            if (k0 >= u_from) copy_row(&S.u[t][8 * (wl - 2) + g][d.nx], u_next, d.nu);
+            u_next -= kC * d.nu;
         }
         copy_commit();
     };
@@ -497,7 +514,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __
         load_bwd_frags<NT>(Wp, bhi, blo, g, t);
         float lam[4] = {0, 0, 0, 0};  // lambda_T = 0
         auto step = [&](const AdjStage<NP>& S, float* out, int q) {
-            const float4 v = *reinterpret_cast<const float4*>(&S.res[q][wl][4 * lane]);
+            const float4 v = *reinterpret_cast<const float4*>(&S.h[q][wl][4 * lane]);
             const float2 pv = *reinterpret_cast<const float2*>(S.p[q][8 * wl + g]);
             const float pp[2] = {(pv.x - pm[0]) * ip[0], (pv.y - pm[1]) * ip[1]};
             // rows 0-7 the high, rows 8-15 the low parts (as in the free run)
@@ -550,12 +567,28 @@ __global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __
         ik[0] = kt == 1 ? ips[0][0] : ips[0][1];
         ik[1] = kt == 1 ? ips[1][0] : ips[1][1];
     }
+    // where this lane's two columns of z_k lie in a stage, in x_k or in u, as
+    // steps and groups of 8 rows are as far apart in both, and their factors
+    int at[2];
+    float2 f;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int c = 8 * h + 2 * t + j - d.nx;
+        at[j] = c < 0 ? 4 * lane + 2 * h + j : kC * 2 * kFrag + 16 * g + 8 * h + 2 * t + j;
+        (j ? f.y : f.x) = c < 0 ? 1.f : c < d.nu ? d.inv_su[c] : 0.f;
+    }
+    static_assert(offsetof(AdjStage<NP>, u) == kC * 2 * kFrag * sizeof(float) && sizeof(AdjStage<NP>::u) == sizeof(AdjStage<NP>::h),
+                  "u follows h, steps and rows as far apart");
     float acc[4] = {0, 0, 0, 0};
-    auto step = [&](const AdjStage<NP>& S, const float* in, int q) {
+    auto step = [&](auto paired, const AdjStage<NP>& S, const float* in, int q) {
         const uint4 ga = *reinterpret_cast<const uint4*>(in + (q * 2) * kFrag + 4 * lane);
         const uint4 gb = *reinterpret_cast<const uint4*>(in + (q * 2 + 1) * kFrag + 4 * lane);
-        float2 za = *reinterpret_cast<const float2*>(&S.z[q][0][4 * lane + 2 * h]);
-        float2 zb = *reinterpret_cast<const float2*>(&S.z[q][1][4 * lane + 2 * h]);
+        auto z = [&](int r) {
+            const float* s = &S.h[0][0][0] + (2 * q + r) * kFrag;
+            const float2 v = decltype(paired)::value ? *reinterpret_cast<const float2*>(s + at[0]) : make_float2(s[at[0]], s[at[1]]);
+            return mul2(v, f);
+        };
+        float2 za = z(0), zb = z(1);
         if (scaled) {
             const float pa = (S.p[q][g][kt - 1] - pk) * ik[0], pb = (S.p[q][8 + g][kt - 1] - pk) * ik[1];
             za = mul2(za, make_float2(pa, pa));
@@ -572,20 +605,25 @@ __global__ void __launch_bounds__(32 * kAdjWarps<NP>) adj_kernel(const float* __
         mma16816(acc, ahi, b0l, b1l);
         mma16816(acc, alo, b0h, b1h);
     };
-    for (int c = 0; c <= n_chunk; ++c) {
-        copy_wait<1>();
-        __syncthreads();
-        if (c < n_chunk) fetch(c + 2);
-        if (c == 0) continue;
-        const AdjStage<NP>& S = sm[(c - 1) % kStages];
-        const float* in = &sG[(c - 1) & 1][0][0][0];
-        if (c * kC <= T) {
+    auto run = [&](auto paired) {
+        for (int c = 0; c <= n_chunk; ++c) {
+            copy_wait<1>();
+            __syncthreads();
+            if (c < n_chunk) fetch(c + 2);
+            if (c == 0) continue;
+            const AdjStage<NP>& S = sm[(c - 1) % kStages];
+            const float* in = &sG[(c - 1) & 1][0][0][0];
+            if (c * kC <= T) {
 #pragma unroll
-            for (int q = 0; q < kC; ++q) step(S, in, q);
-        } else {
-            for (int q = 0; (c - 1) * kC + q < T; ++q) step(S, in, q);
+                for (int q = 0; q < kC; ++q) step(paired, S, in, q);
+            } else {
+                for (int q = 0; (c - 1) * kC + q < T; ++q) step(paired, S, in, q);
+            }
         }
-    }
+    };
+    // both columns of every lane in one of the two: all warps of an even state, and the half of an odd one without its end
+    if (d.nx % 2 == 0 || d.nx / 8 != h) run(std::true_type{});
+    else run(std::false_type{});
     // acc: (o = g, f = 8 h + 2t), (g, +1), (g + 8, 2t), (g + 8, 2t + 1) of block kt
     constexpr int ld = kFB * kMaxKT;
     float* out = gpart + (size_t)blockIdx.x * kWN;
@@ -811,14 +849,14 @@ static void by_np(int np, F&& f)
 }
 
 cudaError_t launch_forward(int mode, const float* Wp, const Dims& d, const float* u, const float* p, const float* y,
-                           int n_traj, int T, float* y_out, float* zfrag, float* gfrag, double* loss_part,
-                           float grad_scale, cudaStream_t st)
+                           int n_traj, int T, float* y_out, float* hist, double* loss_part, float grad_scale,
+                           cudaStream_t st)
 {
     const int warps = serial_warps(n_traj);
     by_np(d.np, [&](auto np) {
         constexpr int NP = decltype(np)::value;
         auto go = [&](auto kernel) {
-            kernel<<<warps, 32, 0, st>>>(Wp, d, u, p, y, n_traj, T, y_out, zfrag, gfrag, loss_part, grad_scale);
+            kernel<<<warps, 32, 0, st>>>(Wp, d, u, p, y, n_traj, T, y_out, hist, loss_part, grad_scale);
         };
         const bool low = d.nx < 8, one = row_groups(n_traj) == 1;
         if (mode == 0) {
@@ -832,12 +870,12 @@ cudaError_t launch_forward(int mode, const float* Wp, const Dims& d, const float
     return cudaGetLastError();
 }
 
-cudaError_t launch_backward(const float* Wp, const Dims& d, const float* p, int n_traj, int T, const float* zfrag,
-                            const float* gfrag, float* gpart, cudaStream_t st)
+cudaError_t launch_backward(const float* Wp, const Dims& d, const float* u, const float* p, int n_traj, int T,
+                            const float* hist, float* gpart, cudaStream_t st)
 {
     by_np(d.np, [&](auto np) {
         constexpr int NP = decltype(np)::value;
-        adj_kernel<NP><<<grad_parts(n_traj), 32 * kAdjWarps<NP>, 0, st>>>(Wp, d, p, n_traj, T, zfrag, gfrag, gpart);
+        adj_kernel<NP><<<grad_parts(n_traj), 32 * kAdjWarps<NP>, 0, st>>>(Wp, d, u, p, n_traj, T, hist, gpart);
     });
     return cudaGetLastError();
 }

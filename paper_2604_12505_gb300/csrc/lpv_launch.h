@@ -13,21 +13,20 @@ struct BodyParHost {
 // Groups of 8 trajectories that n trajectories make.
 inline int groups_for(int n) { return (n + 7) / 8; }
 
-// Fragments in device memory: 128 floats per step of a group of 8
-// trajectories, of an even number of groups.
-constexpr int kFragFloats = 128;
-inline size_t frag_floats(int n_traj, int T) { return (size_t)((groups_for(n_traj) + 1) / 2 * 2) * T * kFragFloats; }
+// The history that launch_forward leaves for launch_backward: a row of 16
+// floats per trajectory and step, and one to spare.
+inline size_t hist_floats(int n_traj, int T) { return (size_t)n_traj * T * 16 + 16; }
 // Warps of the serial passes, and loss partials that launch_forward writes.
 int serial_warps(int n_traj);
-// mode 0: prediction into y_out; mode 1: loss partials per warp, z_k (zfrag)
-// and the residuals' part of G_k (gfrag).
+// mode 0: prediction into y_out; mode 1: loss partials per warp, and x_k and
+// the residuals' part of G_k (hist).
 cudaError_t launch_forward(int mode, const float* Wp, const Dims& d, const float* u, const float* p, const float* y,
-                           int n_traj, int T, float* y_out, float* zfrag, float* gfrag, double* loss_part,
-                           float grad_scale, cudaStream_t st);
+                           int n_traj, int T, float* y_out, float* hist, double* loss_part, float grad_scale,
+                           cudaStream_t st);
 // The adjoint and the weight gradient's partials gpart[grad_parts(n_traj)][768].
 inline int grad_parts(int n_traj) { return (n_traj + 15) / 16; }
-cudaError_t launch_backward(const float* Wp, const Dims& d, const float* p, int n_traj, int T, const float* zfrag,
-                            const float* gfrag, float* gpart, cudaStream_t st);
+cudaError_t launch_backward(const float* Wp, const Dims& d, const float* u, const float* p, int n_traj, int T,
+                            const float* hist, float* gpart, cudaStream_t st);
 cudaError_t launch_closed_loop(const float* Wp, const Dims& d, int B, int T, const double* F, const double* tau,
                                const double* ref, const double* fill, const BodyParHost& bp, double* out,
                                cudaStream_t st);
