@@ -477,23 +477,18 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
         __syncthreads();
         // the rows of the own tiles, for their sums
         if (const int i = kThreads - 1 - tid; i < sh.n_tile) {
-            int acc = 0;
-            for (int r = 0; r < kTile; ++r) {
-                sh.row[i][r] = (unsigned short)acc;
-                if (r < sh.down[i]) {
-                    const int c = sh.at[i] + r * P;
-                    acc += (int)start[c + sh.across[i]] - (int)start[c];
-                }
+            int acc = 0, around = 0;
+            const int at = sh.at[i], wide = sh.across[i], high = sh.down[i];
+#pragma unroll
+            for (int r = -1; r <= kTile; ++r) {
+                const int c = at + r * P;
+                if (r >= 0) sh.row[i][r] = (unsigned short)acc;
+                if (r >= 0 && r < high) acc += (int)start[c + wide] - (int)start[c];
+                if (r <= high) around += (int)start[c + wide + 1] - (int)start[c - 1];
             }
-            sh.row[i][kTile] = (unsigned short)acc;
-            if (acc > kTileThreads) atomicMax(&sh.most, acc);
             // a tank that the step kernels cannot stage is refused here too
-            if (acc > 0 && n_in > kStage) {
-                const int first = (int)sh.at[i] - P - 1, wide = sh.across[i] + 2;
-                int around = 0;
-                for (int r = 0; r < sh.down[i] + 2; ++r) around += (int)start[first + r * P + wide] - (int)start[first + r * P];
-                if (around > kStage) atomicOr(&sh.flags, SPH_FLAG_STAGE_FULL);
-            }
+            if (acc > 0 && around > kStage) atomicOr(&sh.flags, SPH_FLAG_STAGE_FULL);
+            if (acc > kTileThreads) atomicMax(&sh.most, acc);
         }
         const int first = warp * (32 / kLanes);  // the warp's first particle, and this lane's
         const int mine = tid / kLanes;
