@@ -181,7 +181,7 @@ __device__ __forceinline__ float ghost_sum(const TankDev& T, const Runs& Q, floa
     return Sg;
 }
 
-// Eqs. 10 and 12 added to (ax, ay); returns the neighbours that this lane met.
+// Eqs. 10 and 12 as (ax, ay), zero before; returns the neighbours that this lane met.
 template <int LN>
 __device__ __forceinline__ int fluid_forces(const TankDev& T, const Runs& R, int e, float4 pi, float2 li, float2 ri,
                                             const float4* pv, const float2* plo, const float2* rho, int sub, float& ax,
@@ -215,6 +215,10 @@ __device__ __forceinline__ int fluid_forces(const TankDev& T, const Runs& R, int
             ay = from_lane<LN>(ty, l);
         }
     }
+    // At a position that is not finite the sums of zero forces are not zero.  (Such
+    // a particle lies in the grid's outermost cells, where fluid inside the wall
+    // has it in no stencil.)
+    if (const float a = ax + ay; a != a && !(isfinite(pi.x) && isfinite(pi.y))) ax = ay = 0.f;
     return met;
 }
 
@@ -224,6 +228,13 @@ __device__ __forceinline__ int ghost_forces(const TankDev& T, const Runs& Q, flo
                                             const float4* gp, const float4* gvel, int sub, W_& W)
 {
     int n_met = 0;
+    if (Q.most == 0) return 0;
+    // a particle that reaches no ghost, one off the grid among them, goes
+    // through the rounds of its warp with forces of zero over finite distances
+    if (Q.n == 0) {
+        pi.x = pi.y = 0.f;
+        li = make_float2(0.f, 0.f);
+    }
     for (int k0 = 0; k0 < Q.most; k0 += LN * kChunk) {
         float f[kChunk];
         float2 d[kChunk], arm[kChunk];
