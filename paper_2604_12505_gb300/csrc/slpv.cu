@@ -429,8 +429,10 @@ __global__ void __launch_bounds__(32)
     const int tr = sg / per_traj, seg = sg % per_traj + (MAP ? 1 : 0);
     const bool own = tr < n_traj && l < NX;
     const size_t t = tr < n_traj ? tr : n_traj - 1;
-    const int k0 = seg * seg_len, n = min(len - k0, seg_len);  // the segment's samples
-    float v = MAP ? (j == col ? 1.f : 0.f) : first ? 0.f : carry_in[t * NX + j];
+    const int k0 = seg * seg_len, own_n = min(len - k0, seg_len);  // the segment's samples
+    const float v_end = MAP ? (j == col ? 1.f : 0.f) : first ? 0.f : carry_in[t * NX + j];
+    float v = v_end;
+    int n = own_n, n_chunk = (seg_len + C - 1) / C;  // samples to go back over; chunks, the same in all groups of a warp
     auto at_map = [&](int s, int c) { return map + ((t * n_seg + s) * (NX + 1) + c) * NX + j; };
     if constexpr (!MAP) {
 #pragma unroll 4
@@ -440,10 +442,18 @@ __global__ void __launch_bounds__(32)
             for (int r = 0; r < NX; ++r) w = fmaf(*at_map(s, r), __shfl_sync(0xffffffffu, v, r, L), w);
             if (s > seg) v = w;
         }
+        // a map that overflowed says nothing of the lambda it maps: from the window's end instead
+        const unsigned bad = __ballot_sync(0xffffffffu, !isfinite(v));
+        if (bad) {
+            if (bad >> (threadIdx.x - l) & ((1u << L) - 1u)) {
+                v = v_end;
+                n = len - k0;
+            }
+            n_chunk = __reduce_max_sync(0xffffffffu, (n + C - 1) / C);
+        }
     }
     float* lt = lam + (t * ld + k0) * NX + j;
     const float* at = adj + (t * ld + k0) * R;
-    const int n_chunk = (seg_len + C - 1) / C;  // the same in all groups of a warp
     // chunk c holds steps n - (c + 1) C and on, C of them; those below 0 are not there
     auto fetch = [&](int c) {
         const int lo = n - (c + 1) * C;
@@ -460,7 +470,7 @@ __global__ void __launch_bounds__(32)
         copy_commit();
     };
     auto step = [&](int k, const float* rec, bool in) {
-        if (!MAP && own && in) lt[(ptrdiff_t)k * NX] = v;
+        if (!MAP && own && in && k < own_n) lt[(ptrdiff_t)k * NX] = v;
         float J[NX], a = col == NX ? rec[NX * NX + j] : 0.f, m = 0.f;
         load_vec<NX>(rec + j * NX, J);
 #pragma unroll
