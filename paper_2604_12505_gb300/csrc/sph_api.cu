@@ -696,9 +696,14 @@ int sph_samples_for(const sph_sim* sim, int32_t n_steps, int32_t* n_samples)
 }
 
 namespace {
-// Steps of a launch of the resident kernel: long enough to make its start and
-// end (about two steps' time) disappear, short enough (milliseconds) to share the GPU.
-constexpr int kResidentSteps = 1024;
+// Steps of a launch of the resident kernel.  The tiles are dealt out to its CTAs
+// when it starts, so fluid that moves during a launch gathers in some of them;
+// a launch's start and end take about two steps' time.  1,000 steps of 1 ms in
+// one call, us a step by the launch's length 1,024, 256, 128 and 64: the
+// paper's tank at rest 18.2, 16.6, 16.0, 15.9; under 3 m/s^2 to one side at 0.2
+// fill 39.5, 18.9, 16.4, 15.6 (37.1 in passes), under 9.5 m/s^2 141, 42, 31, 27
+// (44.9); 938 particles at rest, steps of 0.05 ms, 10.5, 10.6, 10.6, 10.8.
+constexpr int kResidentSteps = 128;
 
 int run_resident(sph_sim* sim, int n_steps, cudaStream_t st)
 {
