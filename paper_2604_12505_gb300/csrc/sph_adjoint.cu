@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_force_kernel(SimDe
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, true, false> sm;
-    __shared__ GhostStage<true> gs;
+    __shared__ GhostStage<> gs;
     __shared__ float2 sab[Sh::MAXS];  // acceleration adjoint of each staged particle
     const int4 td = S.tiles[blockIdx.x];
     const int tank = td.x;
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS) adj_density_kernel(Sim
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, true, false> sm;
-    __shared__ GhostStage<true> gs;
+    __shared__ GhostStage<> gs;
     __shared__ float srb[Sh::MAXS];  // density adjoint of each staged particle
     const int4 td = S.tiles[blockIdx.x];
     const int tank = td.x;

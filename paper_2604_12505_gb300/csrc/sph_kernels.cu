@@ -1,8 +1,8 @@
 // sph_kernels.cu -- the per-step kernels of the SPH sloshing simulator.
 //
-// One inner step (Algorithm 1 + symplectic Euler, Section 3.4) is two
+// One inner step (Algorithm 1 + symplectic Euler, Section 3.4) is three
 // launches over all tanks of a batch, chained by programmatic dependent
-// launch (each kernel lets its successor be scheduled at once and waits for
+// launch (each kernel lets its successor be scheduled early and waits for
 // its predecessor only before touching data the predecessor writes):
 //   density_kernel  Eq. 21 for the ghosts each particle meets (two-float
 //                   arithmetic on the FP32 pipe), Eqs. 14 and 11 (+ the
@@ -14,10 +14,13 @@
 //   force_kernel    Eqs. 10, 12 (fluid pairs), 16-19 (ghost pairs), the fluid
 //                   acceleration of Algorithm 1, kick-then-drift of the fluid,
 //                   and the re-binning of the moved particle into the other
-//                   grid buffer.  Per-tile compensated force/torque partials;
-//                   the last CTA of a tank reduces them in fixed order,
-//                   assembles them in FP64 and integrates the FP64 body
+//                   grid buffer.  Each tile adds its force, torque and position
+//                   sums to the tank's fixed-point accumulators.
+//   body_kernel     converts these to FP64 and integrates the FP64 body
 //                   (Eq. 20), samples outputs and runs the PD law (Eq. 28).
+// The tangent variants leave the tiles' partials, which tan_body_kernel sums in
+// fixed order.  Tanks that do not fill the GPU take the passes of sph_lanes.cu
+// in place of the first two, or the kernel of sph_resident.cu for all three.
 // No warp-wide FP64 arithmetic runs in the tile kernels: this GPU's FP64
 // pipe issues a warp instruction in about 16 cycles per SM.
 #include <algorithm>
@@ -44,7 +47,7 @@ __device__ __forceinline__ void density_pass(const SimDev& S, const EvalOut& E, 
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, false, TAN> sm;
-    __shared__ GhostStage<true, TAN> gs;
+    __shared__ GhostStage<TAN> gs;
     const int4 td = S.tiles[blockIdx.x];
     const TankDev T = S.tank[td.x];  // by value: the constants live in registers
     const int cx0 = td.y, cy0 = td.z;
@@ -754,7 +757,7 @@ __global__ void __launch_bounds__(Shape<TX, TY>::THREADS, TAN ? 1 : Shape<TX, TY
 {
     using Sh = Shape<TX, TY>;
     __shared__ Stage<TX, TY, true, TAN> sm;
-    __shared__ GhostStage<true> gs;
+    __shared__ GhostStage<> gs;
     __shared__ Red scratch[32];
     // the successor is the body update, a few warps: placed at once, it
     // prepares its update during this pass

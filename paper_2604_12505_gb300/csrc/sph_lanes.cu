@@ -31,7 +31,7 @@ constexpr int kThreads = kPlaces * kLanes;
 
 // The runs of staged ghosts within clip of a particle, in the order of
 // for_staged_ghosts; lane r looks in row r of the 3x3 ghost cells.
-__device__ __forceinline__ Runs ghost_runs(const TankDev& T, const GhostStage<true>& gs, bool on, float x, float y, float bc,
+__device__ __forceinline__ Runs ghost_runs(const TankDev& T, const GhostStage<>& gs, bool on, float x, float y, float bc,
                                            float bs, float brx, float bry, float clip, int sub)
 {
     int gx, gy, a = 0, b = 0;
@@ -57,7 +57,7 @@ __device__ __forceinline__ Runs ghost_runs(const TankDev& T, const GhostStage<tr
 __global__ void __launch_bounds__(kThreads, 2) density_lanes_kernel(SimDev S, int chained)
 {
     __shared__ Stage<4, 4, false, false> sm;
-    __shared__ GhostStage<true> gs;
+    __shared__ GhostStage<> gs;
     const int4 td = S.tiles[blockIdx.x];
     const TankDev T = S.tank[td.x];
     const int cx0 = td.y, cy0 = td.z;
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, 2) density_lanes_kernel(SimDev S, in
 __global__ void __launch_bounds__(kThreads, 2) force_lanes_kernel(SimDev S)
 {
     __shared__ Stage<4, 4, true, false> sm;
-    __shared__ GhostStage<true> gs;
+    __shared__ GhostStage<> gs;
     __shared__ Red scratch[kPlaces / 32];
     __shared__ float part[5][kPlaces];  // wall force and torque, position sums of each place
     __shared__ unsigned pairs_all;

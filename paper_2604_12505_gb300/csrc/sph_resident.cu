@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1) resident_kernel(SimDev S, int n_s
             sh.frame = Frame{{b0.drx, b0.dry, {0.f, 0.f}, {b0.fvx, 0.f}, {b0.fvy, 0.f}, {b0.fw, 0.f}, {b0.fo_next[0], 0.f},
                               {b0.fo_next[1], 0.f}, b0.dc, b0.ds}};
     }
-    unsigned pairs_sum = 0;  // of this thread: at most a tank's pairs a step, by 1024 steps
+    unsigned pairs_sum = 0;  // of this thread: at most a tank's pairs a step, by the steps of a launch
     cluster_sync();  // every CTA has read the state, and may be written to
 
     // sorted index of particle t of own tile i

@@ -447,13 +447,13 @@ __device__ __forceinline__ void ghost_world(const GhostFrame& f, float4 gb, floa
 constexpr int kGhostMax = 256;  // staged ghosts per tile
 constexpr int kGhostDim = 16;   // staged ghost-cell rows and columns per tile
 
-template <bool ON, bool TAN = false>
+template <bool TAN = false>
 struct GhostStage {
-    float4 gp[ON ? kGhostMax : 1];                    // world position (x_hi, y_hi, x_lo, y_lo)
-    float4 gv[ON ? kGhostMax : 1];                    // (v_x, v_y, arm_x, arm_y)
+    float4 gp[kGhostMax];                    // world position (x_hi, y_hi, x_lo, y_lo)
+    float4 gv[kGhostMax];                    // (v_x, v_y, arm_x, arm_y)
     float4 tg[TAN ? kGhostMax : 1];                   // tangent (d r_g, d v_g)
-    float bx[ON ? kGhostMax : 1];                     // body-frame x (a row of cells is sorted by it)
-    int tab[ON ? kGhostDim : 1][kGhostDim + 1];      // ghost-cell starts of the staged cells (global index)
+    float bx[kGhostMax];                     // body-frame x (a row of cells is sorted by it)
+    int tab[kGhostDim][kGhostDim + 1];      // ghost-cell starts of the staged cells (global index)
     int base[kGhostDim];                             // staged index of ghost g of row r: base[r] + g
     int pre[kGhostDim + 1];                          // first staged index of each row
     int box[4];                                      // first, last staged cell column; first, last row
@@ -473,7 +473,7 @@ enum { kGhostsNone = 0, kGhostsStaged = 1, kGhostsGlobal = 2 };
 template <bool FILL, int TX, int TY, bool RHO, bool TAN, bool GTAN, class Tangent>
 __device__ __forceinline__ int stage_ghosts(const SimDev& S, const TankDev& T, float bc, float bs, float brx, float bry,
                                             const GhostFrame& fr, const Stage<TX, TY, RHO, TAN>& sm, int n_own,
-                                            GhostStage<true, GTAN>& gs, Tangent&& tangent)
+                                            GhostStage<GTAN>& gs, Tangent&& tangent)
 {
     if (threadIdx.x == 0) {
         gs.box[0] = INT_MAX;
